@@ -29,7 +29,7 @@ inline size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 enum Slot {
     kStatus, kTileMask, kOctpath, kRect, kCount, kTileCount, kRecord, kScanBlocks,
     kKeys0, kKeys1, kVals0, kVals1, kRanges, kDcol, kBox, kTileOrder, kBlockList, kBlockLen,
-    kHitMask, kSegment, kTotal, kNumSlots
+    kHitMask, kSegment, kSortPlan, kTotal, kNumSlots
 };
 
 struct Layout {
@@ -65,7 +65,7 @@ Layout make_layout(int64_t n_vox, int n_views, int64_t cap, int64_t ntiles, int 
     take(kOctpath, 8 * N);
     take(kRect, 8 * VN);
     take(kCount, 4 * VN);
-    take(kTileCount, 4 * (2 * svr::kTileSub + 1) * (size_t)ntiles);
+    take(kTileCount, 4 * 2 * svr::kTileSub * (size_t)ntiles);
     take(kRecord, sizeof(svr::Record) * VN);
     take(kScanBlocks, 4 * (((size_t)ntiles * svr::kTileSub + svr::kScanTile - 1) / svr::kScanTile + 1));
     take(kKeys0, 8 * C);
@@ -82,6 +82,7 @@ Layout make_layout(int64_t n_vox, int n_views, int64_t cap, int64_t ntiles, int 
     take(kBlockLen, 4 * B * (size_t)ntiles);
     take(kHitMask, 4 * B * (C + 32 * (size_t)ntiles));   // the block lists' positions + 32 per (tile, block)
     take(kSegment, seg_bytes(ntiles, slots, B).total);
+    take(kSortPlan, align256(sizeof(svr::SortPlan)) + 8 * (size_t)svr::sort_chunk_capacity(cap));
     L.off[kTotal] = o;
     return L;
 }
@@ -202,7 +203,6 @@ svr::FrameDev frame_dev(const svr_frame *f) {
     d.count = (uint32_t *)(ws + o[kCount]);
     d.tile_cnt = (uint32_t *)(ws + o[kTileCount]);
     d.cursor = d.tile_cnt + (size_t)svr::kTileSub * f->total_tiles;
-    d.tile_end = d.cursor + (size_t)svr::kTileSub * f->total_tiles;
     d.rec = (svr::Record *)(ws + o[kRecord]);
     d.box = (ushort4 *)(ws + o[kBox]);
     d.scan_blocks = (uint32_t *)(ws + o[kScanBlocks]);
@@ -210,6 +210,8 @@ svr::FrameDev frame_dev(const svr_frame *f) {
     d.keys[1] = (uint64_t *)(ws + o[kKeys1]);
     d.vals[0] = (uint32_t *)(ws + o[kVals0]);
     d.vals[1] = (uint32_t *)(ws + o[kVals1]);
+    d.plan = (svr::SortPlan *)(ws + o[kSortPlan]);
+    d.chunks = (uint2 *)(ws + o[kSortPlan] + align256(sizeof(svr::SortPlan)));
     d.ranges = (uint2 *)(ws + o[kRanges]);
     d.order = (uint2 *)(ws + o[kTileOrder]);
     d.blist = (uint2 *)(ws + o[kBlockList]);
@@ -230,6 +232,11 @@ svr::FrameDev frame_dev(const svr_frame *f) {
     d.world_size = f->scene.world_size;
     for (int i = 0; i < 3; ++i) d.world_min[i] = f->scene.world_center[i] - 0.5f * f->scene.world_size;
     d.max_level = f->scene.max_level;
+    d.sort_bits = 3 * (d.max_level < svr::kMaxLevel ? d.max_level + 1 : svr::kMaxLevel);
+    // bits that hold every voxel id and leave the all-ones word free
+    int vb = 1;
+    while (((int64_t)1 << vb) <= d.n_vox) ++vb;
+    d.vid_bits = d.sort_bits + svr::word_sign_bits(d.max_level) + vb <= 64 ? vb : 0;
     d.K = f->params.K;
     d.t_stop = f->params.t_stop;
     for (int i = 0; i < 3; ++i) d.bg[i] = f->params.bg[i];
@@ -416,9 +423,7 @@ SVR_API int svr_bin_sort(svr_frame *frame, int64_t *n_pairs_out, void *stream) {
     if (e != cudaSuccess) return cuda_fail(e, "ranges and work order");
     e = svr::launch_emit(d, s);
     if (e != cudaSuccess) return cuda_fail(e, "emit");
-    const int lmax = frame->scene.max_level;
-    const int morton_bits = 3 * (lmax < 16 ? lmax + 1 : 16);
-    e = svr::launch_tile_sort(d, frame->key_shift - morton_bits, morton_bits, lmax == 16, s);
+    e = svr::launch_tile_sort(d, s);
     if (e != cudaSuccess) return cuda_fail(e, "sort");
     frame->sorted_alt = 0;
     e = svr::launch_block_lists(d, 0, s);
@@ -433,7 +438,8 @@ SVR_API int svr_bin_sort(svr_frame *frame, int64_t *n_pairs_out, void *stream) {
         *n_pairs_out = P;
         frame->n_pairs = P;
         if (flags & SVR_FLAG_INVALID_VOXEL)
-            return fail(SVR_ERR_INVALID, "a voxel is off its lattice or its level is outside [1, %d]", lmax);
+            return fail(SVR_ERR_INVALID, "a voxel is off its lattice or its level is outside [1, %d]",
+                        frame->scene.max_level);
         if (flags & SVR_FLAG_CAPACITY)
             return fail(SVR_ERR_CAPACITY, "%lld pairs > capacity %lld", (long long)P,
                         (long long)frame->pair_capacity);

@@ -14,12 +14,15 @@
 //   k_scan_*      exclusive scan of the tiles' pair counts (block sums, then
 //                 each block scans its part after summing the earlier blocks;
 //                 kTileSub sub-buckets per tile, adjacent): each sub-bucket's
-//                 start, each tile's end, the total, the capacity check
+//                 start, each tile's range and segments, the work order's
+//                 group counts, the total, the capacity check
 //   k_emit        writes each (voxel, tile, sign pattern s) pair into its
 //                 tile's range (an atomic cursor per sub-bucket; the order
 //                 within a tile is left to the per-tile sort):
 //                 key = tile << S | top S bits of (octpath ^ s replicated),
-//                 value = s << 29 | voxel id (Sec. B.1; the per-triple
+//                 value = s << 29 | voxel id, written as one word that the
+//                 sort turns into them where it fits 64 bits (pair_word; one
+//                 8-byte store instead of 12 bytes in two) (Sec. B.1; the per-triple
 //                 permutation of Sec. B.2 is b ^ s, applied to all 16
 //                 triples at once).  S = 48 for one view (the paper's layout:
 //                 16-bit tile id over the 48-bit order); a batch of views uses
@@ -328,64 +331,99 @@ __device__ __forceinline__ int64_t sub_index(int64_t i, int64_t ntiles) {
     return (i % kTileSub) * ntiles + i / kTileSub;
 }
 
-__global__ void __launch_bounds__(256) k_scan_reduce(const uint32_t *__restrict__ count, int64_t ntiles,
-                                                     uint32_t *__restrict__ block_sums) {
+// Also clears the counters of the work order and the sort for k_scan_down.
+__global__ void __launch_bounds__(256) k_scan_reduce(FrameDev f) {
     __shared__ uint32_t ws[8];
-    const int64_t n = ntiles * kTileSub;
-    const int64_t base = (int64_t)blockIdx.x * kScanTile;
-    uint64_t acc = 0;
-    for (int r = 0; r < kScanTile / 256; ++r) {
-        int64_t i = base + r * 256 + threadIdx.x;
-        if (i < n) acc += count[sub_index(i, ntiles)];
+    if (blockIdx.x == 0) {
+        for (int i = threadIdx.x; i < (int)(sizeof(SortPlan) / 4); i += 256) reinterpret_cast<unsigned *>(f.plan)[i] = 0u;
+        if (threadIdx.x == 0) f.status->slots_used = 0;
     }
+    const int64_t ntiles = f.total_tiles, n = ntiles * kTileSub;
+    const int64_t i = (int64_t)blockIdx.x * kScanTile + threadIdx.x;
+    const uint64_t acc = i < n ? f.tile_cnt[sub_index(i, ntiles)] : 0u;
     uint32_t tot;
     // a block sum beyond 2^32 saturates; the capacity check on the 64-bit
     // total catches it
     block_exclusive_scan((uint32_t)tmin<uint64_t>(acc, 0xFFFFFFFFull), ws, tot);
-    if (threadIdx.x == 0) block_sums[blockIdx.x] = tot;
+    if (threadIdx.x == 0) f.scan_blocks[blockIdx.x] = tot;
 }
 
-// Sub-bucket starts (the emission cursors) and tile ends from the counts;
-// k_tile_order turns them into the tiles' ranges.  Each CTA first sums the
-// block sums of all earlier CTAs (64-bit), so no separate top-level scan is
-// launched; the last CTA records the total and checks it against the
-// capacity.  A start beyond 2^32 saturates; the capacity flag covers it.
-__global__ void __launch_bounds__(256) k_scan_down(const uint32_t *__restrict__ count, int64_t ntiles,
-                                                   const uint32_t *__restrict__ block_sums, int nb,
-                                                   uint32_t *__restrict__ cursor, uint32_t *__restrict__ tile_end,
-                                                   Status *st, int64_t capacity) {
+// Sub-bucket starts (the emission cursors) from the counts, and per tile its
+// range, its segments (with slots for a split list's) and its work-order
+// group's count.  Each CTA first sums the block sums of all earlier CTAs
+// (64-bit), so no separate top-level scan is launched, and of all CTAs, so
+// that every one knows whether the pairs exceed the capacity (then all
+// ranges are empty).  A start beyond 2^32 saturates; the capacity flag covers
+// it.
+__global__ void __launch_bounds__(256) k_scan_down(FrameDev f, int nb) {
     __shared__ uint32_t ws[8];
-    __shared__ unsigned long long wpre[8];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned long long pre = 0;
-    for (int j = threadIdx.x; j < (int)blockIdx.x; j += 256) pre += block_sums[j];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) pre += __shfl_xor_sync(0xffffffffu, pre, o);
-    if (lane == 0) wpre[warp] = pre;
-    __syncthreads();
-    pre = 0;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) pre += wpre[w];
-    const int64_t n = ntiles * kTileSub;
-    const int64_t base = (int64_t)blockIdx.x * kScanTile;
-    unsigned long long carry = pre;
-    for (int r = 0; r < kScanTile / 256; ++r) {
-        const int64_t i = base + r * 256 + threadIdx.x;
-        const uint32_t x = i < n ? count[sub_index(i, ntiles)] : 0u;
-        uint32_t tot;
-        const uint32_t ex = block_exclusive_scan(x, ws, tot);
-        if (i < n) {
-            const uint32_t c = (uint32_t)tmin<unsigned long long>(carry + ex, 0xFFFFFFFFull);
-            cursor[sub_index(i, ntiles)] = c;
-            if (i % kTileSub == kTileSub - 1)
-                tile_end[i / kTileSub] = (uint32_t)tmin<unsigned long long>(carry + ex + x, 0xFFFFFFFFull);
-        }
-        carry += tot;
+    __shared__ unsigned long long wpre[8], wall[8];
+    __shared__ unsigned group_cnt[2 * kOrderGroups], slots, slot0;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    if (t < 2 * kOrderGroups) group_cnt[t] = 0u;
+    if (t == 0) slots = 0u;
+    unsigned long long pre = 0, all = 0;
+    for (int j = t; j < nb; j += 256) {
+        const unsigned x = f.scan_blocks[j];
+        all += x;
+        if (j < (int)blockIdx.x) pre += x;
     }
-    if (blockIdx.x == nb - 1 && threadIdx.x == 0) {
-        st->n_pairs_lo = (unsigned)(carry & 0xFFFFFFFFull);
-        st->n_pairs_hi = (unsigned)(carry >> 32);
-        if (carry > (unsigned long long)capacity) atomicOr(&st->flags, SVR_FLAG_CAPACITY);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        pre += __shfl_xor_sync(0xffffffffu, pre, o);
+        all += __shfl_xor_sync(0xffffffffu, all, o);
+    }
+    if (lane == 0) {
+        wpre[warp] = pre;
+        wall[warp] = all;
+    }
+    __syncthreads();
+    pre = all = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+        pre += wpre[w];
+        all += wall[w];
+    }
+    const bool over = all > (unsigned long long)f.capacity;
+    const int64_t ntiles = f.total_tiles, n = ntiles * kTileSub;
+    const int64_t i = (int64_t)blockIdx.x * kScanTile + t;
+    const uint32_t x = i < n ? f.tile_cnt[sub_index(i, ntiles)] : 0u;
+    uint32_t tot;
+    const uint32_t ex = block_exclusive_scan(x, ws, tot);
+    const uint32_t c = (uint32_t)tmin<unsigned long long>(pre + ex, 0xFFFFFFFFull);
+    const uint32_t e = (uint32_t)tmin<unsigned long long>(pre + ex + x, 0xFFFFFFFFull);
+    if (i < n) f.cursor[sub_index(i, ntiles)] = c;
+    // the kTileSub lanes of a tile: the first one takes the tile
+    const uint32_t end = __shfl_sync(0xffffffffu, e, lane | (kTileSub - 1));
+    const bool tile = i < n && i % kTileSub == 0;
+    const uint2 r = over || end == c ? make_uint2(0u, 0u) : make_uint2(c, end);
+    const unsigned len = r.y - r.x;
+    unsigned nseg = len > (unsigned)kSegLen ? (len + kSegLen - 1) / kSegLen : 1u, base = 0;
+    if (tile && nseg > 1) base = atomicAdd(&slots, nseg);
+    __syncthreads();
+    if (t == 0) slot0 = slots ? atomicAdd(&f.status->slots_used, slots) : 0u;
+    __syncthreads();
+    if (tile) {
+        if (nseg > 1) {
+            base += slot0;
+            if ((int64_t)base + nseg > f.seg_slots) nseg = 1, base = 0;  // only past the pair capacity
+        }
+        const int bk = order_bucket(len, nseg);
+        if (nseg > 1) {
+            atomicAdd(&group_cnt[kFirstSeg + bk], 1u);
+            atomicAdd(&group_cnt[bk], nseg - 1);
+        } else {
+            atomicAdd(&group_cnt[bk], 1u);
+        }
+        f.ranges[i / kTileSub] = r;
+        f.tile_seg[i / kTileSub] = make_uint2(nseg, base);
+    }
+    __syncthreads();
+    if (t < 2 * kOrderGroups && group_cnt[t]) atomicAdd(&f.plan->cnt[t], group_cnt[t]);
+    if (blockIdx.x == 0 && t == 0) {
+        f.status->n_pairs_lo = (unsigned)(all & 0xFFFFFFFFull);
+        f.status->n_pairs_hi = (unsigned)(all >> 32);
+        if (over) atomicOr(&f.status->flags, SVR_FLAG_CAPACITY);
     }
 }
 
@@ -406,6 +444,7 @@ __global__ void __launch_bounds__(kEmitThreads) k_emit(FrameDev f) {
     const short4 rc = f.rect[iv];
     const uint64_t code = f.octpath[v];
     const int drop = 48 - f.key_shift;
+    const bool words = f.vid_bits > 0;
     uint64_t *keys = f.keys[0];
     uint32_t *vals = f.vals[0];
     uint32_t *cur = f.cursor + (size_t)(v & (kTileSub - 1)) * f.total_tiles;
@@ -440,8 +479,12 @@ __global__ void __launch_bounds__(kEmitThreads) k_emit(FrameDev f) {
             while (m) {
                 const unsigned s = __ffs(m) - 1;
                 m &= m - 1;
-                keys[o] = ((uint64_t)gb[i] << f.key_shift) | ((code ^ ((uint64_t)s * kTripleOnes)) >> drop);
-                vals[o] = (s << 29) | (uint32_t)v;
+                if (words) {
+                    keys[o] = pair_word(f, code, s, (uint32_t)v);
+                } else {
+                    keys[o] = ((uint64_t)gb[i] << f.key_shift) | ((code ^ ((uint64_t)s * kTripleOnes)) >> drop);
+                    vals[o] = (s << 29) | (uint32_t)v;
+                }
                 ++o;
             }
         }
@@ -468,8 +511,9 @@ cudaError_t launch_preprocess(const FrameDev &f, cudaStream_t s) {
 cudaError_t launch_scan(const FrameDev &f, cudaStream_t s) {
     const int64_t T = f.total_tiles;
     const int nb = (int)((T * kTileSub + kScanTile - 1) / kScanTile);
-    k_scan_reduce<<<nb, 256, 0, s>>>(f.tile_cnt, T, f.scan_blocks);
-    k_scan_down<<<nb, 256, 0, s>>>(f.tile_cnt, T, f.scan_blocks, nb, f.cursor, f.tile_end, f.status, f.capacity);
+    static_assert(kScanTile == 256, "one entry per thread");
+    k_scan_reduce<<<nb, 256, 0, s>>>(f);
+    k_scan_down<<<nb, 256, 0, s>>>(f, nb);
     return cudaGetLastError();
 }
 

@@ -35,6 +35,16 @@ constexpr int kSegFields = 14;
 // lines; the sub-buckets of a tile are adjacent in its range.
 constexpr int kTileSub = 8;
 
+// A tile list up to kSortCap pairs is sorted by one group of threads in shared
+// memory; a longer one as chunks of at most kSortCap pairs, merged afterwards.
+constexpr int kSortCap = 8192;
+
+// Chunks a workspace holds for pair_capacity pairs: a list of L >= kSortCap
+// pairs takes ceil(L / kSortCap) <= 2 L / kSortCap chunks.
+__host__ __device__ __forceinline__ int64_t sort_chunk_capacity(int64_t capacity) {
+    return 2 * capacity / kSortCap + 1;
+}
+
 // Segment slots a workspace holds for pair_capacity pairs: a split tile of
 // L > kSegLen entries takes ceil(L / kSegLen) < 2 L / kSegLen slots.
 __host__ __device__ __forceinline__ int64_t seg_slot_capacity(int64_t capacity) {
@@ -67,12 +77,41 @@ struct Status {
     unsigned slots_used;  // segment slots taken by the split tiles
     unsigned fwd_done;    // bit 0: a forward filled the segment sums of the current sort; bit 1: with
                           // the normal image; bit 2: with the distortion loss
-    unsigned sort_next;   // next work-order entry of the long-list sort
+    unsigned unused0;
     unsigned fwd_exit;    // warps of the running forward launch that ran out of work
     unsigned maxw_next;   // next work item of the maximum-weight pass over split lists (reset before it)
-    unsigned n_long;      // split tiles: the first n_long work-order entries are their first segments
+    unsigned unused1;
     unsigned n_listed;    // work-order entries of non-empty lists (the empty tiles' entries come last)
     unsigned pad[2];
+};
+
+// Groups of the render work order: floor(log2(length)) + 1 of a tile's list,
+// one more for a split list, so that every split list (longer than kSegLen)
+// precedes every unsplit one; a split list's first segment goes to group
+// kFirstSeg + its group, ahead of all others.  Group 0: the empty lists.
+constexpr int kOrderGroups = 34;
+constexpr int kFirstSeg = kOrderGroups;
+
+__device__ __forceinline__ int order_bucket(unsigned len, unsigned nseg) {
+    return len ? 32 - __clz(len) + (nseg > 1 ? 1 : 0) : 0;
+}
+
+// Sort classes by list length: threads per list.  A list of 2^(c+8) to
+// 2^(c+9) - 1 pairs goes to class c = 1 .. 5 (32 2^(c-1) threads of 16 pairs
+// each, at least the longer end), a shorter one to class 0, whose lists take
+// a warp each as well (1024 pairs exactly, an unsplit list, fits class 2).
+constexpr int kSortClasses = 6;
+
+// Counters of the work order and the sort (cleared by k_scan_reduce, counted
+// by k_scan_down, the rest filled by k_order).
+struct SortPlan {
+    unsigned cnt[2 * kOrderGroups];   // work-order entries of each group
+    unsigned pos[2 * kOrderGroups];   // entries of each group already placed
+    unsigned n_chunks;                // chunks of the lists of at least kSortCap pairs
+    unsigned n_huge;                  // such lists: the first n_huge work-order entries
+    unsigned next;                    // next unit of k_sort_lists
+    unsigned first[kSortClasses];     // first work-order entry of each class's lists
+    unsigned count[kSortClasses];     // and their number
 };
 
 // Index checks of the SVR_DEBUG build (compiled out otherwise).  A failed
@@ -202,12 +241,16 @@ struct FrameDev {
     uint32_t *count;         // [V * N] pairs of each (view, voxel)
     uint32_t *tile_cnt;      // [kTileSub][total_tiles] pairs of each tile's sub-buckets (k_preprocess)
     uint32_t *cursor;        // [kTileSub][total_tiles] next free slot of each sub-bucket
-    uint32_t *tile_end;      // [total_tiles] end of each tile's range (from the scan)
     Record *rec;             // [V * N]
     ushort4 *box;            // [V * N] inclusive pixel range x0, x1, y0, y1 a hit can fall in
-    uint32_t *scan_blocks;   // [ceil(total_tiles / kScanTile) + 1]
+    uint32_t *scan_blocks;   // [ceil(kTileSub total_tiles / kScanTile) + 1]
     uint64_t *keys[2];
     uint32_t *vals[2];
+    SortPlan *plan;
+    uint2 *chunks;           // [sort_chunk_capacity] (tile, chunk) of the long lists
+    int sort_bits;           // Morton bits that can differ between two pairs of a tile
+    int vid_bits;            // > 0: a pair is emitted and sorted as one 64-bit word (see pair_word),
+                             // with this many low bits for the voxel id; 0: as its key and value
     uint2 *ranges;           // [total_tiles]
     uint2 *order;            // [total_tiles + seg slots] (tile, segment), longest segments first
     uint2 *tile_seg;         // [total_tiles] segments of the tile's list, first segment slot
@@ -240,6 +283,32 @@ struct FrameDev {
     const float *sh;
     DebugBlock *debug;       // index-check report of the SVR_DEBUG build (else nullptr)
 };
+
+// The word of a pair where its parts fit 64 bits: the Morton bits that can
+// differ, then (max level 16 only) the sign pattern, then the voxel id.
+// Words of one tile order like its (key, value) pairs: below max level 16 the
+// lowest Morton triple is the sign pattern itself (a padded triple).
+__host__ __device__ __forceinline__ int word_sign_bits(int max_level) { return max_level >= kMaxLevel ? 3 : 0; }
+
+__device__ __forceinline__ uint64_t pair_word(const FrameDev &f, uint64_t code, unsigned s, uint32_t vid) {
+    const uint64_t m = (code ^ ((uint64_t)s * kTripleOnes)) >> (48 - f.sort_bits);
+    const uint64_t hi = f.max_level >= kMaxLevel ? (m << 3) | s : m;
+    return (hi << f.vid_bits) | vid;
+}
+
+// Key and value of tile g's pair from its Morton bits, sign pattern and voxel id.
+__device__ __forceinline__ uint64_t pair_key(const FrameDev &f, int g, uint64_t morton, unsigned s) {
+    const int lo = f.key_shift - f.sort_bits;   // low bits of the order: padded triples, all s
+    return ((uint64_t)g << f.key_shift) | (morton << lo) | (((uint64_t)s * kTripleOnes) & ((1ull << lo) - 1ull));
+}
+
+__device__ __forceinline__ void word_pair(const FrameDev &f, int g, uint64_t word, uint64_t &key, uint32_t &val) {
+    const uint32_t vid = (uint32_t)(word & ((1ull << f.vid_bits) - 1ull));
+    const uint64_t hi = word >> f.vid_bits;
+    const unsigned s = (unsigned)hi & 7u;
+    key = pair_key(f, g, f.max_level >= kMaxLevel ? hi >> 3 : hi, s);
+    val = (s << 29) | vid;
+}
 
 // View that owns global tile g.
 __device__ __forceinline__ int view_of_tile(const FrameDev &f, int g) {
@@ -277,7 +346,7 @@ cudaError_t launch_preprocess(const FrameDev &f, cudaStream_t s);
 cudaError_t launch_scan(const FrameDev &f, cudaStream_t s);
 cudaError_t launch_order(const FrameDev &f, cudaStream_t s);
 cudaError_t launch_emit(const FrameDev &f, cudaStream_t s);
-cudaError_t launch_tile_sort(const FrameDev &f, int lo_bit, int nbits, bool ties, cudaStream_t s);
+cudaError_t launch_tile_sort(const FrameDev &f, cudaStream_t s);
 cudaError_t launch_block_lists(const FrameDev &f, int sorted_alt, cudaStream_t s);
 cudaError_t launch_render_fwd(const FrameDev &f, float *rgb, float *depth,
                               float *alpha, float *T_final, int32_t *last, int2 *stats, float *normal,
