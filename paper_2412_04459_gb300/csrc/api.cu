@@ -73,7 +73,7 @@ Layout make_layout(int64_t n_vox, int n_views, int64_t cap, int64_t ntiles, int 
     take(kVals0, 4 * C);
     take(kVals1, 4 * C);
     take(kRanges, 8 * (size_t)ntiles);
-    take(kDcol, 12 * VN);
+    take(kDcol, 16 * VN + 32 * N);   // colour accumulators per view, corner-density accumulators
     take(kBox, 8 * VN);
     const size_t slots = (size_t)svr::seg_slot_capacity(cap);
     take(kTileOrder, 8 * ((size_t)ntiles + slots));
@@ -225,7 +225,8 @@ svr::FrameDev frame_dev(const svr_frame *f) {
     d.merge_cnt = (uint32_t *)(seg + sb.merge_cnt);
     d.seg_len = (uint32_t *)(seg + sb.seg_len);
     d.seg_part = (float *)(seg + sb.seg_part);
-    d.dcol = (float *)(ws + o[kDcol]);
+    d.dcol = (float4 *)(ws + o[kDcol]);
+    d.dgrid = d.dcol + (size_t)f->n_views * f->scene.n_vox;
     d.n_vox = f->scene.n_vox;
     d.n_pts = f->scene.n_pts;
     d.capacity = f->pair_capacity;

@@ -212,6 +212,16 @@ __device__ __forceinline__ void load_sh(const FrameDev &f, int64_t v, float sh[4
     }
 }
 
+// A voxel's density polynomial from its gathered corner densities.
+__device__ __forceinline__ void gather_density(const FrameDev &f, const int4 &i0, const int4 &i1, float4 &r1,
+                                               float4 &r2) {
+    float g[8] = {__ldg(f.grid + i0.x), __ldg(f.grid + i0.y), __ldg(f.grid + i0.z), __ldg(f.grid + i0.w),
+                  __ldg(f.grid + i1.x), __ldg(f.grid + i1.y), __ldg(f.grid + i1.z), __ldg(f.grid + i1.w)};
+    density_coeffs(g);
+    r1 = make_float4(g[0], g[1], g[2], g[3]);
+    r2 = make_float4(g[4], g[5], g[6], g[7]);
+}
+
 __device__ __forceinline__ void write_octpath(const FrameDev &f, int64_t v, int l, const int ijk[3]) {
     f.octpath[v] = ((spread3(ijk[0]) << 2) | (spread3(ijk[1]) << 1) | spread3(ijk[2])) << (3 * (kMaxLevel - l));
 }
@@ -243,8 +253,7 @@ __global__ void __launch_bounds__(128, 8) k_preprocess(FrameDev f) {
     // gathered raw densities, colour
     Record r;
     r.r0 = make_float4((c0 - h) - cam.ro[0], (c1 - h) - cam.ro[1], (c2 - h) - cam.ro[2], vs);
-    r.r1 = make_float4(__ldg(f.grid + i0.x), __ldg(f.grid + i0.y), __ldg(f.grid + i0.z), __ldg(f.grid + i0.w));
-    r.r2 = make_float4(__ldg(f.grid + i1.x), __ldg(f.grid + i1.y), __ldg(f.grid + i1.z), __ldg(f.grid + i1.w));
+    gather_density(f, i0, i1, r.r1, r.r2);
     float Y[16], sh[48];
     view_basis(cam, c0, c1, c2, Y);
     load_sh(f, v, sh);
@@ -284,8 +293,8 @@ __global__ void __launch_bounds__(128) k_preprocess_views(FrameDev f) {
             f.rec[(int64_t)view * f.n_vox + v].r3 = voxel_colour(Y, sh);
         }
     }
-    const float4 g0 = make_float4(__ldg(f.grid + i0.x), __ldg(f.grid + i0.y), __ldg(f.grid + i0.z), __ldg(f.grid + i0.w));
-    const float4 g1 = make_float4(__ldg(f.grid + i1.x), __ldg(f.grid + i1.y), __ldg(f.grid + i1.z), __ldg(f.grid + i1.w));
+    float4 g0, g1;
+    gather_density(f, i0, i1, g0, g1);
     const float h = 0.5f * vs;
     for (int view = 0; view < f.n_views; ++view) {
         const DevCam &cam = f.views[view];

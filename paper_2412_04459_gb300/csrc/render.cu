@@ -41,7 +41,8 @@
 //   dC/dc_i = T_i alpha_i,
 //   dd_i/dx_ik = P_{k+1} t_k - sum_{m>k} P_m (1 - e_m) t_m  (P_k = prod_{j<k} e_j;
 //                the general form of the K <= 3 closed forms of Sec. A.4),
-//   dx_ik/dv_k = (l/K) explin'(v_k), dv_k/dV_c = trilinear weight of corner c.
+//   dx_ik/dv_k = (l/K) explin'(v_k), dv_k/da_m = monomial m of the density
+//   polynomial (its adjoint takes the sums to the corners).
 // T_i is recovered as T_{i+1} / exp(-x_i).  Pixels whose T_final is below
 // 1e-30 (where that division loses precision) take a front-to-back phase
 // instead, with SC_i, SD_i from totals recomputed in a first sweep.  The
@@ -70,13 +71,13 @@ constexpr int kBatch = 32;
 // Staged list entry, padded to 112 bytes: lanes reading different entries
 // then spread over 8 bank groups rather than 4.
 struct Entry {
-    float4 a;    // entry plane (near corner) relative to r_o, sign bits (int)
+    float4 a;    // entry plane (near corner) relative to r_o, clamp bits of the colour channels (uint)
     float4 b;    // exit plane (far corner) relative to r_o, 1 / size
-    float4 c;    // (min corner - r_o) / size, index in the sorted list (int)
-    float4 g0;   // raw corner densities 0..3
-    float4 g1;   // raw corner densities 4..7
+    float4 c;    // (centre - r_o) / size, index in the sorted list (int)
+    float4 g0;   // density polynomial: 1, z, y, yz
+    float4 g1;   // x, xz, xy, xyz
     float4 col;  // colour, voxel id (int)
-    float4 pad;  // x: clamp bits of the colour channels (uint); y, z, w unused
+    float4 pad;  // unused
 };
 
 __device__ __forceinline__ void stage_entry(Entry &e, uint32_t val, int idx, const Record *__restrict__ rec) {
@@ -87,25 +88,22 @@ __device__ __forceinline__ void stage_entry(Entry &e, uint32_t val, int idx, con
     const float lx = r0.x, ly = r0.y, lz = r0.z, size = r0.w;
     const float hx = lx + size, hy = ly + size, hz = lz + size;
     const float inv = 1.0f / size;
-    e.a = make_float4((s & 4) ? hx : lx, (s & 2) ? hy : ly, (s & 1) ? hz : lz, __int_as_float((int)s));
     e.b = make_float4((s & 4) ? lx : hx, (s & 2) ? ly : hy, (s & 1) ? lz : hz, inv);
-    e.c = make_float4(lx * inv, ly * inv, lz * inv, __int_as_float(idx));
+    e.c = make_float4(fmaf(lx, inv, 0.5f), fmaf(ly, inv, 0.5f), fmaf(lz, inv, 0.5f), __int_as_float(idx));
     e.g0 = __ldg(&r->r1);
     e.g1 = __ldg(&r->r2);
     const float4 c3 = __ldg(&r->r3);
+    e.a = make_float4((s & 4) ? hx : lx, (s & 2) ? hy : ly, (s & 1) ? hz : lz, c3.w);
     e.col = make_float4(c3.x, c3.y, c3.z, __int_as_float((int)vid));
-    e.pad.x = c3.w;
 }
 
-// Trilinear interpolation of Eq. interp; corner bits (x, y, z), x most significant.
+// Raw density at (qx, qy, qz) in [-1/2, 1/2]^3 about the centre (density_coeffs).
 __device__ __forceinline__ float trilerp(const float4 &g0, const float4 &g1, float qx, float qy, float qz) {
-    const float c00 = fmaf(qz, g0.y - g0.x, g0.x);  // 000, 001
-    const float c01 = fmaf(qz, g0.w - g0.z, g0.z);  // 010, 011
-    const float c10 = fmaf(qz, g1.y - g1.x, g1.x);  // 100, 101
-    const float c11 = fmaf(qz, g1.w - g1.z, g1.z);  // 110, 111
-    const float c0 = fmaf(qy, c01 - c00, c00);
-    const float c1 = fmaf(qy, c11 - c10, c10);
-    return fmaf(qx, c1 - c0, c0);
+    const float c00 = fmaf(g0.y, qz, g0.x);
+    const float c01 = fmaf(g0.w, qz, g0.z);
+    const float c10 = fmaf(g1.y, qz, g1.x);
+    const float c11 = fmaf(g1.w, qz, g1.z);
+    return fmaf(fmaf(c11, qy, c10), qx, fmaf(c01, qy, c00));
 }
 
 // alpha = 1 - exp(-X) of a segment with optical depth X = sum_k (l/K) sigma_k
@@ -491,7 +489,7 @@ __device__ __forceinline__ void hit_fwd(const Entry &e, const PixelRay &p, float
                                         float &dloc, float &alpha) {
     const float inv_k = 1.0f / K;
     const float seg = b - a;
-    const float xs = seg * p.rdn * inv_k;
+    const float xs = seg * p.rdn * (inv_k * kLog2e);   // optical depths in units of ln 2
     const float step = seg * inv_k;
     const float inv_size = e.b.w;
     const float rx = p.rd.x * inv_size, ry = p.rd.y * inv_size, rz = p.rd.z * inv_size;
@@ -501,7 +499,7 @@ __device__ __forceinline__ void hit_fwd(const Entry &e, const PixelRay &p, float
     for (int k = 0; k < K; ++k) {
         const float v = trilerp(e.g0, e.g1, fmaf(t, rx, -e.c.x), fmaf(t, ry, -e.c.y), fmaf(t, rz, -e.c.z));
         const float xk = xs * explin(v);
-        const float ek = __expf(-xk);
+        const float ek = ex2(-xk);
         d = fmaf(P * (1.f - ek), t, d);
         P *= ek;
         X += xk;
@@ -509,7 +507,7 @@ __device__ __forceinline__ void hit_fwd(const Entry &e, const PixelRay &p, float
     }
     trans = P;
     dloc = d;
-    alpha = seg_alpha(X, P);
+    alpha = seg_alpha(X * kLn2, P);
 }
 
 struct FwdOut {
@@ -551,16 +549,12 @@ __device__ __forceinline__ void dist_add(FwdState &s, float w, float a, float b)
     s.PS = fmaf(w, m, s.PS);
 }
 
-// Voxel normal of Eq. vox_normal from the 8 raw corner densities (corner c:
-// bit 2 = x, bit 1 = y, bit 0 = z; g0 = corners 0..3, g1 = 4..7): the
-// gradient of the trilinear field at the centre, Eq. interp_grad (a quarter
-// of far face minus near face per axis; the factor cancels here), normalised;
-// zero where the gradient vanishes.  Returns the gradient's length (of the
-// unscaled differences times 1/4).
+// Voxel normal of Eq. vox_normal from the density polynomial: the gradient of
+// the trilinear field at the centre, Eq. interp_grad, is its linear
+// coefficients; normalised, zero where the gradient vanishes.  Returns the
+// gradient's length.
 __device__ __forceinline__ float voxel_normal(const float4 &g0, const float4 &g1, float3 &n) {
-    const float gx = 0.25f * ((g1.x + g1.y + g1.z + g1.w) - (g0.x + g0.y + g0.z + g0.w));
-    const float gy = 0.25f * ((g0.z + g0.w + g1.z + g1.w) - (g0.x + g0.y + g1.x + g1.y));
-    const float gz = 0.25f * ((g0.y + g0.w + g1.y + g1.w) - (g0.x + g0.z + g1.x + g1.z));
+    const float gx = g1.x, gy = g0.z, gz = g0.y;
     const float len = sqrtf(gx * gx + gy * gy + gz * gz);
     const float inv = len > 0.f ? 1.0f / len : 0.f;
     n = make_float3(gx * inv, gy * inv, gz * inv);
@@ -575,8 +569,8 @@ __device__ __forceinline__ float voxel_normal(const float4 &g0, const float4 &g1
 // lanes reading different slots over the shared-memory banks.
 struct FwdSlot {
     float4 a;    // copied: min corner relative to r_o, size; then: entry plane, 1 / size
-    float4 g0;   // raw corner densities 0..3
-    float4 g1;   // raw corner densities 4..7
+    float4 g0;   // density polynomial: 1, z, y, yz
+    float4 g1;   // x, xz, xy, xyz
     float4 col;  // colour, clamp bits
     float4 b;    // exit plane
 };
@@ -645,12 +639,12 @@ __device__ __forceinline__ void hit_fwd_slot(const FwdSlot &e, const PixelRay &p
                                              float b, float &trans, float &dloc, float &alpha) {
     const float inv_k = 1.0f / K;
     const float seg = b - a;
-    const float xs = seg * p.rdn * inv_k;
+    const float xs = seg * p.rdn * (inv_k * kLog2e);   // optical depths in units of ln 2
     const float step = seg * inv_k;
     const float4 ea = e.a, eb = e.b;
     const float inv = ea.w;
-    const float cx = (sb.x != 0.f ? eb.x : ea.x) * inv, cy = (sb.y != 0.f ? eb.y : ea.y) * inv,
-                cz = (sb.z != 0.f ? eb.z : ea.z) * inv;
+    const float cx = fmaf(sb.x != 0.f ? eb.x : ea.x, inv, 0.5f), cy = fmaf(sb.y != 0.f ? eb.y : ea.y, inv, 0.5f),
+                cz = fmaf(sb.z != 0.f ? eb.z : ea.z, inv, 0.5f);
     const float4 g0 = e.g0, g1 = e.g1;
     const float rx = p.rd.x * inv, ry = p.rd.y * inv, rz = p.rd.z * inv;
     float t = fmaf(0.5f, step, a);
@@ -659,7 +653,7 @@ __device__ __forceinline__ void hit_fwd_slot(const FwdSlot &e, const PixelRay &p
     for (int k = 0; k < K; ++k) {
         const float v = trilerp(g0, g1, fmaf(t, rx, -cx), fmaf(t, ry, -cy), fmaf(t, rz, -cz));
         const float xk = xs * explin(v);
-        const float ek = __expf(-xk);
+        const float ek = ex2(-xk);
         d = fmaf(P * (1.f - ek), t, d);
         P *= ek;
         X += xk;
@@ -667,7 +661,7 @@ __device__ __forceinline__ void hit_fwd_slot(const FwdSlot &e, const PixelRay &p
     }
     trans = P;
     dloc = d;
-    alpha = seg_alpha(X, P);
+    alpha = seg_alpha(X * kLn2, P);
 }
 
 // Phase B of a batch, hit-parallel: the batch's (pixel, entry) hits are
@@ -1192,7 +1186,7 @@ __device__ __forceinline__ void hit_grad(const Entry &e, const PixelRay &p, cons
                                          float &w, float &dloc, float3 &nrm, float &prio, float &cdist) {
     const float inv_k = 1.0f / K;
     const float seg = b - a;
-    const float xs = seg * p.rdn * inv_k;
+    const float xs = seg * p.rdn * inv_k, xs2 = xs * kLog2e;   // X: optical depth in units of ln 2
     const float step = seg * inv_k;
     const float inv_size = e.b.w;
     const float rx = p.rd.x * inv_size, ry = p.rd.y * inv_size, rz = p.rd.z * inv_size;
@@ -1207,8 +1201,8 @@ __device__ __forceinline__ void hit_grad(const Entry &e, const PixelRay &p, cons
         const float v = trilerp(e.g0, e.g1, qx[k], qy[k], qz[k]);
         const float sig = explin(v);
         dsig[k] = v > 1.1f ? 1.f : sig * 0.909090909f;
-        const float xk = xs * sig;
-        ek[k] = __expf(-xk);
+        const float xk = xs2 * sig;
+        ek[k] = ex2(-xk);
         X += xk;
         tk[k] = t;
         d = fmaf(trans * (1.f - ek[k]), t, d);
@@ -1224,7 +1218,7 @@ __device__ __forceinline__ void hit_grad(const Entry &e, const PixelRay &p, cons
         T_i = T_known;
         T_after = T_known * trans;
     }
-    const float al = seg_alpha(X, trans);
+    const float al = seg_alpha(X * kLn2, trans);
     w = T_i * al;
     dloc = d;
     float nlen = 0.f;
@@ -1273,54 +1267,66 @@ __device__ __forceinline__ void hit_grad(const Entry &e, const PixelRay &p, cons
     for (int k = K - 1; k >= 0; --k) {
         const float gxk = fmaf(gdT, fmaf(Pk[k + 1], tk[k], -Q), gx);
         const float dv = gxk * xs * dsig[k];
-        // trilinear adjoint, the x and y weights folded into dv first
-        const float ax1 = dv * qx[k], ax0 = dv - ax1;
-        const float b01 = ax0 * qy[k], b00 = ax0 - b01, b11 = ax1 * qy[k], b10 = ax1 - b11;
-        const float uz = 1.f - qz[k];
-        dgeo[0] = fmaf(b00, uz, dgeo[0]);
-        dgeo[1] = fmaf(b00, qz[k], dgeo[1]);
-        dgeo[2] = fmaf(b01, uz, dgeo[2]);
-        dgeo[3] = fmaf(b01, qz[k], dgeo[3]);
-        dgeo[4] = fmaf(b10, uz, dgeo[4]);
-        dgeo[5] = fmaf(b10, qz[k], dgeo[5]);
-        dgeo[6] = fmaf(b11, uz, dgeo[6]);
-        dgeo[7] = fmaf(b11, qz[k], dgeo[7]);
+        // adjoint of the polynomial's coefficients (trilerp)
+        const float ax = dv * qx[k], ay = dv * qy[k], axy = ax * qy[k];
+        dgeo[0] += dv;
+        dgeo[1] = fmaf(dv, qz[k], dgeo[1]);
+        dgeo[2] += ay;
+        dgeo[3] = fmaf(ay, qz[k], dgeo[3]);
+        dgeo[4] += ax;
+        dgeo[5] = fmaf(ax, qz[k], dgeo[5]);
+        dgeo[6] += axy;
+        dgeo[7] = fmaf(axy, qz[k], dgeo[7]);
         Q = fmaf(Pk[k] * (1.f - ek[k]), tk[k], Q);
     }
     // normal: dL/dn = w g_N, through the normalisation (I - n n^T) / |grad|
-    // and Eq. interp_grad_grad: dgrad/dV_c = (2 x_c - 1, 2 y_c - 1, 2 z_c - 1) / 4
+    // to the linear coefficients (Eq. interp_grad_grad)
     if (XN && nlen > 0.f) {
         const float dnx = w * g.gN0, dny = w * g.gN1, dnz = w * g.gN2;
         const float dot = dnx * nrm.x + dny * nrm.y + dnz * nrm.z;
-        const float il = 0.25f / nlen;
-        const float gx_ = (dnx - nrm.x * dot) * il, gy_ = (dny - nrm.y * dot) * il, gz_ = (dnz - nrm.z * dot) * il;
-#pragma unroll
-        for (int c = 0; c < 8; ++c)
-            dgeo[c] += ((c & 4) ? gx_ : -gx_) + ((c & 2) ? gy_ : -gy_) + ((c & 1) ? gz_ : -gz_);
+        const float il = 1.0f / nlen;
+        dgeo[4] += (dnx - nrm.x * dot) * il;
+        dgeo[2] += (dny - nrm.y * dot) * il;
+        dgeo[1] += (dnz - nrm.z * dot) * il;
     }
 }
 
 // ------------------------------------------------------- gradient records
 //
-// The gradients of one batch's hits go to per-hit records of kRec floats (8
-// corner densities, 3 colour channels) laid out entry by entry: the hits of
-// staged entry j get consecutive slots, in pixel order, so a lane writes each
-// of its hits' records to a slot of its own with no coordination.  Once the
-// hits are done, lane j sums entry j's records and adds the sums to the
-// global gradients (one set of atomics per entry and warp).  At most kRecCap
-// records are held at a time: a batch with more hits is processed in runs of
-// consecutive entries, which keeps every pixel's hits in list order.
-constexpr int kRecStride = 12;   // floats per record slot: 11 used, 16-byte aligned
+// The gradients of one batch's hits go to per-hit records of 12 floats (8
+// density coefficients, 3 colour channels, the priority term) laid out entry by
+// entry: the hits of staged entry j get consecutive slots, in pixel order, so
+// a lane writes each of its hits' records to a slot of its own with no
+// coordination.  At most kRecCap records are held at a time: a batch with
+// more hits is processed in runs of consecutive entries, which keeps every
+// pixel's hits in list order.
+//
+// Once a run's hits are done, the lanes sum its records: lane l takes the
+// kRecLane slots from kRecLane l, and adds each stretch of one entry to the
+// voxel's accumulators in global memory with three 16-byte atomics (density
+// coefficients per voxel, colour and priority per view and voxel; k_voxel_bwd
+// takes them on to d_grid, d_sh and the priorities).  So the work is even
+// over the lanes whatever the entries' hit counts; with lane j summing entry
+// j's records, the warp waited for the entry with most hits (30 % of the
+// kernel, 16 mixed views: 4.99 ms in all), and each entry took 11 scalar
+// atomics after two loads of its corner indices.
 #ifndef SVR_BWD_REC_CAP
 #define SVR_BWD_REC_CAP 128
 #endif
 constexpr int kRecCap = SVR_BWD_REC_CAP;
+constexpr int kRecLane = kRecCap / 32;
+static_assert(kRecCap % 32 == 0, "the lanes share the slots evenly");
 
 struct RecSmem {
-    float4 rec[kRecCap * kRecStride / 4];
-    int off[kBatch];       // first slot of entry j (numbered over the whole batch)
-    unsigned pix[kBatch];  // lanes whose pixel hits entry j
+    float4 rec[kRecCap * 3 + 32];  // see rec_at
+    int off[kBatch];               // first slot of entry j (numbered over the whole batch)
+    unsigned pix[kBatch];          // lanes whose pixel hits entry j
+    uint8_t ent[kRecCap];          // staged entry of each slot
 };
+
+// Records are 48 bytes, with 16 free after every kRecLane of them: the lanes'
+// stretches then start in distinct banks.
+__device__ __forceinline__ int rec_at(int slot) { return slot * 3 + slot / kRecLane; }
 
 // Lays out the records of a batch from the lanes' hit masks; lane j returns
 // entry j's first slot and end slot, and the batch's record count.
@@ -1342,21 +1348,15 @@ __device__ __forceinline__ int rec_slot(const RecSmem &rs, int k, int base) {
     return rs.off[k] + __popc(rs.pix[k] & lt) - base;
 }
 
-// Record: 8 corner-density gradients, 3 colour gradients and the
-// subdivision priority term (extras; 0 otherwise).
-__device__ __forceinline__ void rec_write(RecSmem &rs, int slot, const float dgeo[8], const float dcol[3],
+// Record of a hit on entry k: 8 coefficient gradients, 3 colour gradients
+// and the subdivision priority term (extras; 0 otherwise).
+__device__ __forceinline__ void rec_write(RecSmem &rs, int slot, int k, const float dgeo[8], const float dcol[3],
                                           float prio) {
-    float4 *r = rs.rec + slot * (kRecStride / 4);
+    float4 *r = rs.rec + rec_at(slot);
     r[0] = make_float4(dgeo[0], dgeo[1], dgeo[2], dgeo[3]);
     r[1] = make_float4(dgeo[4], dgeo[5], dgeo[6], dgeo[7]);
     r[2] = make_float4(dcol[0], dcol[1], dcol[2], prio);
-}
-
-__device__ __forceinline__ void rec_add(float row[kRecStride], const float4 *r) {
-    const float4 a = r[0], b = r[1], c = r[2];
-    row[0] += a.x, row[1] += a.y, row[2] += a.z, row[3] += a.w;
-    row[4] += b.x, row[5] += b.y, row[6] += b.z, row[7] += b.w;
-    row[8] += c.x, row[9] += c.y, row[10] += c.z, row[11] += c.w;
+    rs.ent[slot] = (uint8_t)k;
 }
 
 // End of the run of entries from k_lo whose records fit in kRecCap slots
@@ -1367,47 +1367,47 @@ __device__ __forceinline__ int rec_run_end(int k_lo, int end, int base) {
     return 32 - __clz(fit);
 }
 
-// Adds an entry's summed record to the global gradients of voxel vid; a
-// colour channel that the clamp cut (bit clear) has no gradient.
-__device__ __forceinline__ void add_row(const float row[kRecStride], int vid, unsigned bits,
-                                        const int32_t *__restrict__ corner_idx, float *__restrict__ d_grid,
-                                        float *__restrict__ acc_col, float *__restrict__ priority,
-                                        DebugBlock *dbg, int64_t n_pts) {
-    const int4 *ci = reinterpret_cast<const int4 *>(corner_idx + 8 * (size_t)vid);
-    const int4 i0 = __ldg(ci), i1 = __ldg(ci + 1);
-    if (!(SVR_IN_BOUNDS(dbg, kDbgGradPoint, i0.x, n_pts) && SVR_IN_BOUNDS(dbg, kDbgGradPoint, i0.y, n_pts) &&
-          SVR_IN_BOUNDS(dbg, kDbgGradPoint, i0.z, n_pts) && SVR_IN_BOUNDS(dbg, kDbgGradPoint, i0.w, n_pts) &&
-          SVR_IN_BOUNDS(dbg, kDbgGradPoint, i1.x, n_pts) && SVR_IN_BOUNDS(dbg, kDbgGradPoint, i1.y, n_pts) &&
-          SVR_IN_BOUNDS(dbg, kDbgGradPoint, i1.z, n_pts) && SVR_IN_BOUNDS(dbg, kDbgGradPoint, i1.w, n_pts)))
-        return;
-    atomicAdd(d_grid + i0.x, row[0]);
-    atomicAdd(d_grid + i0.y, row[1]);
-    atomicAdd(d_grid + i0.z, row[2]);
-    atomicAdd(d_grid + i0.w, row[3]);
-    atomicAdd(d_grid + i1.x, row[4]);
-    atomicAdd(d_grid + i1.y, row[5]);
-    atomicAdd(d_grid + i1.z, row[6]);
-    atomicAdd(d_grid + i1.w, row[7]);
-    if (bits & 1u) atomicAdd(acc_col + 3 * (size_t)vid + 0, row[8]);
-    if (bits & 2u) atomicAdd(acc_col + 3 * (size_t)vid + 1, row[9]);
-    if (bits & 4u) atomicAdd(acc_col + 3 * (size_t)vid + 2, row[10]);
-    if (priority) atomicAdd(priority + vid, row[11]);
+__device__ __forceinline__ void add4(float4 &a, const float4 &b) {
+    a.x += b.x, a.y += b.y, a.z += b.z, a.w += b.w;
 }
 
-// Lane j in [k_lo, k_hi) sums entry j's records and adds the sums to the
-// global gradients of its voxel.
-__device__ __forceinline__ void rec_flush(const RecSmem &rs, const Entry *st, int k_lo, int k_hi, int off, int end,
-                                          int base, const FrameDev &f, float *__restrict__ d_grid,
-                                          float *__restrict__ acc_col, float *__restrict__ priority) {
-    const int lane = threadIdx.x & 31;
+// Adds a sum of entry e's records to its voxel's accumulators; a colour
+// channel that the clamp cut (bit clear) has no gradient.
+__device__ __forceinline__ void add_sum(const Entry &e, const float4 &g0, const float4 &g1, float4 c,
+                                        float4 *__restrict__ acc_grid, float4 *__restrict__ acc_col) {
+    const size_t vid = (size_t)__float_as_int(e.col.w);
+    const unsigned bits = __float_as_uint(e.a.w);
+    if (!(bits & 1u)) c.x = 0.f;
+    if (!(bits & 2u)) c.y = 0.f;
+    if (!(bits & 4u)) c.z = 0.f;
+    atomicAdd(acc_grid + 2 * vid, g0);
+    atomicAdd(acc_grid + 2 * vid + 1, g1);
+    atomicAdd(acc_col + vid, c);
+}
+
+// Sums the run's n records and adds the sums to the voxels' accumulators.
+__device__ __forceinline__ void rec_flush(const RecSmem &rs, const Entry *st, int n, float4 *__restrict__ acc_grid,
+                                          float4 *__restrict__ acc_col) {
     __syncwarp();
-    if (lane >= k_lo && lane < k_hi && end > off) {
-        float row[kRecStride];
+    const int r0 = (threadIdx.x & 31) * kRecLane;
+    if (r0 < n) {
+        int k = rs.ent[r0];
+        const float4 *r = rs.rec + rec_at(r0);
+        float4 g0 = r[0], g1 = r[1], c = r[2];
 #pragma unroll
-        for (int c = 0; c < kRecStride; ++c) row[c] = 0.f;
-        for (int r = off - base; r < end - base; ++r) rec_add(row, rs.rec + r * (kRecStride / 4));
-        add_row(row, __float_as_int(st[lane].col.w), __float_as_uint(st[lane].pad.x), f.corner_idx, d_grid, acc_col,
-                priority, f.debug, f.n_pts);
+        for (int i = 1; i < kRecLane; ++i) {
+            if (r0 + i >= n) break;
+            const int k2 = rs.ent[r0 + i];
+            if (k2 != k) {
+                add_sum(st[k], g0, g1, c, acc_grid, acc_col);
+                g0 = g1 = c = make_float4(0.f, 0.f, 0.f, 0.f);
+                k = k2;
+            }
+            add4(g0, r[3 * i]);
+            add4(g1, r[3 * i + 1]);
+            add4(c, r[3 * i + 2]);
+        }
+        add_sum(st[k], g0, g1, c, acc_grid, acc_col);
     }
     __syncwarp();
 }
@@ -1421,9 +1421,7 @@ __device__ __forceinline__ unsigned range_mask(int k_lo, int k_hi) {
 struct BwdIn {
     const float *d_rgb, *d_depth, *d_alpha, *T;
     const int32_t *last;
-    float *d_grid;
     const float *d_normal;  // extras: upstream gradient of the normal image [3][H][W], or NULL
-    float *priority;        // extras: [N] subdivision priority, accumulated, or NULL
     const float *d_dist;    // extras: upstream gradient of each ray's distortion loss [H][W], or NULL
     const float *dist;      // extras: the forward's [2][H][W] distortion output (plane 1: sum w m)
     float *max_weight;      // extras: [N] per-voxel maximum of T_i alpha_i (atomicMax), or NULL
@@ -1440,7 +1438,7 @@ __device__ __noinline__ void bwd_front_to_back(const FrameDev &f, const ItemList
                                                int last, bool fallback, float T_before, float SC0, float SC1, float SC2,
                                                float SD, NrmSums SN, DistSums DSb, const ViewData vd,
                                                const WarpBlock wb, const PixelRay p, const PixelGrad g, Entry *st,
-                                               RecSmem &rs, const BwdIn &in, float *dcol) {
+                                               RecSmem &rs, const BwdIn &in, float4 *dcol) {
     constexpr bool XN = (XM & kXNrm) != 0, XD = (XM & kXDist) != 0, XS = (XM & kXStat) != 0;
     const int lane = threadIdx.x & 31;
     const int n_fb = lower_pos(L.list, p0, p1, __reduce_max_sync(0xffffffffu, fallback ? last + 1 : idx0));
@@ -1562,9 +1560,9 @@ __device__ __noinline__ void bwd_front_to_back(const FrameDev &f, const ItemList
                     PR = fmaf(w_own, c_own, PR);
                 }
                 Tf = Ta;
-                rec_write(rs, checked(f.debug, kDbgRecSlot, rec_slot(rs, k, rb), kRecCap), dgeo, dc, prio);
+                rec_write(rs, checked(f.debug, kDbgRecSlot, rec_slot(rs, k, rb), kRecCap), k, dgeo, dc, prio);
             }
-            rec_flush(rs, st, k_lo, k_hi, off, end, rb, f, in.d_grid, dcol, XS ? in.priority : nullptr);
+            rec_flush(rs, st, __shfl_sync(0xffffffffu, end, k_hi - 1) - rb, f.dgrid, dcol);
             k_lo = k_hi;
             if (k_lo >= 32) break;
         }
@@ -1579,7 +1577,7 @@ __device__ __forceinline__ void bwd_item(const FrameDev &f, const Item &it, Entr
     const ItemView iv = item_view(f, it.g);
     const DevCam &cam = f.views[iv.view];
     const ViewData &vd = iv.vd;
-    float *dcol = f.dcol + 3 * (size_t)iv.view * f.n_vox;
+    float4 *dcol = f.dcol + (size_t)iv.view * f.n_vox;
     WarpBlock wb;
     const PixelRay p = pixel_ray(cam, iv.tile, it.blk, wb);
     if (wb.smask == 0) return;
@@ -1663,7 +1661,6 @@ __device__ __forceinline__ void bwd_item(const FrameDev &f, const Item &it, Entr
     const bool has = p.inside && last >= idx0;
     const bool fallback = has && T_after < 1e-30f;
     const bool active = has && !fallback;
-    float *prio_out = XS ? in.priority : nullptr;
 
     // ---- back to front, over the forward's batches [p0 + 32 k, p0 + 32 k + 32):
     // each pixel's hits in a batch are the forward's hit mask (which tested
@@ -1693,14 +1690,21 @@ __device__ __forceinline__ void bwd_item(const FrameDev &f, const Item &it, Entr
             // staged indices fall with j (lane j: list position base + 31 - j):
             // the first j whose index is <= last
             const int idx_j = cur.valid ? (int)cur.vi.y : INT_MAX;
-            int lo = 0, hi = kBatch;
+            int lo = max(0, base + kBatch - top_all), hi = kBatch;   // lo: the first valid lane
+            // only a pixel that stopped inside the batch has hits behind its
+            // last voxel (or, in a split list, one that stopped before its
+            // segment's own walk did): most batches need no search
+            const int idx_top = __shfl_sync(0xffffffffu, idx_j, lo);
+            const bool cut = active && m != 0u && last < idx_top;
+            if (__any_sync(0xffffffffu, cut)) {
 #pragma unroll
-            for (int step = 0; step < 6; ++step) {
-                const int mid = (lo + hi) >> 1;
-                const int v = __shfl_sync(0xffffffffu, idx_j, mid & 31);
-                if (lo < hi) {
-                    if (v > last) lo = mid + 1;
-                    else hi = mid;
+                for (int step = 0; step < 6; ++step) {
+                    const int mid = (lo + hi) >> 1;
+                    const int v = __shfl_sync(0xffffffffu, idx_j, mid & 31);
+                    if (lo < hi) {
+                        if (v > last) lo = mid + 1;
+                        else hi = mid;
+                    }
                 }
             }
             const unsigned hits = active && lo < kBatch ? __brev(m) & (0xffffffffu << lo) : 0u;
@@ -1745,9 +1749,9 @@ __device__ __forceinline__ void bwd_item(const FrameDev &f, const Item &it, Entr
                         DS.R = fmaf(w, cdist, DS.R);
                     }
                     T_after = T_i;
-                    rec_write(rs, checked(f.debug, kDbgRecSlot, rec_slot(rs, k, base), kRecCap), dgeo, dc, prio);
+                    rec_write(rs, checked(f.debug, kDbgRecSlot, rec_slot(rs, k, base), kRecCap), k, dgeo, dc, prio);
                 }
-                rec_flush(rs, st, k_lo, k_hi, off, end, base, f, in.d_grid, dcol, prio_out);
+                rec_flush(rs, st, __shfl_sync(0xffffffffu, end, k_hi - 1) - base, f.dgrid, dcol);
                 k_lo = k_hi;
                 if (k_lo >= 32) break;
             }
@@ -1779,14 +1783,16 @@ __global__ void __launch_bounds__(kBwdThreads, kBwdMinBlocks) k_render_bwd(Frame
 
 // Per voxel: dL/dsh[n][c] = sum over views of Y_n(d_v) * dL/dc_{v,c}, over
 // the views where the voxel is in view (dL/dc_{v,c} holds only the channels
-// that were > 0 before the clamp, Eq. vox_color); zero for a voxel in no view.  Each thread sums its
+// that were > 0 before the clamp, Eq. vox_color); zero for a voxel in no view;
+// and its priority terms, added to the priorities.  Each thread sums its
 // voxel's 48 values in registers and stores them to a shared row (rows 52
 // floats apart: float4 stores of a quarter warp fall in distinct banks); the
 // block then writes its rows as consecutive float4s.
 constexpr int kVoxBwdThreads = 128;
 constexpr int kShRow = 52;
 
-__global__ void __launch_bounds__(kVoxBwdThreads) k_voxel_bwd(FrameDev f, float *__restrict__ d_sh) {
+__global__ void __launch_bounds__(kVoxBwdThreads) k_voxel_bwd(FrameDev f, float *__restrict__ d_sh,
+                                                              float *__restrict__ priority) {
     __shared__ __align__(16) float rows[kVoxBwdThreads * kShRow];
     const int64_t v0 = (int64_t)blockIdx.x * kVoxBwdThreads;
     const int64_t v = v0 + threadIdx.x;
@@ -1794,11 +1800,13 @@ __global__ void __launch_bounds__(kVoxBwdThreads) k_voxel_bwd(FrameDev f, float 
         float o[48];
 #pragma unroll
         for (int i = 0; i < 48; ++i) o[i] = 0.f;
+        float prio = 0.f;
         for (int view = 0; view < f.n_views; ++view) {
             const int64_t iv = (int64_t)view * f.n_vox + v;
             if (f.count[iv] == 0) continue;
             const DevCam &cam = f.views[view];
-            const float g0 = f.dcol[3 * iv + 0], g1 = f.dcol[3 * iv + 1], g2 = f.dcol[3 * iv + 2];
+            const float4 g = f.dcol[iv];
+            prio += g.w;
             float dx = f.centre[3 * v + 0] - cam.ro[0];
             float dy = f.centre[3 * v + 1] - cam.ro[1];
             float dz = f.centre[3 * v + 2] - cam.ro[2];
@@ -1807,14 +1815,15 @@ __global__ void __launch_bounds__(kVoxBwdThreads) k_voxel_bwd(FrameDev f, float 
             sh_basis(dx * inv, dy * inv, dz * inv, Y);
 #pragma unroll
             for (int n = 0; n < 16; ++n) {
-                o[3 * n + 0] = fmaf(Y[n], g0, o[3 * n + 0]);
-                o[3 * n + 1] = fmaf(Y[n], g1, o[3 * n + 1]);
-                o[3 * n + 2] = fmaf(Y[n], g2, o[3 * n + 2]);
+                o[3 * n + 0] = fmaf(Y[n], g.x, o[3 * n + 0]);
+                o[3 * n + 1] = fmaf(Y[n], g.y, o[3 * n + 1]);
+                o[3 * n + 2] = fmaf(Y[n], g.z, o[3 * n + 2]);
             }
         }
         float4 *row = reinterpret_cast<float4 *>(rows + threadIdx.x * kShRow);
 #pragma unroll
         for (int q = 0; q < 12; ++q) row[q] = make_float4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
+        if (priority && prio != 0.f) priority[v] += prio;
     }
     __syncthreads();
     const int nv = (int)tmin<int64_t>(kVoxBwdThreads, f.n_vox - v0);
@@ -1824,6 +1833,46 @@ __global__ void __launch_bounds__(kVoxBwdThreads) k_voxel_bwd(FrameDev f, float 
         const int r = i / 12;
         out[i] = src[r * (kShRow / 4) + (i - 12 * r)];
     }
+}
+
+// The voxels' density gradients, summed over all hits in all views, taken
+// from the polynomial's coefficients to the corners and added to the grid
+// points (a voxel that no pixel hit has none).  Eight lanes take a voxel's
+// eight corners, so that the corner indices are read coalesced and the
+// adjacent grid points of corners 2 i and 2 i + 1 share a sector of one
+// instruction.  Bound by the latency of its two dependent loads and the
+// scattered atomics: kGridIlp corners per thread are in flight.  A kernel of
+// its own, before k_voxel_bwd while the accumulators are in L2: inside it,
+// 79 us (1M voxels) and 1.28 ms (8M, 8 views) for both against 37 + 37 us and
+// 0.31 + 0.72 ms; as other CTAs of one launch, 116 us and 1.54 ms.
+constexpr int kGridThreads = 256, kGridIlp = 4;
+
+__global__ void __launch_bounds__(kGridThreads) k_grid_bwd(FrameDev f, float *__restrict__ d_grid) {
+    const int c = threadIdx.x & 7;
+    const float sz = (c & 1) ? 1.f : -1.f, sy = (c & 2) ? 1.f : -1.f, sx = (c & 4) ? 1.f : -1.f;
+    const int64_t n = f.n_vox * 8;
+    const int64_t i0 = (int64_t)blockIdx.x * (kGridThreads * kGridIlp) + threadIdx.x;   // corners of all voxels
+    float d[kGridIlp];
+    float4 g0[kGridIlp], g1[kGridIlp];
+#pragma unroll
+    for (int r = 0; r < kGridIlp; ++r) {
+        const int64_t i = i0 + r * kGridThreads;
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        g0[r] = i < n ? __ldg(f.dgrid + 2 * (i >> 3)) : zero;
+        g1[r] = i < n ? __ldg(f.dgrid + 2 * (i >> 3) + 1) : zero;
+    }
+    int p[kGridIlp];
+#pragma unroll
+    for (int r = 0; r < kGridIlp; ++r) {
+        // corner c's share: half a mean plus or minus a difference, per axis
+        const float a = fmaf(0.5f, g0[r].x, sx * g1[r].x), b = fmaf(0.5f, g0[r].y, sx * g1[r].y);
+        const float e = fmaf(0.5f, g0[r].z, sx * g1[r].z), h = fmaf(0.5f, g0[r].w, sx * g1[r].w);
+        d[r] = fmaf(0.5f, fmaf(0.5f, a, sy * e), sz * fmaf(0.5f, b, sy * h));
+        p[r] = d[r] != 0.f ? __ldg(f.corner_idx + i0 + r * kGridThreads) : 0;
+    }
+#pragma unroll
+    for (int r = 0; r < kGridIlp; ++r)
+        if (d[r] != 0.f && SVR_IN_BOUNDS(f.debug, kDbgGradPoint, p[r], f.n_pts)) atomicAdd(d_grid + p[r], d[r]);
 }
 
 // ---------------------------------------------------------------- launchers
@@ -1917,9 +1966,9 @@ cudaError_t launch_render_bwd(const FrameDev &f, const float *d_rgb, const float
                               const float *dist, float *max_weight, cudaStream_t s) {
     cudaError_t e = cudaMemsetAsync(&f.status->bwd_next, 0, sizeof(unsigned), s);
     if (e == cudaSuccess && f.n_vox > 0)
-        e = cudaMemsetAsync(f.dcol, 0, sizeof(float) * 3 * (size_t)f.n_vox * f.n_views, s);
+        e = cudaMemsetAsync(f.dcol, 0, sizeof(float4) * (size_t)f.n_vox * (f.n_views + 2), s);  // dcol and dgrid
     if (e != cudaSuccess) return e;
-    const BwdIn in = {d_rgb, d_depth, d_alpha, T_final, last, d_grid, d_normal, priority, d_dist, dist, max_weight};
+    const BwdIn in = {d_rgb, d_depth, d_alpha, T_final, last, d_normal, d_dist, dist, max_weight};
     // extras: none; the distortion gradient alone (the training step's); it
     // and the pruning/subdivision statistics (the training step that gathers
     // them); every extra (the normal gradient as well)
@@ -1942,7 +1991,10 @@ cudaError_t launch_render_bwd(const FrameDev &f, const float *d_rgb, const float
     }
     if (e != cudaSuccess) return e;
     if (f.n_vox > 0) {
-        k_voxel_bwd<<<(unsigned)((f.n_vox + kVoxBwdThreads - 1) / kVoxBwdThreads), kVoxBwdThreads, 0, s>>>(f, d_sh);
+        const unsigned blocks = (unsigned)((f.n_vox + kVoxBwdThreads - 1) / kVoxBwdThreads);
+        const int64_t per = kGridThreads * kGridIlp / 8;
+        k_grid_bwd<<<(unsigned)((f.n_vox + per - 1) / per), kGridThreads, 0, s>>>(f, d_grid);
+        k_voxel_bwd<<<blocks, kVoxBwdThreads, 0, s>>>(f, d_sh, priority);
         e = cudaGetLastError();
     }
     return e;

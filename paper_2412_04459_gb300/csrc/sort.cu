@@ -480,7 +480,8 @@ static cudaError_t sort_lists(const FrameDev &f, cudaStream_t s) {
     });
     k_sort_lists<MODE><<<(unsigned)tmin<int64_t>(units, resident), kSortThreads, kSortSmemBytes, s>>>(f);
     e = cudaGetLastError();
-    if (e != cudaSuccess || f.capacity <= kSortCap) return e;
+    // no list can be longer than every voxel with every sign pattern
+    if (e != cudaSuccess || f.capacity <= kSortCap || 8 * f.n_vox <= kSortCap) return e;
     // clusters: one per possible long list, at most two CTAs per SM
     const int64_t lists = f.capacity / kSortCap;
     const unsigned clusters = (unsigned)tmin<int64_t>(lists, tmin<int64_t>(f.total_tiles, sm_count() / (kMergeCluster / 2)));

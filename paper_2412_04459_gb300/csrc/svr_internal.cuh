@@ -161,8 +161,9 @@ DebugBlock *debug_block();
 
 // Per-voxel record of one view (64 bytes):
 //   r0 = (lo - r_o).xyz, size      lo = centre - size / 2, the min corner
-//   r1 = corner densities 0..3     (raw, gathered from the grid)
-//   r2 = corner densities 4..7
+//   r1, r2 = the raw density as a polynomial about the voxel's centre, from
+//            the 8 gathered corner densities: coefficients of 1, z, y, yz and
+//            x, xz, xy, xyz (see density_coeffs)
 //   r3 = colour rgb, bit c of the w word set if channel c was > 0 before the clamp
 // Asynchronous 16-byte global -> shared copy (cp.async, L2 only), its
 // commit and the wait for all but the N most recent groups.
@@ -195,10 +196,46 @@ __device__ __forceinline__ int sign_bits(float3 d) {
     return (d.x < 0.f ? 4 : 0) | (d.y < 0.f ? 2 : 0) | (d.z < 0.f ? 1 : 0);
 }
 
-// explin (Eq. explin): x above 1.1, else exp(x / 1.1 - 1 + ln 1.1).
-__device__ __forceinline__ float explin(float x) {
-    return x > 1.1f ? x : __expf(fmaf(x, 0.909090909f, -0.904689820f));
+// Trilinear interpolation of Eq. interp written about the voxel's centre: with
+// x, y, z in [-1/2, 1/2] the raw density is sum_m a_m x^i y^j z^k over m = 4 i
+// + 2 j + k, whose coefficients follow from the corners g (corner bit order
+// as m's) by taking mean and difference along each axis in turn.  Seven
+// multiply-adds evaluate it, against four differences, seven multiply-adds
+// and three more differences per sample from the corners.
+// The linear ones, whose direction is the voxel's normal, are taken as far
+// face minus near face, so that a nearly constant voxel's normal does not
+// depend on the order of the axes.
+__device__ __forceinline__ void density_coeffs(float g[8]) {
+    const float gx = 0.25f * ((g[4] + g[5] + g[6] + g[7]) - (g[0] + g[1] + g[2] + g[3]));
+    const float gy = 0.25f * ((g[2] + g[3] + g[6] + g[7]) - (g[0] + g[1] + g[4] + g[5]));
+    const float gz = 0.25f * ((g[1] + g[3] + g[5] + g[7]) - (g[0] + g[2] + g[4] + g[6]));
+#pragma unroll
+    for (int bit = 1; bit < 8; bit *= 2)
+#pragma unroll
+        for (int m = 0; m < 8; ++m)
+            if (!(m & bit)) {
+                const float lo = g[m], hi = g[m + bit];
+                g[m] = 0.5f * (lo + hi);
+                g[m + bit] = hi - lo;
+            }
+    g[1] = gz;
+    g[2] = gy;
+    g[4] = gx;
 }
+
+// 2^x.  The hardware instruction on its own: expf's fast form adds a multiply
+// by log2(e) and, without flush to zero, three more instructions that keep
+// results below 2^-126, which no sum here can show.
+__device__ __forceinline__ float ex2(float x) {
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+constexpr float kLog2e = 1.44269504f, kLn2 = 0.693147181f;
+
+// explin (Eq. explin): x above 1.1, else exp(x / 1.1 - 1 + ln 1.1), whose
+// exponent in base 2 is (x / 1.1 - 1 + ln 1.1) log2(e).
+__device__ __forceinline__ float explin(float x) { return x > 1.1f ? x : ex2(fmaf(x, 1.31154095f, -1.30519153f)); }
 
 // Real SH basis, degree 0..3, index l*l + l + m, no Condon-Shortley phase,
 // as polynomials of the unit direction (x, y, z).  Constants are
@@ -266,7 +303,8 @@ struct FrameDev {
                              // p in batch [32 k, 32 k + 32) of the block's walk, the mask of the
                              // batch's entries (bit i: position 32 k + i) that pixel p mod 32 hit
     int blocks_per_tile;     // B = tile * tile / 32
-    float *dcol;             // [V * N][3] colour gradient accumulator
+    float4 *dcol;            // [V * N] colour gradient and priority accumulators
+    float4 *dgrid;           // [N][2] density-coefficient gradient accumulators (after dcol)
     int64_t n_vox;
     int64_t n_pts;
     int64_t capacity;
