@@ -36,34 +36,66 @@ namespace svr {
 
 // --------------------------------------------------------------- tile masks
 
-// One warp per tile, looping over its 8x4 pixel blocks (the render's warp
-// blocks, tile / 8 per block row): each block's sign-bit mask goes to
-// block_sign, their OR to tile_mask.
-constexpr int kMaskWarps = 8;
+// A ray component is a rounded affine function of the pixel, monotonic along
+// each image axis, so where the four corner pixels of a tile agree in its sign
+// every pixel between does, and the tile and its blocks hold that one pattern.
+// Four lanes take a tile's corners.  The few tiles whose corners differ (or
+// whose rays overflow) are walked by the whole warp, 8x4 pixel block by block
+// (the render's warp blocks, tile / 8 per block row): each block's sign-bit
+// mask goes to block_sign, their OR to tile_mask.  A warp takes up to eight
+// tiles at a time, which lie far apart, so that a row of tiles along an axis of
+// the image is walked by many warps.
+// Every tile walked, at two divisions per pixel, was 100 us of the 8 x
+// 2560x1440 batch; a warp's tiles side by side, 74 us.
+constexpr int kMaskThreads = 128;
+constexpr int kMaskWarps = 4096;
 
-__global__ void __launch_bounds__(32 * kMaskWarps) k_tile_mask(FrameDev f) {
+__global__ void __launch_bounds__(kMaskThreads) k_tile_mask(FrameDev f) {
     // also starts the frame: status cleared (no smallest invalid voxel yet)
     // and the tiles' pair counters zeroed, before k_preprocess counts
     if (blockIdx.x == 0 && threadIdx.x < sizeof(Status) / 4)
         reinterpret_cast<unsigned *>(f.status)[threadIdx.x] =
             threadIdx.x == offsetof(Status, bad_voxel) / 4 ? 0xFFFFFFFFu : 0u;
-    const int g = blockIdx.x * kMaskWarps + (threadIdx.x >> 5);
-    if (g >= f.total_tiles) return;
-    if ((threadIdx.x & 31) < kTileSub) f.tile_cnt[(size_t)(threadIdx.x & 31) * f.total_tiles + g] = 0u;
-    const DevCam &cam = f.views[view_of_tile(f, g)];
-    const int tile = g - cam.tile_base;
-    const int T = cam.tile, bpr = T >> 3, B = f.blocks_per_tile;
-    const int x0 = (tile % cam.ntx) * T, y0 = (tile / cam.ntx) * T;
     const int lane = threadIdx.x & 31;
-    unsigned m = 0;
-    for (int b = 0; b < B; ++b) {
-        const int x = x0 + (b % bpr) * 8 + (lane & 7), y = y0 + (b / bpr) * 4 + (lane >> 3);
-        const unsigned bit = (x < cam.W && y < cam.H) ? 1u << sign_bits(pixel_dir(cam, x, y)) : 0u;
-        const unsigned bm = __reduce_or_sync(0xffffffffu, bit);
-        if (lane == b) f.block_sign[(size_t)g * B + b] = (uint8_t)bm;
-        m |= bm;
+    const int n_threads = gridDim.x * kMaskThreads, n_warps = n_threads / 32;
+    const int warp = blockIdx.x * (kMaskThreads / 32) + (threadIdx.x >> 5);
+    for (int64_t i = blockIdx.x * kMaskThreads + threadIdx.x; i < (int64_t)kTileSub * f.total_tiles; i += n_threads)
+        f.tile_cnt[i] = 0u;
+    const int B = f.blocks_per_tile;
+    for (int base = 0; base + warp < f.total_tiles; base += 8 * n_warps) {
+        const int g = base + (lane >> 2) * n_warps + warp, c = lane & 3;
+        const bool valid = g < f.total_tiles;
+        const DevCam &cam = f.views[view_of_tile(f, valid ? g : base + warp)];
+        const int T = cam.tile, bpr = T >> 3, tile = (valid ? g : base + warp) - cam.tile_base;
+        const int x0 = (tile % cam.ntx) * T, y0 = (tile / cam.ntx) * T;
+        const int x1 = min(x0 + T, cam.W) - 1, y1 = min(y0 + T, cam.H) - 1;
+        const float3 d = pixel_dir(cam, (c & 1) ? x1 : x0, (c & 2) ? y1 : y0);
+        const int s = isfinite(d.x) && isfinite(d.y) && isfinite(d.z) ? sign_bits(d) : 8;
+        const int s0 = __shfl_sync(0xffffffffu, s, lane & ~3);
+        const unsigned differ = __ballot_sync(0xffffffffu, s != s0 || s == 8);
+        const bool walk = valid && ((differ >> (lane & ~3)) & 0xFu) != 0u;
+        if (valid && !walk) {
+            for (int b = c; b < B; b += 4)
+                f.block_sign[(size_t)g * B + b] =
+                    x0 + (b % bpr) * 8 <= x1 && y0 + (b / bpr) * 4 <= y1 ? (uint8_t)(1u << s) : (uint8_t)0;
+            if (c == 0) f.tile_mask[g] = (uint8_t)(1u << s);
+        }
+        for (unsigned todo = __ballot_sync(0xffffffffu, walk && c == 0); todo; todo &= todo - 1u) {
+            const int h = __shfl_sync(0xffffffffu, g, __ffs(todo) - 1);
+            const DevCam &hc = f.views[view_of_tile(f, h)];
+            const int ht = h - hc.tile_base;
+            const int hx = (ht % hc.ntx) * T, hy = (ht / hc.ntx) * T;
+            unsigned m = 0;
+            for (int b = 0; b < B; ++b) {
+                const int x = hx + (b % bpr) * 8 + (lane & 7), y = hy + (b / bpr) * 4 + (lane >> 3);
+                const unsigned bit = (x < hc.W && y < hc.H) ? 1u << sign_bits(pixel_dir(hc, x, y)) : 0u;
+                const unsigned bm = __reduce_or_sync(0xffffffffu, bit);
+                if (lane == b) f.block_sign[(size_t)h * B + b] = (uint8_t)bm;
+                m |= bm;
+            }
+            if (lane == 0) f.tile_mask[h] = (uint8_t)m;
+        }
     }
-    if (lane == 0) f.tile_mask[g] = (uint8_t)m;
 }
 
 // --------------------------------------------------------------- preprocess
@@ -111,12 +143,48 @@ __device__ __forceinline__ bool voxel_valid(const FrameDev &f, int64_t v, float 
     return ok && lo >= 0 && (int64_t)hi < np;
 }
 
-// Projection of voxel v in one view: tile rectangle, conservative pixel box
-// and pair count (the tiles' counts raised by atomics); writes rect and
-// count of (view, voxel) iv and returns the count.
-__device__ __forceinline__ uint32_t project_voxel(const FrameDev &f, const DevCam &cam, int64_t v, int64_t iv,
-                                                  float c0, float c1, float c2, float h, ushort4 &box) {
-    float umin = INFINITY, umax = -INFINITY, vmin = INFINITY, vmax = -INFINITY;
+// Pixel box of a voxel across the camera plane (some corners at depth <=
+// kNear): its rectangle is the whole image, but a ray meets only the part in
+// front, whose points have X / Z beyond the nearest X over the largest Z where
+// the voxel lies to one side of the axis (the same for Y).  Widened by a margin
+// far above the rounding of the projection and of the ray test; empty
+// (x0 > x1) where no pixel is left, which is usual: most such voxels lie far
+// to the side.
+__device__ __noinline__ ushort4 straddle_box(const DevCam &cam, float c0, float c1, float c2, float h) {
+    float X0 = INFINITY, X1 = -INFINITY, Y0 = INFINITY, Y1 = -INFINITY, Z1 = -INFINITY;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        const float px = (c & 4) ? c0 + h : c0 - h;
+        const float py = (c & 2) ? c1 + h : c1 - h;
+        const float pz = (c & 1) ? c2 + h : c2 - h;
+        const float X = fmaf(cam.R[0], px, fmaf(cam.R[1], py, fmaf(cam.R[2], pz, cam.t[0])));
+        const float Y = fmaf(cam.R[3], px, fmaf(cam.R[4], py, fmaf(cam.R[5], pz, cam.t[1])));
+        const float Z = fmaf(cam.R[6], px, fmaf(cam.R[7], py, fmaf(cam.R[8], pz, cam.t[2])));
+        X0 = fminf(X0, X);
+        X1 = fmaxf(X1, X);
+        Y0 = fminf(Y0, Y);
+        Y1 = fmaxf(Y1, Y);
+        Z1 = fmaxf(Z1, Z);
+    }
+    const float m = 2e-5f * (fmaxf(fabsf(X0), fabsf(X1)) + fmaxf(fabsf(Y0), fabsf(Y1)) + Z1 + h) +
+                    4e-6f * (fabsf(cam.t[0]) + fabsf(cam.t[1]) + fabsf(cam.t[2]) + fabsf(c0) + fabsf(c1) + fabsf(c2));
+    const float iz = 1.0f / (Z1 + m);
+    const float u0 = X0 - m > 0.f ? fmaf(cam.fx, (X0 - m) * iz, cam.cx) : -INFINITY;
+    const float u1 = X1 + m < 0.f ? fmaf(cam.fx, (X1 + m) * iz, cam.cx) : INFINITY;
+    const float v0 = Y0 - m > 0.f ? fmaf(cam.fy, (Y0 - m) * iz, cam.cy) : -INFINITY;
+    const float v1 = Y1 + m < 0.f ? fmaf(cam.fy, (Y1 + m) * iz, cam.cy) : INFINITY;
+    const float fx0 = fmaxf(floorf(u0 - 1.f - 1e-4f * fabsf(u0)), 0.f);
+    const float fx1 = fminf(floorf(u1 + 1.f + 1e-4f * fabsf(u1)), (float)(cam.W - 1));
+    const float fy0 = fmaxf(floorf(v0 - 1.f - 1e-4f * fabsf(v0)), 0.f);
+    const float fy1 = fminf(floorf(v1 + 1.f + 1e-4f * fabsf(v1)), (float)(cam.H - 1));
+    if (!(fx0 <= fx1 && fy0 <= fy1)) return make_ushort4(1, 0, 1, 0);
+    return make_ushort4((unsigned short)fx0, (unsigned short)fx1, (unsigned short)fy0, (unsigned short)fy1);
+}
+
+// Projection of a voxel in one view: tile rectangle and conservative pixel box.
+__device__ __forceinline__ short4 project_voxel(const DevCam &cam, float c0, float c1, float c2, float h,
+                                                ushort4 &box) {
+    float umin = INFINITY, umax = -INFINITY, vmin = INFINITY, vmax = -INFINITY, zmin = INFINITY;
     int behind = 0;
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
@@ -131,6 +199,7 @@ __device__ __forceinline__ uint32_t project_voxel(const FrameDev &f, const DevCa
         } else {
             const float u = fmaf(cam.fx, X / Z, cam.cx);
             const float w = fmaf(cam.fy, Y / Z, cam.cy);
+            zmin = fminf(zmin, Z);
             umin = fminf(umin, u);
             umax = fmaxf(umax, u);
             vmin = fminf(vmin, w);
@@ -143,15 +212,23 @@ __device__ __forceinline__ uint32_t project_voxel(const FrameDev &f, const DevCa
         // culled
     } else if (behind > 0) {
         rc = make_short4(0, (short)(cam.ntx - 1), 0, (short)(cam.nty - 1));
+        box = straddle_box(cam, c0, c1, c2, h);
     } else if (!(umax < 0.f || umin >= (float)cam.W || vmax < 0.f || vmin >= (float)cam.H)) {
         // pixels whose centre (x + 1/2, y + 1/2) can lie in the projected box,
-        // widened by a rounding margin: a conservative filter for the render
-        const float mu = 0.01f + 1e-5f * fmaxf(fabsf(umin), fabsf(umax));
-        const float mv = 0.01f + 1e-5f * fmaxf(fabsf(vmin), fabsf(vmax));
-        const float fx0 = fmaxf(floorf(umin - 0.5f - mu), 0.f), fx1 = fminf(floorf(umax - 0.5f + mu), (float)(cam.W - 1));
-        const float fy0 = fmaxf(floorf(vmin - 0.5f - mv), 0.f), fy1 = fminf(floorf(vmax - 0.5f + mv), (float)(cam.H - 1));
-        box = make_ushort4((unsigned short)fx0, (unsigned short)fmaxf(fx1, fx0), (unsigned short)fy0,
-                           (unsigned short)fmaxf(fy1, fy0));
+        // widened by a rounding margin: a conservative filter for the render.
+        // Empty (x0 > x1) for a voxel that falls between the pixel centres, as
+        // most of the finest ones do.
+        // The margin's last term is the rounding of coordinates far from the
+        // world's origin, in pixels.
+        const float e = 5e-7f / zmin *
+                        (fabsf(cam.t[0]) + fabsf(cam.t[1]) + fabsf(cam.t[2]) + fabsf(c0) + fabsf(c1) + fabsf(c2));
+        const float mu = 0.01f + 1e-5f * fmaxf(fabsf(umin), fabsf(umax)) + cam.fx * e;
+        const float mv = 0.01f + 1e-5f * fmaxf(fabsf(vmin), fabsf(vmax)) + cam.fy * e;
+        const float fx0 = fmaxf(ceilf(umin - 0.5f - mu), 0.f), fx1 = fminf(floorf(umax - 0.5f + mu), (float)(cam.W - 1));
+        const float fy0 = fmaxf(ceilf(vmin - 0.5f - mv), 0.f), fy1 = fminf(floorf(vmax - 0.5f + mv), (float)(cam.H - 1));
+        box = fx0 <= fx1 && fy0 <= fy1 ? make_ushort4((unsigned short)fx0, (unsigned short)fx1, (unsigned short)fy0,
+                                                      (unsigned short)fy1)
+                                       : make_ushort4(1, 0, 1, 0);
         const float T = (float)cam.tile;
         const int tx0 = umin < 0.f ? 0 : min(cam.ntx - 1, (int)floorf(umin / T));
         const int tx1 = umax >= (float)cam.W ? cam.ntx - 1 : min(cam.ntx - 1, (int)floorf(umax / T));
@@ -159,20 +236,60 @@ __device__ __forceinline__ uint32_t project_voxel(const FrameDev &f, const DevCa
         const int ty1 = vmax >= (float)cam.H ? cam.nty - 1 : min(cam.nty - 1, (int)floorf(vmax / T));
         rc = make_short4((short)tx0, (short)tx1, (short)ty0, (short)ty1);
     }
-    uint32_t cnt = 0;
+    return rc;
+}
+
+// Voxels over more tiles than this are counted and emitted by their whole
+// warp: those near the camera or across its plane cover up to every tile of
+// the image, and one thread at a time over them was 142 + 334 us of a 1.3 ms
+// view from inside a scene (1,200 tiles, 2,400 such voxels).
+constexpr int kCoopTiles = 16;
+
+__device__ __forceinline__ int rect_tiles(const short4 &rc) {
+    return max((int)rc.y - rc.x + 1, 0) * max((int)rc.w - rc.z + 1, 0);
+}
+
+__device__ __forceinline__ short4 shfl_rect(const short4 &rc, int src) {
+    const int lo = __shfl_sync(0xffffffffu, ((int)(unsigned short)rc.x) | ((int)rc.y << 16), src);
+    const int hi = __shfl_sync(0xffffffffu, ((int)(unsigned short)rc.z) | ((int)rc.w << 16), src);
+    return make_short4((short)(lo & 0xFFFF), (short)(lo >> 16), (short)(hi & 0xFFFF), (short)(hi >> 16));
+}
+
+// Pair count of voxel v with tile rectangle rc (the tiles' counts raised by
+// atomics).  Called by all lanes of the warp; an empty rc counts nothing.
+__device__ __forceinline__ uint32_t count_pairs(const FrameDev &f, const DevCam &cam, int64_t v, const short4 &rc) {
+    const int lane = threadIdx.x & 31;
     const uint8_t *mask = f.tile_mask + cam.tile_base;
-    for (int ty = rc.z; ty <= rc.w; ++ty) {
-        for (int tx = rc.x; tx <= rc.y; ++tx) {
-            const uint32_t c = __popc(mask[ty * cam.ntx + tx]);
-            if (c)
-                atomicAdd(f.tile_cnt + (size_t)(v & (kTileSub - 1)) * f.total_tiles + cam.tile_base + ty * cam.ntx + tx,
-                          c);
-            cnt += c;
+    uint32_t *cnt = f.tile_cnt + cam.tile_base;
+    const int sub = (int)(v & (kTileSub - 1));
+    const bool coop = rect_tiles(rc) > kCoopTiles;
+    uint32_t n = 0;
+    if (!coop) {
+        for (int ty = rc.z; ty <= rc.w; ++ty) {
+            for (int tx = rc.x; tx <= rc.y; ++tx) {
+                const int tile = ty * cam.ntx + tx;
+                const uint32_t c = __popc(mask[tile]);
+                if (c) atomicAdd(cnt + (size_t)sub * f.total_tiles + tile, c);
+                n += c;
+            }
         }
     }
-    f.rect[iv] = rc;
-    f.count[iv] = cnt;
-    return cnt;
+    for (unsigned todo = __ballot_sync(0xffffffffu, coop); todo; todo &= todo - 1u) {
+        const int src = __ffs(todo) - 1;
+        const short4 q = shfl_rect(rc, src);
+        const int w = q.y - q.x + 1, area = rect_tiles(q);
+        uint32_t *to = cnt + (size_t)__shfl_sync(0xffffffffu, sub, src) * f.total_tiles;
+        uint32_t all = 0;
+        for (int i = lane; i < area; i += 32) {
+            const int tile = (q.z + i / w) * cam.ntx + q.x + i % w;
+            const uint32_t c = __popc(mask[tile]);
+            if (c) atomicAdd(to + tile, c);
+            all += c;
+        }
+        all = __reduce_add_sync(0xffffffffu, all);
+        if (lane == src) n = all;
+    }
+    return n;
 }
 
 // Colour of the voxel in one view (Eq. vox_color): degree-3 SH at the
@@ -226,31 +343,41 @@ __device__ __forceinline__ void write_octpath(const FrameDev &f, int64_t v, int 
     f.octpath[v] = ((spread3(ijk[0]) << 2) | (spread3(ijk[1]) << 1) | spread3(ijk[2])) << (3 * (kMaxLevel - l));
 }
 
-// One view (grid.y = view): one thread per (view, voxel).
+// One view (grid.y = view): one thread per (view, voxel).  No thread leaves
+// before the pair count, which the warp takes together.
 __global__ void __launch_bounds__(128, 8) k_preprocess(FrameDev f) {
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= f.n_vox) return;
+    const bool in = v < f.n_vox;
     const int view = blockIdx.y;
     const DevCam &cam = f.views[view];
     const int64_t iv = (int64_t)view * f.n_vox + v;
-    const float c0 = f.centre[3 * v + 0], c1 = f.centre[3 * v + 1], c2 = f.centre[3 * v + 2];
-    const int l = f.level[v];
-    float vs;
-    int ijk[3];
-    int4 i0, i1;
-    if (!voxel_valid(f, v, c0, c1, c2, l, vs, ijk, i0, i1)) {
-        if (view == 0) mark_invalid(f.status, v);
-        f.count[iv] = 0;
-        f.rect[iv] = make_short4(0, -1, 0, -1);
-        return;
+    const short4 none = make_short4(0, -1, 0, -1);
+    float c0 = 0.f, c1 = 0.f, c2 = 0.f, vs = 0.f;
+    int4 i0 = make_int4(0, 0, 0, 0), i1 = i0;
+    short4 rc = none;
+    ushort4 box = make_ushort4(0, 0, 0, 0);
+    if (in) {
+        c0 = f.centre[3 * v + 0];
+        c1 = f.centre[3 * v + 1];
+        c2 = f.centre[3 * v + 2];
+        const int l = f.level[v];
+        int ijk[3];
+        if (voxel_valid(f, v, c0, c1, c2, l, vs, ijk, i0, i1)) {
+            if (view == 0) write_octpath(f, v, l, ijk);
+            rc = project_voxel(cam, c0, c1, c2, 0.5f * vs, box);
+        } else if (view == 0) {
+            mark_invalid(f.status, v);
+        }
     }
-    if (view == 0) write_octpath(f, v, l, ijk);
-    const float h = 0.5f * vs;
-    ushort4 box;
-    if (project_voxel(f, cam, v, iv, c0, c1, c2, h, box) == 0) return;
+    const uint32_t cnt = count_pairs(f, cam, v, rc);
+    if (!in) return;
+    f.rect[iv] = rc;
+    f.count[iv] = cnt;
+    if (cnt == 0) return;
     f.box[iv] = box;
+    const float h = 0.5f * vs;
     // record of this view: min corner relative to the ray origin, size,
-    // gathered raw densities, colour
+    // density polynomial, colour
     Record r;
     r.r0 = make_float4((c0 - h) - cam.ro[0], (c1 - h) - cam.ro[1], (c2 - h) - cam.ro[2], vs);
     gather_density(f, i0, i1, r.r1, r.r2);
@@ -268,39 +395,43 @@ __global__ void __launch_bounds__(128, 8) k_preprocess(FrameDev f) {
 // rest of its record.
 __global__ void __launch_bounds__(128) k_preprocess_views(FrameDev f) {
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= f.n_vox) return;
-    const float c0 = f.centre[3 * v + 0], c1 = f.centre[3 * v + 1], c2 = f.centre[3 * v + 2];
-    const int l = f.level[v];
-    float vs;
-    int ijk[3];
-    int4 i0, i1;
-    if (!voxel_valid(f, v, c0, c1, c2, l, vs, ijk, i0, i1)) {
-        mark_invalid(f.status, v);
-        for (int view = 0; view < f.n_views; ++view) {
-            const int64_t iv = (int64_t)view * f.n_vox + v;
-            f.count[iv] = 0;
-            f.rect[iv] = make_short4(0, -1, 0, -1);
-        }
-        return;
-    }
-    write_octpath(f, v, l, ijk);
-    {
-        float sh[48];
-        load_sh(f, v, sh);
-        for (int view = 0; view < f.n_views; ++view) {
-            float Y[16];
-            view_basis(f.views[view], c0, c1, c2, Y);
-            f.rec[(int64_t)view * f.n_vox + v].r3 = voxel_colour(Y, sh);
-        }
-    }
+    const bool in = v < f.n_vox;
+    float c0 = 0.f, c1 = 0.f, c2 = 0.f, vs = 0.f;
+    int4 i0 = make_int4(0, 0, 0, 0), i1 = i0;
+    bool ok = false;
     float4 g0, g1;
-    gather_density(f, i0, i1, g0, g1);
+    if (in) {
+        c0 = f.centre[3 * v + 0];
+        c1 = f.centre[3 * v + 1];
+        c2 = f.centre[3 * v + 2];
+        const int l = f.level[v];
+        int ijk[3];
+        ok = voxel_valid(f, v, c0, c1, c2, l, vs, ijk, i0, i1);
+        if (!ok) {
+            mark_invalid(f.status, v);
+        } else {
+            write_octpath(f, v, l, ijk);
+            float sh[48];
+            load_sh(f, v, sh);
+            for (int view = 0; view < f.n_views; ++view) {
+                float Y[16];
+                view_basis(f.views[view], c0, c1, c2, Y);
+                f.rec[(int64_t)view * f.n_vox + v].r3 = voxel_colour(Y, sh);
+            }
+            gather_density(f, i0, i1, g0, g1);
+        }
+    }
     const float h = 0.5f * vs;
     for (int view = 0; view < f.n_views; ++view) {
         const DevCam &cam = f.views[view];
         const int64_t iv = (int64_t)view * f.n_vox + v;
-        ushort4 box;
-        if (project_voxel(f, cam, v, iv, c0, c1, c2, h, box) == 0) continue;
+        ushort4 box = make_ushort4(0, 0, 0, 0);
+        const short4 rc = ok ? project_voxel(cam, c0, c1, c2, h, box) : make_short4(0, -1, 0, -1);
+        const uint32_t cnt = count_pairs(f, cam, v, rc);
+        if (!in) continue;
+        f.rect[iv] = rc;
+        f.count[iv] = cnt;
+        if (cnt == 0) continue;
         f.box[iv] = box;
         Record *r = f.rec + iv;
         r->r0 = make_float4((c0 - h) - cam.ro[0], (c1 - h) - cam.ro[1], (c2 - h) - cam.ro[2], vs);
@@ -439,29 +570,50 @@ __global__ void __launch_bounds__(256) k_scan_down(FrameDev f, int nb) {
 // --------------------------------------------------------------------- emit
 
 constexpr int kEmitBatch = 8;
+constexpr int kEmitCoop = 4;   // tiles per lane of a cooperative batch
 constexpr int kEmitThreads = 256;
 
-// grid.y = view
+// Writes the pairs of voxel v in tile g, whose sign patterns are m, from slot o.
+__device__ __forceinline__ void write_pairs(const FrameDev &f, int g, unsigned m, uint32_t o, uint64_t code,
+                                            uint32_t v) {
+    if ((int64_t)o + __popc(m) > f.capacity) {  // counts and emission disagree: never expected
+        atomicOr(&f.status->flags, SVR_FLAG_CAPACITY);
+        return;
+    }
+    while (m) {
+        const unsigned s = __ffs(m) - 1;
+        m &= m - 1;
+        if (f.vid_bits > 0) {
+            f.keys[0][o] = pair_word(f, code, s, v);
+        } else {
+            f.keys[0][o] = ((uint64_t)g << f.key_shift) | ((code ^ ((uint64_t)s * kTripleOnes)) >> (48 - f.key_shift));
+            f.vals[0][o] = (s << 29) | v;
+        }
+        ++o;
+    }
+}
+
+// grid.y = view.  A voxel over more than kCoopTiles tiles is left to the warp.
 __global__ void __launch_bounds__(kEmitThreads) k_emit(FrameDev f) {
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= f.n_vox) return;
-    if (f.status->flags & SVR_FLAG_CAPACITY) return;
-    const int view = blockIdx.y;
+    if (f.status->flags & SVR_FLAG_CAPACITY) return;   // not raised here while the pairs fit
+    const int view = blockIdx.y, lane = threadIdx.x & 31;
     const DevCam &cam = f.views[view];
     const int64_t iv = (int64_t)view * f.n_vox + v;
-    if (f.count[iv] == 0) return;
-    const short4 rc = f.rect[iv];
-    const uint64_t code = f.octpath[v];
-    const int drop = 48 - f.key_shift;
-    const bool words = f.vid_bits > 0;
-    uint64_t *keys = f.keys[0];
-    uint32_t *vals = f.vals[0];
-    uint32_t *cur = f.cursor + (size_t)(v & (kTileSub - 1)) * f.total_tiles;
+    short4 rc = make_short4(0, -1, 0, -1);
+    uint64_t code = 0;
+    if (v < f.n_vox && f.count[iv] != 0) {
+        rc = f.rect[iv];
+        code = f.octpath[v];
+    }
+    const int sub = (int)(v & (kTileSub - 1));
+    uint32_t *cur = f.cursor + (size_t)sub * f.total_tiles;
+    const bool coop = rect_tiles(rc) > kCoopTiles;
     // the rectangle's tiles in row-major batches of kEmitBatch: a batch's
-    // cursor atomics are issued together, so a voxel over many tiles waits
+    // cursor atomics are issued together, so a voxel over several tiles waits
     // for one atomic round trip per batch rather than per tile
     int tx = rc.x, ty = rc.z;
-    while (ty <= rc.w) {
+    while (!coop && ty <= rc.w) {
         int gb[kEmitBatch];
         unsigned mb[kEmitBatch];
 #pragma unroll
@@ -478,24 +630,30 @@ __global__ void __launch_bounds__(kEmitThreads) k_emit(FrameDev f) {
 #pragma unroll
         for (int i = 0; i < kEmitBatch; ++i) ob[i] = mb[i] ? atomicAdd(cur + gb[i], (uint32_t)__popc(mb[i])) : 0u;
 #pragma unroll
-        for (int i = 0; i < kEmitBatch; ++i) {
-            unsigned m = mb[i];
-            uint32_t o = ob[i];
-            if ((int64_t)o + __popc(m) > f.capacity) {  // counts and emission disagree: never expected
-                atomicOr(&f.status->flags, SVR_FLAG_CAPACITY);
-                return;
+        for (int i = 0; i < kEmitBatch; ++i) write_pairs(f, gb[i], mb[i], ob[i], code, (uint32_t)v);
+    }
+    for (unsigned todo = __ballot_sync(0xffffffffu, coop); todo; todo &= todo - 1u) {
+        const int src = __ffs(todo) - 1;
+        const short4 q = shfl_rect(rc, src);
+        const int w = q.y - q.x + 1, area = rect_tiles(q);
+        const uint64_t qcode = __shfl_sync(0xffffffffu, code, src);
+        const uint32_t qv = __shfl_sync(0xffffffffu, (uint32_t)v, src);
+        uint32_t *to = f.cursor + (size_t)__shfl_sync(0xffffffffu, sub, src) * f.total_tiles;
+        for (int i0 = lane; i0 < area; i0 += 32 * kEmitCoop) {
+            int gb[kEmitCoop];
+            unsigned mb[kEmitCoop];
+            uint32_t ob[kEmitCoop];
+#pragma unroll
+            for (int j = 0; j < kEmitCoop; ++j) {
+                const int i = i0 + 32 * j;
+                gb[j] = cam.tile_base + (q.z + i / w) * cam.ntx + q.x + i % w;
+                mb[j] = i < area && SVR_IN_BOUNDS(f.debug, kDbgTile, gb[j], f.total_tiles) ? (unsigned)f.tile_mask[gb[j]]
+                                                                                         : 0u;
             }
-            while (m) {
-                const unsigned s = __ffs(m) - 1;
-                m &= m - 1;
-                if (words) {
-                    keys[o] = pair_word(f, code, s, (uint32_t)v);
-                } else {
-                    keys[o] = ((uint64_t)gb[i] << f.key_shift) | ((code ^ ((uint64_t)s * kTripleOnes)) >> drop);
-                    vals[o] = (s << 29) | (uint32_t)v;
-                }
-                ++o;
-            }
+#pragma unroll
+            for (int j = 0; j < kEmitCoop; ++j) ob[j] = mb[j] ? atomicAdd(to + gb[j], (uint32_t)__popc(mb[j])) : 0u;
+#pragma unroll
+            for (int j = 0; j < kEmitCoop; ++j) write_pairs(f, gb[j], mb[j], ob[j], qcode, qv);
         }
     }
 }
@@ -503,7 +661,8 @@ __global__ void __launch_bounds__(kEmitThreads) k_emit(FrameDev f) {
 // ---------------------------------------------------------------- launchers
 
 cudaError_t launch_tile_mask(const FrameDev &f, cudaStream_t s) {
-    k_tile_mask<<<(unsigned)((f.total_tiles + kMaskWarps - 1) / kMaskWarps), 32 * kMaskWarps, 0, s>>>(f);
+    const int warps = tmin(f.total_tiles, kMaskWarps), per = kMaskThreads / 32;
+    k_tile_mask<<<(unsigned)((warps + per - 1) / per), kMaskThreads, 0, s>>>(f);
     return cudaGetLastError();
 }
 

@@ -1386,29 +1386,74 @@ __device__ __forceinline__ void add_sum(const Entry &e, const float4 &g0, const 
 }
 
 // Sums the run's n records and adds the sums to the voxels' accumulators.
-__device__ __forceinline__ void rec_flush(const RecSmem &rs, const Entry *st, int n, float4 *__restrict__ acc_grid,
+__device__ __forceinline__ void rec_flush(RecSmem &rs, const Entry *st, int n, float4 *__restrict__ acc_grid,
                                           float4 *__restrict__ acc_col) {
     __syncwarp();
-    const int r0 = (threadIdx.x & 31) * kRecLane;
+    const int lane = threadIdx.x & 31, r0 = lane * kRecLane;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    // the lane's last stretch (k), and its first one (kf) if it has several
+    int k = -1, kf = -1;
+    float4 g0 = zero, g1 = zero, c = zero, f0 = zero, f1 = zero, fc = zero;
     if (r0 < n) {
-        int k = rs.ent[r0];
+        k = rs.ent[r0];
         const float4 *r = rs.rec + rec_at(r0);
-        float4 g0 = r[0], g1 = r[1], c = r[2];
+        g0 = r[0];
+        g1 = r[1];
+        c = r[2];
 #pragma unroll
         for (int i = 1; i < kRecLane; ++i) {
             if (r0 + i >= n) break;
             const int k2 = rs.ent[r0 + i];
             if (k2 != k) {
-                add_sum(st[k], g0, g1, c, acc_grid, acc_col);
-                g0 = g1 = c = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (kf < 0) {
+                    kf = k;
+                    f0 = g0;
+                    f1 = g1;
+                    fc = c;
+                } else {
+                    add_sum(st[k], g0, g1, c, acc_grid, acc_col);
+                }
+                g0 = g1 = c = zero;
                 k = k2;
             }
             add4(g0, r[3 * i]);
             add4(g1, r[3 * i + 1]);
             add4(c, r[3 * i + 2]);
         }
-        add_sum(st[k], g0, g1, c, acc_grid, acc_col);
     }
+    __syncwarp();
+    // an entry over several lanes is summed by the first of them: a lane
+    // publishes its first stretch, or its only one, if it continues the lane
+    // before (three shared stores; the records have been read)
+    const int k_up = __shfl_up_sync(0xffffffffu, k, 1);
+    const bool joins = lane > 0 && kf >= 0 && kf == k_up;             // first of several stretches
+    const bool whole = lane > 0 && kf < 0 && k >= 0 && k == k_up;     // the only one
+    const unsigned wm = __ballot_sync(0xffffffffu, whole), jm = __ballot_sync(0xffffffffu, joins);
+    if (kf >= 0 && !joins) add_sum(st[kf], f0, f1, fc, acc_grid, acc_col);
+    if (wm | jm) {
+        float4 *pub = rs.rec + 3 * lane;
+        if (joins) {
+            pub[0] = f0;
+            pub[1] = f1;
+            pub[2] = fc;
+        } else if (whole) {
+            pub[0] = g0;
+            pub[1] = g1;
+            pub[2] = c;
+        }
+        __syncwarp();
+        if (!whole) {
+            const unsigned w = lane < 31 ? wm >> (lane + 1) : 0u, j = lane < 31 ? jm >> (lane + 1) : 0u;
+            int m = __ffs(~w) - 1;       // lanes after this one that it holds whole
+            m += (int)((j >> m) & 1u);   // and one that starts with the rest
+            for (int i = 1; i <= m; ++i) {
+                add4(g0, pub[3 * i]);
+                add4(g1, pub[3 * i + 1]);
+                add4(c, pub[3 * i + 2]);
+            }
+        }
+    }
+    if (k >= 0 && !whole) add_sum(st[k], g0, g1, c, acc_grid, acc_col);
     __syncwarp();
 }
 

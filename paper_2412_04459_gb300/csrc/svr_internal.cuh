@@ -351,7 +351,9 @@ __device__ __forceinline__ void word_pair(const FrameDev &f, int g, uint64_t wor
 // View that owns global tile g.
 __device__ __forceinline__ int view_of_tile(const FrameDev &f, int g) {
     int v = 0;
-    while (v + 1 < f.n_views && g >= f.views[v + 1].tile_base) ++v;
+#pragma unroll
+    for (int step = kMaxViews / 2; step > 0; step /= 2)
+        if (v + step < f.n_views && g >= f.views[v + step].tile_base) v += step;
     return v;
 }
 
