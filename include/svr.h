@@ -449,6 +449,14 @@ SVR_API int svr_adam(float *param, const float *grad, float *m, float *v, int64_
 SVR_API int svr_frame_status(const svr_frame *frame, uint32_t *flags, int64_t *n_pairs,
                              void *stream);
 
+/* svr_frame_status without the wait: enqueues a copy of the frame's status
+ * block, uint32[16] = flags, pair count (low, high), ..., into host_status,
+ * 64 bytes of page-locked host memory that stay valid until the copy is done
+ * (the caller waits for the stream or for an event recorded after this call).
+ * So a caller can enqueue the render before it learns the pair count.  After
+ * an overflow the tiles are empty and the render writes the background. */
+SVR_API int svr_frame_status_async(const svr_frame *frame, uint32_t *host_status, void *stream);
+
 /* Device pointers of a frame's internal buffers (valid while the frame is). */
 SVR_API int svr_frame_buffers(const svr_frame *frame, svr_buffers *out);
 

@@ -102,6 +102,7 @@ SIGNATURES = {
     "svr_adam": (ctypes.c_int, [_P, _P, _P, _P, ctypes.c_int64, ctypes.c_int32, ctypes.c_int32, ctypes.c_float,
                                 ctypes.c_float, ctypes.c_float, ctypes.c_float, ctypes.c_float, ctypes.c_int64, _P]),
     "svr_frame_status": (ctypes.c_int, [_P, _P, _P, _P]),
+    "svr_frame_status_async": (ctypes.c_int, [_P, _P, _P]),
     "svr_frame_buffers": (ctypes.c_int, [_P, _P]),
     "svr_last_error": (ctypes.c_char_p, []),
     "svr_version": (ctypes.c_int, []),

@@ -413,6 +413,17 @@ SVR_API int svr_frame_status(const svr_frame *frame, uint32_t *flags, int64_t *n
     return SVR_OK;
 }
 
+SVR_API int svr_frame_status_async(const svr_frame *frame, uint32_t *host_status, void *stream) {
+    g_err[0] = 0;
+    if (!frame || frame->stage < 1) return fail(SVR_ERR_INVALID, "frame not preprocessed");
+    if (!host_status) return fail(SVR_ERR_INVALID, "null host_status");
+    const void *st = (const char *)frame->ws + frame->offsets[kStatus];
+    const cudaError_t e =
+        cudaMemcpyAsync(host_status, st, sizeof(svr::Status), cudaMemcpyDeviceToHost, (cudaStream_t)stream);
+    if (e != cudaSuccess) return cuda_fail(e, "status read");
+    return SVR_OK;
+}
+
 SVR_API int svr_bin_sort(svr_frame *frame, int64_t *n_pairs_out, void *stream) {
     g_err[0] = 0;
     if (!frame || frame->stage < 1) return fail(SVR_ERR_INVALID, "frame not preprocessed");

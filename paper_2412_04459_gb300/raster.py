@@ -17,6 +17,7 @@ from __future__ import annotations
 
 import ctypes
 import dataclasses
+import threading
 from typing import Optional
 
 import numpy as np
@@ -38,9 +39,7 @@ def camera_struct(cam) -> N.SvrCamera:
     """svr_camera from any object with fx, fy, cx, cy, w2c [3, 4], width, height."""
     c = N.SvrCamera()
     c.fx, c.fy, c.cx, c.cy = (float(np.float32(v)) for v in (cam.fx, cam.fy, cam.cx, cam.cy))
-    w2c = np.asarray(cam.w2c, np.float32).reshape(-1)
-    for i in range(12):
-        c.w2c[i] = float(w2c[i])
+    c.w2c[:] = np.asarray(cam.w2c, np.float32).reshape(-1)[:12].tolist()
     c.width, c.height = int(cam.width), int(cam.height)
     return c
 
@@ -116,6 +115,25 @@ def workspace_size(n_vox: int, pair_capacity: int, cams, K=1, t_stop=1e-4, tile=
     return int(n)
 
 
+class _StatusRead(threading.local):
+    """Per thread and device: 64 bytes of page-locked memory and an event, for
+    reading a frame's status while the render runs.  Used within one call
+    (copy, event, wait), so calls on any streams of a thread can share it."""
+
+    def __init__(self):
+        self.slots = {}
+
+    def get(self, device: torch.device):
+        slot = self.slots.get(device.index)
+        if slot is None:
+            slot = (torch.empty(16, dtype=torch.int32, pin_memory=True), torch.cuda.Event())
+            self.slots[device.index] = slot
+        return slot
+
+
+_status_read = _StatusRead()
+
+
 class Frame:
     """One view (cams = a camera) or a batch of views (cams = a list) of a
     scene: the workspace, the svr_frame and the outputs.  Outputs of a batch
@@ -145,9 +163,14 @@ class Frame:
 
     # -- workspace -----------------------------------------------------------
     def ws_bytes(self) -> int:
-        return workspace_size(self.scene.n_vox, self.pair_capacity, self.cams if self.batched else self.cam,
-                              self.pstruct.K, self.pstruct.t_stop, self.pstruct.tile, tuple(self.pstruct.bg),
-                              batched=self.batched)
+        n_vox, cap, p = self.scene.n_vox, self.pair_capacity, N.ref(self.pstruct)
+        if self.batched:
+            n = N.lib().svr_workspace_size_views(n_vox, cap, self.cstructs, len(self.cams), p)
+        else:
+            n = N.lib().svr_workspace_size(n_vox, cap, self.cstructs, p)
+        if n == 0:
+            raise N.SvrError(N.SVR_ERR_INVALID, "workspace size", "invalid arguments")
+        return int(n)
 
     def _alloc(self):
         nbytes = self.ws_bytes()
@@ -259,9 +282,30 @@ class Frame:
         return out
 
     def render(self, grid=None, sh=None, sync: bool = True, stream=None):
-        self.preprocess(grid, sh, stream)
-        self.bin_sort(sync=sync, stream=stream)
-        return self.forward(stream=stream)
+        """preprocess, bin_sort, forward.  sync=True reads the pair count back
+        (and redoes the view with a larger workspace if it did not fit); the
+        forward is enqueued before the host waits for the count, so the GPU
+        does not wait for the host (it used to stand still for about 50 us)."""
+        if not sync:
+            self.preprocess(grid, sh, stream)
+            self.bin_sort(sync=False, stream=stream)
+            return self.forward(stream=stream)
+        s = stream if stream is not None else torch.cuda.current_stream()
+        out = self.new_outputs()
+        self.preprocess(grid, sh, s)
+        self.bin_sort(sync=False, stream=s)
+        host, event = _status_read.get(self.scene.centre.device)
+        N.check(N.lib().svr_frame_status_async(N.ref(self.frame), _ptr(host), _stream(s)), "svr_frame_status_async")
+        event.record(s)
+        self.forward(out, stream=s)
+        event.synchronize()
+        flags, lo, hi = host[:3].tolist()
+        if flags:   # an invalid voxel (raises) or too many pairs (grows the workspace)
+            self.bin_sort(sync=True, stream=s)
+            return self.forward(out, stream=s)
+        self.n_pairs = (hi & 0xFFFFFFFF) << 32 | lo & 0xFFFFFFFF
+        self.frame.n_pairs = self.n_pairs
+        return out
 
     def backward(self, g_rgb, g_depth, g_alpha, out, d_grid=None, d_sh=None, stream=None):
         dev = self.scene.centre.device
@@ -435,13 +479,15 @@ class SVRasterFn(torch.autograd.Function):
         frame = Frame(scene, cam, K=K, t_stop=t_stop, bg=bg, pair_capacity=pair_capacity)
         out = frame.render(grid.detach().contiguous(), sh.detach().contiguous())
         ctx.frame = frame
-        ctx.out = out
+        # what the backward reads; not the returned images, whose graph node
+        # holds ctx (a cycle that would keep every call's workspace alive)
+        ctx.saved = {"T_final": out["T_final"], "last": out["last"]}
         return out["rgb"], out["depth"], out["alpha"]
 
     @staticmethod
     def backward(ctx, g_rgb, g_depth, g_alpha):
         frame = ctx.frame
-        d_grid, d_sh = frame.backward(g_rgb, g_depth, g_alpha, ctx.out)
+        d_grid, d_sh = frame.backward(g_rgb, g_depth, g_alpha, ctx.saved)
         return d_grid, d_sh, None, None, None, None, None, None
 
 
