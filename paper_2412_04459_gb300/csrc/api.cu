@@ -79,7 +79,7 @@ Layout make_layout(int64_t n_vox, int n_views, int64_t cap, int64_t ntiles, int 
     take(kTileOrder, 8 * ((size_t)ntiles + slots));
     const size_t B = (size_t)tile * tile / 32;
     take(kBlockList, 8 * B * C);
-    take(kBlockLen, 4 * B * (size_t)ntiles);
+    take(kBlockLen, sizeof(svr::RenderItem) * B * ((size_t)ntiles + slots));   // render items
     take(kHitMask, 4 * B * (C + 32 * (size_t)ntiles));   // the block lists' positions + 32 per (tile, block)
     take(kSegment, seg_bytes(ntiles, slots, B).total);
     take(kSortPlan, align256(sizeof(svr::SortPlan)) + 8 * (size_t)svr::sort_chunk_capacity(cap));
@@ -215,7 +215,7 @@ svr::FrameDev frame_dev(const svr_frame *f) {
     d.ranges = (uint2 *)(ws + o[kRanges]);
     d.order = (uint2 *)(ws + o[kTileOrder]);
     d.blist = (uint2 *)(ws + o[kBlockList]);
-    d.blen = (uint32_t *)(ws + o[kBlockLen]);
+    d.items = (svr::RenderItem *)(ws + o[kBlockLen]);
     d.hmask = (uint32_t *)(ws + o[kHitMask]);
     d.blocks_per_tile = f->params.tile * f->params.tile / 32;
     d.seg_slots = svr::seg_slot_capacity(f->pair_capacity);

@@ -3,8 +3,8 @@
 // Work is split into items of (tile, list segment, 8x4 pixel block): 8
 // blocks per 16x16 tile, and one segment per tile unless its list is longer
 // than kSegLen entries.  A persistent grid of warps pulls items from a device
-// counter in the order of k_tile_order (longest segments first, so the heavy
-// work does not form the tail).  A warp walks the part of its block's list
+// counter in the order of k_order (longest segments first, so the heavy work
+// does not form the tail).  A warp walks the part of its block's list
 // (the tile's entries whose pixel box meets the block, k_block_lists) that its
 // segment covers, 32 entries per batch, with no CTA-wide barrier: lane j
 // reads entry j of the batch (its value, then the voxel's conservative pixel
@@ -144,15 +144,19 @@ __device__ __forceinline__ uint32_t vid_of(const ViewData &vd, uint32_t val) {
     return checked(vd.dbg, kDbgVoxel, val & 0x1FFFFFFFu, vd.n);
 }
 
+// Pixel origin of block blk of a tile.
+__device__ __forceinline__ void block_origin(const DevCam &cam, int tile, int blk, int &x0, int &y0) {
+    const int tx = tile % cam.ntx, ty = tile / cam.ntx, bpr = cam.tile >> 3;
+    x0 = tx * cam.tile + (blk % bpr) * 8;
+    y0 = ty * cam.tile + (blk / bpr) * 4;
+}
+
 // Pixel of the calling lane in block blk of a tile (tile edge 8, 16 or 32:
 // tile / 8 blocks of 8x4 pixels per block row).
 __device__ __forceinline__ PixelRay pixel_ray(const DevCam &cam, int tile, int blk, WarpBlock &wb) {
     PixelRay p;
-    const int tx = tile % cam.ntx, ty = tile / cam.ntx;
     const int lane = threadIdx.x & 31;
-    const int bpr = cam.tile >> 3;
-    wb.x0 = tx * cam.tile + (blk % bpr) * 8;
-    wb.y0 = ty * cam.tile + (blk / bpr) * 4;
+    block_origin(cam, tile, blk, wb.x0, wb.y0);
     p.x = wb.x0 + (lane & 7);
     p.y = wb.y0 + (lane >> 3);
     p.inside = p.x < cam.W && p.y < cam.H;
@@ -162,11 +166,14 @@ __device__ __forceinline__ PixelRay pixel_ray(const DevCam &cam, int tile, int b
     p.inv = make_float3(1.0f / (p.rd.x + 0.0f), 1.0f / (p.rd.y + 0.0f), 1.0f / (p.rd.z + 0.0f));
     p.rdn = sqrtf(p.rd.x * p.rd.x + p.rd.y * p.rd.y + p.rd.z * p.rd.z);
     wb.smask = __reduce_or_sync(0xffffffffu, p.inside ? (1u << p.s) : 0u);
-    wb.spix = 0;
+    const unsigned in = __ballot_sync(0xffffffffu, p.inside);
+    wb.spix = (wb.smask >> (lane & 7)) & 1u ? in : 0u;
+    if (wb.smask & (wb.smask - 1u)) {   // several patterns: rare
 #pragma unroll
-    for (int t = 0; t < 8; ++t) {
-        const unsigned m = __ballot_sync(0xffffffffu, p.inside && p.s == t);
-        if (lane == t) wb.spix = m;
+        for (int t = 0; t < 8; ++t) {
+            const unsigned m = __ballot_sync(0xffffffffu, p.inside && p.s == t);
+            if (lane == t) wb.spix = m;
+        }
     }
     return p;
 }
@@ -222,8 +229,9 @@ __device__ __forceinline__ bool slab(const Entry &e, const PixelRay &p, float &a
 // owns the region B beg + b (end - beg) of the block lists, so the lists need
 // no allocation scan; segment s of a split tile writes from offset s kSegLen
 // of that region (it keeps at most kSegLen entries) and records its count per
-// block.  The CTA of segment 0 also clears the tile's merge counters for the
-// next forward.  The CTAs form a persistent grid that strides over the
+// block.  Then the CTA writes the render items of its blocks, in the work
+// order's place.  The CTA of segment 0 also clears the tile's merge counters
+// for the next forward.  The CTAs form a persistent grid that strides over the
 // entries.
 
 constexpr int kListThreads = 128;
@@ -232,7 +240,7 @@ constexpr int kMaxBlocksPerWarp = 32 / kListWarps;  // tile 32: 32 blocks over t
 constexpr int kListChunk = kSegLen;
 
 __device__ __forceinline__ void block_lists_entry(const FrameDev &f, const uint32_t *__restrict__ vals, unsigned e,
-                                                  uint32_t *sval, uint32_t *smsk) {
+                                                  uint32_t *sval, uint32_t *smsk, uint32_t *scnt) {
     const uint2 gs = f.order[e];
     const int g = (int)gs.x, sg = (int)gs.y;
     const int view = view_of_tile(f, g);
@@ -312,10 +320,19 @@ __device__ __forceinline__ void block_lists_entry(const FrameDev &f, const uint3
         __syncthreads();
     }
     if (lane == 0) {
-        uint32_t *len = split ? f.seg_len + (size_t)(ts.y + sg) * B : f.blen + (size_t)g * B;
 #pragma unroll
         for (int k = 0; k < kMaxBlocksPerWarp; ++k)
-            if (warp + kListWarps * k < B) len[warp + kListWarps * k] = cnt[k];
+            if (warp + kListWarps * k < B) scnt[warp + kListWarps * k] = cnt[k];
+    }
+    __syncthreads();
+    if (warp == 0) {
+        const unsigned n = lane < B ? scnt[lane] : 0u;
+        if (split && lane < B) f.seg_len[(size_t)(ts.y + sg) * B + lane] = n;
+        if (lane < B) {
+            uint4 *it = reinterpret_cast<uint4 *>(f.items + (size_t)e * B + lane);
+            it[0] = make_uint4((unsigned)g, (unsigned)lane | ((unsigned)sg << 8), n, rg.x);
+            it[1] = make_uint4(rg.y, split ? ts.y + (unsigned)sg : kNoSlot, 0u, 0u);
+        }
     }
 }
 
@@ -324,9 +341,10 @@ __device__ __forceinline__ void block_lists_entry(const FrameDev &f, const uint3
 __global__ void __launch_bounds__(kListThreads) k_block_lists(FrameDev f, const uint32_t *__restrict__ vals) {
     __shared__ uint32_t sval[kListChunk];
     __shared__ uint32_t smsk[kListChunk];
+    __shared__ uint32_t scnt[32];
     const unsigned nq = f.status->n_listed;  // empty lists have no block lists
     for (unsigned e = blockIdx.x; e < nq; e += gridDim.x) {
-        block_lists_entry(f, vals, e, sval, smsk);
+        block_lists_entry(f, vals, e, sval, smsk, scnt);
         __syncthreads();  // shared memory is reused by the next entry
     }
 }
@@ -393,23 +411,48 @@ __device__ __forceinline__ int lower_pos(const uint2 *__restrict__ list, int lo,
     return lo + __popc(__ballot_sync(0xffffffffu, below));
 }
 
-// Work item of a render warp: segment `seg` of global tile g, 8x4 block blk.
+// Work item of a render warp: segment `seg` of global tile g, 8x4 block blk,
+// with its part of the block list.
 struct Item {
     int g, seg, blk;
+    const uint2 *list;   // the n entries
+    uint32_t *hm;        // their hit masks (see FrameDev::hmask)
+    int n;
+    int beg, end;        // the tile's range in the sorted pairs
+    uint32_t slot;       // segment slot, or kNoSlot
+    uint32_t walked;     // entries the forward took
 };
 
-// Next work item of the calling warp, or false when done.
-__device__ __forceinline__ bool next_item(unsigned *counter, unsigned n_items, unsigned blocks_per_tile,
-                                          const uint2 *order, Item &it) {
-    unsigned item = 0;
-    if ((threadIdx.x & 31) == 0) item = atomicAdd(counter, 1u);
-    item = __shfl_sync(0xffffffffu, item, 0);
-    if (item >= n_items) return false;
-    const uint2 q = order[item / blocks_per_tile];
-    it.g = (int)q.x;
-    it.seg = (int)q.y;
-    it.blk = (int)(item % blocks_per_tile);
-    return true;
+// Next work of the calling warp (a number below n), or false when done.
+__device__ __forceinline__ bool next_work(unsigned *counter, unsigned n, unsigned &w) {
+    if ((threadIdx.x & 31) == 0) w = atomicAdd(counter, 1u);
+    w = __shfl_sync(0xffffffffu, w, 0);
+    return w < n;
+}
+
+// Only an item's first walk writes its hit masks (the merge's second walk of a
+// segment and the max-weight pass leave them), so they hold every pixel's hits
+// up to its stopping voxel.
+__device__ __forceinline__ Item load_item(const FrameDev &f, unsigned i) {
+    const uint4 *q = reinterpret_cast<const uint4 *>(f.items + i);
+    const uint4 a = __ldcg(q), b = __ldcg(q + 1);
+    Item it;
+    it.g = (int)a.x;
+    it.blk = (int)(a.y & 0xFFu);
+    it.seg = (int)(a.y >> 8);
+    it.n = (int)a.z;
+    it.beg = (int)a.w;
+    it.end = (int)b.x;
+    it.slot = b.y;
+    it.walked = b.z;
+    if (!SVR_IN_BOUNDS(f.debug, kDbgRange, f.ranges[it.g].y, f.capacity + 1) ||
+        !SVR_IN_BOUNDS(f.debug, kDbgBlockList, it.n, (it.slot == kNoSlot ? it.end - it.beg : kSegLen) + 1))
+        it.n = 0;
+    const size_t B = (size_t)f.blocks_per_tile;
+    const size_t at = B * it.beg + (size_t)it.blk * (it.end - it.beg) + (it.slot == kNoSlot ? 0 : (size_t)it.seg * kSegLen);
+    it.list = f.blist + at;
+    it.hm = f.hmask + at + 32 * ((size_t)it.g * B + it.blk);
+    return it;
 }
 
 // The view of a global tile and its arrays.
@@ -430,31 +473,19 @@ __device__ __forceinline__ ItemView item_view(const FrameDev &f, int g) {
     return iv;
 }
 
-// The block list of an item and the part of it that its segment covers.
+// The block list of a split tile, for the walks over its segments.
 struct ItemList {
-    const uint2 *list;  // the (tile, block) list
-    int n_list;
-    int beg, end;       // the tile's range in the sorted pairs
+    const uint2 *list;  // the (tile, block) list: segment k's part starts at k kSegLen
     uint2 ts;           // segments of the tile, first slot
-    const uint32_t *seg_len; // split tiles: segment k of this block holds seg_len[k * B] entries
+    const uint32_t *seg_len; // segment k of this block holds seg_len[k * B] entries
     DebugBlock *dbg;         // index checks of the SVR_DEBUG build
 };
 
-__device__ __forceinline__ ItemList item_list(const FrameDev &f, int g, int blk) {
+__device__ __forceinline__ ItemList item_list(const FrameDev &f, const Item &it) {
     ItemList L;
-    const uint2 rg = f.ranges[g];
-    const int B = f.blocks_per_tile;
-    L.beg = (int)rg.x;
-    L.end = (int)rg.y;
-    if (!SVR_IN_BOUNDS(f.debug, kDbgRange, rg.y, f.capacity + 1) || !SVR_IN_BOUNDS(f.debug, kDbgRange, rg.x, rg.y + 1))
-        L.beg = L.end = 0;
-    L.list = f.blist + (size_t)B * L.beg + (size_t)blk * (L.end - L.beg);
-    // unsplit tiles (split ones count per segment); an empty tile's block
-    // lengths are not written (k_block_lists skips empty lists)
-    L.n_list = L.end > L.beg ? (int)f.blen[(size_t)g * B + blk] : 0;
-    L.ts = f.tile_seg[g];
-    if (L.ts.x <= 1 && !SVR_IN_BOUNDS(f.debug, kDbgBlockList, L.n_list, L.end - L.beg + 1)) L.n_list = 0;
-    L.seg_len = f.seg_len + (size_t)L.ts.y * B + blk;
+    L.list = it.list - (size_t)it.seg * kSegLen;
+    L.ts = f.tile_seg[it.g];
+    L.seg_len = f.seg_len + (size_t)L.ts.y * f.blocks_per_tile + it.blk;
     L.dbg = f.debug;
     return L;
 }
@@ -465,14 +496,6 @@ __device__ __forceinline__ void seg_range(const ItemList &L, int B, int sg, int 
     p0 = sg * kSegLen;
     p1 = p0 + (int)L.seg_len[(size_t)sg * B];
     if (!SVR_IN_BOUNDS(L.dbg, kDbgBlockList, p1 - p0, kSegLen + 1)) p1 = p0;
-}
-
-// The hit masks of an item's block list (see FrameDev::hmask): word p of the
-// result belongs to block-list position p.  Only an item's first walk
-// writes them (the merge's second walk of a segment and the max-weight pass
-// leave them), so they hold every pixel's hits up to its stopping voxel.
-__device__ __forceinline__ uint32_t *hit_masks(const FrameDev &f, const ItemList &L, const Item &it) {
-    return f.hmask + (L.list - f.blist) + 32 * ((size_t)it.g * f.blocks_per_tile + it.blk);
 }
 
 // Segment sums of (segment slot, block): kSegFields rows of 32 pixels.
@@ -740,8 +763,10 @@ __device__ __forceinline__ void fwd_hits_parallel(const FwdSlot *st, const uint2
 // Walk block-list positions [p0, p1) front to back from state s.  The list
 // entries are fetched two batches ahead and the next batch's records are
 // copied into the other staging buffer while this batch is composited.
+// Returns the position at which every pixel had stopped (p1 or beyond if the
+// walk went to the end).
 template <int K, int MODE>
-__device__ __forceinline__ void fwd_walk(const uint2 *__restrict__ list, int p0, int p1, const ViewData &vd,
+__device__ __forceinline__ int fwd_walk(const uint2 *__restrict__ list, int p0, int p1, const ViewData &vd,
                                          const PixelRay &p, const WarpBlock &wb, FwdSmem &ws, float t_stop,
                                          FwdState &s, const FwdOut &out, bool true_weights, uint32_t *hm) {
     constexpr bool STATS = MODE == kModeStats, FN = MODE == kModeExtra, FD = FN || MODE == kModeDist;
@@ -753,8 +778,8 @@ __device__ __forceinline__ void fwd_walk(const uint2 *__restrict__ list, int p0,
     fetch_box(cur, vd);
     stage_async(ws, 0, vd, cur);
     fetch_vi(nx, list, p0 + kBatch + lane, p0 + kBatch + lane < p1);
-    int buf = 0;
-    for (int base = p0; base < p1; base += kBatch, buf ^= 1) {
+    int buf = 0, base = p0;
+    for (; base < p1; base += kBatch, buf ^= 1) {
         if (__all_sync(0xffffffffu, s.done)) break;
         fetch_box(nx, vd);
         stage_async(ws, buf ^ 1, vd, nx);
@@ -839,6 +864,7 @@ __device__ __forceinline__ void fwd_walk(const uint2 *__restrict__ list, int p0,
     }
     cp_async_wait<0>();  // no copy may land in a buffer after the walk
     __syncwarp();
+    return base;
 }
 
 // Merge the segments of a split tile's block, front to back: segment sg was
@@ -988,13 +1014,13 @@ __device__ __forceinline__ void fwd_merge(const FrameDev &f, const ItemList &L, 
 }
 
 template <int MODE>
-__device__ __forceinline__ void fwd_write(const FrameDev &f, const DevCam &cam, const PixelRay &p,
+__device__ __forceinline__ void fwd_write(const FrameDev &f, const DevCam &cam, int x, int y,
                                           const FwdState &s, int last, const FwdOut &out) {
     constexpr bool STATS = MODE == kModeStats, FN = MODE == kModeExtra, FD = FN || MODE == kModeDist;
-    if (!p.inside) return;
+    if (x >= cam.W || y >= cam.H) return;
     // outputs of view v start at pixel pix_base (rgb: 3 * pix_base, planar)
     const size_t HW = (size_t)cam.W * cam.H;
-    const size_t px = (size_t)p.y * cam.W + p.x;
+    const size_t px = (size_t)y * cam.W + x;
     const size_t o = (size_t)cam.pix_base + px;
     float *rgb = out.rgb + 3 * (size_t)cam.pix_base + px;
     rgb[0] = fmaf(s.T, f.bg[0], s.C0);
@@ -1018,28 +1044,43 @@ __device__ __forceinline__ void fwd_write(const FrameDev &f, const DevCam &cam, 
     }
 }
 
+// Background of a block without entries.
+template <int MODE>
+__device__ __forceinline__ void fwd_blank(const FrameDev &f, int g, int blk, int last, const FwdOut &out) {
+    const DevCam &cam = f.views[view_of_tile(f, g)];
+    int x0, y0;
+    block_origin(cam, g - cam.tile_base, blk, x0, y0);
+    const int lane = threadIdx.x & 31;
+    const FwdState s = {1.f, 0.f, 0.f, 0.f, 0.f, -1, true, 0, 0, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    fwd_write<MODE>(f, cam, x0 + (lane & 7), y0 + (lane >> 3), s, last, out);
+}
+
 template <int K, int MODE>
-__device__ __forceinline__ void fwd_item(const FrameDev &f, const Item &it, FwdSmem &ws, const FwdOut &out) {
+__device__ __forceinline__ void fwd_item(const FrameDev &f, const Item &it, uint32_t *walked, FwdSmem &ws,
+                                         const FwdOut &out) {
     constexpr bool STATS = MODE == kModeStats, FN = MODE == kModeExtra, FD = FN || MODE == kModeDist;
+    const bool split = it.slot != kNoSlot;
+    if (it.n == 0 && !split) {   // no entries: the background
+        fwd_blank<MODE>(f, it.g, it.blk, it.end - 1, out);
+        return;
+    }
     const ItemView iv = item_view(f, it.g);
     const DevCam &cam = f.views[iv.view];
     WarpBlock wb;
     const PixelRay p = pixel_ray(cam, iv.tile, it.blk, wb);
     if (wb.smask == 0) return;  // the whole block lies outside the image
-    const ItemList L = item_list(f, it.g, it.blk);
     const int lane = threadIdx.x & 31;
     FwdState s = {1.f, 0.f, 0.f, 0.f, 0.f, -1, !p.inside, 0, 0, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (L.ts.x <= 1) {
-        fwd_walk<K, MODE>(L.list, 0, L.n_list, iv.vd, p, wb, ws, f.t_stop, s, out, true, hit_masks(f, L, it));
-        fwd_write<MODE>(f, cam, p, s, s.last >= 0 ? s.last : L.end - 1, out);
+    const int took = fwd_walk<K, MODE>(it.list, 0, it.n, iv.vd, p, wb, ws, f.t_stop, s, out, !split || it.seg == 0, it.hm);
+    if (lane == 0) *walked = (uint32_t)min(took, it.n);
+    if (!split) {
+        fwd_write<MODE>(f, cam, p.x, p.y, s, s.last >= 0 ? s.last : it.end - 1, out);
         return;
     }
     // one segment of a split tile, walked from T = 1
+    const ItemList L = item_list(f, it);
     const int B = f.blocks_per_tile;
-    int p0, p1;
-    seg_range(L, B, it.seg, p0, p1);
-    fwd_walk<K, MODE>(L.list, p0, p1, iv.vd, p, wb, ws, f.t_stop, s, out, it.seg == 0, hit_masks(f, L, it));
-    float *q = seg_fields(f, L.ts.y + it.seg, it.blk);
+    float *q = seg_fields(f, it.slot, it.blk);
     q[0] = s.C0;
     q[32] = s.C1;
     q[2 * 32] = s.C2;
@@ -1071,7 +1112,7 @@ __device__ __forceinline__ void fwd_item(const FrameDev &f, const Item &it, FwdS
     __threadfence();
     FwdState m = {1.f, 0.f, 0.f, 0.f, 0.f, -1, !p.inside, 0, 0, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     fwd_merge<K, MODE>(f, L, it.blk, iv.vd, p, wb, ws, m, out);
-    fwd_write<MODE>(f, cam, p, m, m.last >= 0 ? m.last : L.end - 1, out);
+    fwd_write<MODE>(f, cam, p.x, p.y, m, m.last >= 0 ? m.last : it.end - 1, out);
     if (lane == 0) *cnt = 0;  // ready for the next forward of this sort
 }
 
@@ -1085,11 +1126,18 @@ template <int K, int MODE>
 __global__ void __launch_bounds__(kThreads, kFwdMinBlocks) k_render_fwd(FrameDev f, FwdOut out) {
     __shared__ FwdSmem smem[kWarps];
     FwdSmem &ws = smem[threadIdx.x >> 5];
-    const unsigned bpt = (unsigned)f.blocks_per_tile;
-    const unsigned n_items = f.status->n_queue * bpt;
-    Item it;
-    while (next_item(&f.status->fwd_next, n_items, bpt, f.order, it)) {
-        fwd_item<K, MODE>(f, it, ws, out);
+    // the items, then the empty tiles (the last work-order entries), a tile
+    // at a time
+    const unsigned n_listed = f.status->n_listed, n_items = n_listed * (unsigned)f.blocks_per_tile;
+    const unsigned n_work = n_items + f.status->n_queue - n_listed;
+    unsigned w;
+    while (next_work(&f.status->fwd_next, n_work, w)) {
+        if (w < n_items) {
+            fwd_item<K, MODE>(f, load_item(f, w), &f.items[w].walked, ws, out);
+        } else {
+            const int g = (int)f.order[n_listed + (w - n_items)].x;
+            for (int b = 0; b < f.blocks_per_tile; ++b) fwd_blank<MODE>(f, g, b, -1, out);
+        }
         __syncwarp();
     }
     // the launch's last warp to run out of work resets the work counter for
@@ -1116,24 +1164,20 @@ template <int K>
 __global__ void __launch_bounds__(kThreads, kFwdMinBlocks) k_render_maxw(FrameDev f, FwdOut out) {
     __shared__ FwdSmem smem[kWarps];
     FwdSmem &ws = smem[threadIdx.x >> 5];
-    const unsigned bpt = (unsigned)f.blocks_per_tile;
-    const unsigned n_items = f.status->n_listed * bpt;  // split tiles are among the listed
-    Item it;
-    while (next_item(&f.status->maxw_next, n_items, bpt, f.order, it)) {
-        if (it.seg == 0) continue;
+    const unsigned n_items = f.status->n_listed * (unsigned)f.blocks_per_tile;
+    unsigned w;
+    while (next_work(&f.status->maxw_next, n_items, w)) {
+        const Item it = load_item(f, w);
+        if (it.seg == 0 || it.slot == kNoSlot) continue;
         const ItemView iv = item_view(f, it.g);
         const DevCam &cam = f.views[iv.view];
         WarpBlock wb;
         const PixelRay p = pixel_ray(cam, iv.tile, it.blk, wb);
         if (wb.smask == 0) continue;
-        const ItemList L = item_list(f, it.g, it.blk);
-        if (L.ts.x <= 1) continue;
-        const float Tb = __ldcg(seg_fields(f, L.ts.y + it.seg, it.blk) + 5 * 32);
+        const float Tb = __ldcg(seg_fields(f, it.slot, it.blk) + 5 * 32);
         FwdState s = {Tb, 0.f, 0.f, 0.f, 0.f, -1, !p.inside || !(Tb >= f.t_stop), 0, 0,
                       0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        int p0, p1;
-        seg_range(L, f.blocks_per_tile, it.seg, p0, p1);
-        fwd_walk<K, kModeExtra>(L.list, p0, p1, iv.vd, p, wb, ws, f.t_stop, s, out, true, nullptr);
+        fwd_walk<K, kModeExtra>(it.list, 0, it.n, iv.vd, p, wb, ws, f.t_stop, s, out, true, nullptr);
         __syncwarp();
     }
 }
@@ -1141,8 +1185,8 @@ __global__ void __launch_bounds__(kThreads, kFwdMinBlocks) k_render_maxw(FrameDe
 // ----------------------------------------------------------------- backward
 
 struct PixelGrad {
-    float gC0, gC1, gC2, gD, gA;
-    float Tfin;
+    float gC0, gC1, gC2, gD;
+    float gAT;            // dL/dalpha times T_final
     float gN0, gN1, gN2;  // upstream gradient of the normal image (extras)
     float gL;             // upstream gradient of the ray's distortion loss (extras)
     float Wtot, Stot;     // its totals sum w_i = 1 - T_final and sum w_i m_i
@@ -1241,7 +1285,7 @@ __device__ __forceinline__ void hit_grad(const Entry &e, const PixelRay &p, cons
     dcol[2] = w * g.gC2;
     // dL/dx_i through C, A and the transmittance of later voxels in D
     float gx = g.gC0 * fmaf(T_after, e.col.x, -SC0) + g.gC1 * fmaf(T_after, e.col.y, -SC1) +
-               g.gC2 * fmaf(T_after, e.col.z, -SC2) + g.gA * g.Tfin - g.gD * SD;
+               g.gC2 * fmaf(T_after, e.col.z, -SC2) + g.gAT - g.gD * SD;
     if (XN)
         gx += g.gN0 * fmaf(T_after, nrm.x, -SN.x) + g.gN1 * fmaf(T_after, nrm.y, -SN.y) +
               g.gN2 * fmaf(T_after, nrm.z, -SN.z);
@@ -1321,7 +1365,7 @@ struct RecSmem {
     float4 rec[kRecCap * 3 + 32];  // see rec_at
     int off[kBatch];               // first slot of entry j (numbered over the whole batch)
     unsigned pix[kBatch];          // lanes whose pixel hits entry j
-    uint8_t ent[kRecCap];          // staged entry of each slot
+    __align__(4) uint8_t ent[kRecCap];  // staged entry of each slot
 };
 
 // Records are 48 bytes, with 16 free after every kRecLane of them: the lanes'
@@ -1385,75 +1429,68 @@ __device__ __forceinline__ void add_sum(const Entry &e, const float4 &g0, const 
     atomicAdd(acc_col + vid, c);
 }
 
-// Sums the run's n records and adds the sums to the voxels' accumulators.
+// Sums the run's n records and adds the sums to the voxels' accumulators.  An
+// entry over several lanes is summed by the first of them, so that it is added
+// once: a lane whose first stretch continues the lane before puts that
+// stretch's sum in the place of its first record.
 __device__ __forceinline__ void rec_flush(RecSmem &rs, const Entry *st, int n, float4 *__restrict__ acc_grid,
                                           float4 *__restrict__ acc_col) {
+    static_assert(kRecLane == 4, "a lane's entries are read as one word");
     __syncwarp();
-    const int lane = threadIdx.x & 31, r0 = lane * kRecLane;
-    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-    // the lane's last stretch (k), and its first one (kf) if it has several
-    int k = -1, kf = -1;
-    float4 g0 = zero, g1 = zero, c = zero, f0 = zero, f1 = zero, fc = zero;
+    const int lane = threadIdx.x & 31, r0 = lane * kRecLane, cnt = min(kRecLane, n - r0);
+    const unsigned ids = r0 < n ? *reinterpret_cast<const unsigned *>(rs.ent + r0) : 0u;
+    const int k_first = (int)(ids & 0xFFu), k_last = r0 < n ? (int)((ids >> (8 * cnt - 8)) & 0xFFu) : -1;
+    const int k_up = __shfl_up_sync(0xffffffffu, k_last, 1);
+    const bool cont = lane > 0 && r0 < n && k_first == k_up;
+    const bool whole = cont && k_first == k_last;
+    const unsigned wm = __ballot_sync(0xffffffffu, whole), cm = __ballot_sync(0xffffffffu, cont);
+    float4 *r = rs.rec + rec_at(r0);
+    float4 g0 = r[0], g1 = r[1], c = r[2];
     if (r0 < n) {
-        k = rs.ent[r0];
-        const float4 *r = rs.rec + rec_at(r0);
-        g0 = r[0];
-        g1 = r[1];
-        c = r[2];
+        bool pub = cont;   // the stretch at hand belongs to the lane before
+        int k = k_first;
 #pragma unroll
         for (int i = 1; i < kRecLane; ++i) {
-            if (r0 + i >= n) break;
-            const int k2 = rs.ent[r0 + i];
-            if (k2 != k) {
-                if (kf < 0) {
-                    kf = k;
-                    f0 = g0;
-                    f1 = g1;
-                    fc = c;
+            if (i >= cnt) break;
+            const int ki = (int)((ids >> (8 * i)) & 0xFFu);
+            if (ki != k) {
+                if (pub) {
+                    r[0] = g0;
+                    r[1] = g1;
+                    r[2] = c;
+                    pub = false;
                 } else {
                     add_sum(st[k], g0, g1, c, acc_grid, acc_col);
                 }
-                g0 = g1 = c = zero;
-                k = k2;
+                g0 = g1 = c = make_float4(0.f, 0.f, 0.f, 0.f);
+                k = ki;
             }
             add4(g0, r[3 * i]);
             add4(g1, r[3 * i + 1]);
             add4(c, r[3 * i + 2]);
         }
+        if (pub) {
+            r[0] = g0;
+            r[1] = g1;
+            r[2] = c;
+        }
     }
     __syncwarp();
-    // an entry over several lanes is summed by the first of them: a lane
-    // publishes its first stretch, or its only one, if it continues the lane
-    // before (three shared stores; the records have been read)
-    const int k_up = __shfl_up_sync(0xffffffffu, k, 1);
-    const bool joins = lane > 0 && kf >= 0 && kf == k_up;             // first of several stretches
-    const bool whole = lane > 0 && kf < 0 && k >= 0 && k == k_up;     // the only one
-    const unsigned wm = __ballot_sync(0xffffffffu, whole), jm = __ballot_sync(0xffffffffu, joins);
-    if (kf >= 0 && !joins) add_sum(st[kf], f0, f1, fc, acc_grid, acc_col);
-    if (wm | jm) {
-        float4 *pub = rs.rec + 3 * lane;
-        if (joins) {
-            pub[0] = f0;
-            pub[1] = f1;
-            pub[2] = fc;
-        } else if (whole) {
-            pub[0] = g0;
-            pub[1] = g1;
-            pub[2] = c;
-        }
-        __syncwarp();
-        if (!whole) {
-            const unsigned w = lane < 31 ? wm >> (lane + 1) : 0u, j = lane < 31 ? jm >> (lane + 1) : 0u;
-            int m = __ffs(~w) - 1;       // lanes after this one that it holds whole
+    if (r0 < n && !whole) {
+        if (cm) {
+            const unsigned w = lane < 31 ? wm >> (lane + 1) : 0u, j = lane < 31 ? cm >> (lane + 1) : 0u;
+            int m = __ffs(~w) - 1;       // lanes after this one that hold nothing else
             m += (int)((j >> m) & 1u);   // and one that starts with the rest
-            for (int i = 1; i <= m; ++i) {
-                add4(g0, pub[3 * i]);
-                add4(g1, pub[3 * i + 1]);
-                add4(c, pub[3 * i + 2]);
+            const float4 *q = r;
+            for (; m > 0; --m) {
+                q += 3 * kRecLane + 1;
+                add4(g0, q[0]);
+                add4(g1, q[1]);
+                add4(c, q[2]);
             }
         }
+        add_sum(st[k_last], g0, g1, c, acc_grid, acc_col);
     }
-    if (k >= 0 && !whole) add_sum(st[k], g0, g1, c, acc_grid, acc_col);
     __syncwarp();
 }
 
@@ -1472,29 +1509,151 @@ struct BwdIn {
     float *max_weight;      // extras: [N] per-voxel maximum of T_i alpha_i (atomicMax), or NULL
 };
 
+// What the backward of an item starts from: the calling lane's pixel, its
+// upstream gradients, and the state behind the item's part of the list (in
+// front of it: T_before).
+struct BwdPixel {
+    PixelRay p;
+    PixelGrad g;
+    int last, idx0;       // last voxel's sorted index; the part's first one
+    float T_after, T_before, SC0, SC1, SC2, SD;
+    NrmSums SN;
+    DistSums DS;
+    bool has, fallback;   // whether it has hits here; whether they are taken front to back
+};
+
+// False if the item has nothing to do.
+template <int XM>
+__device__ __forceinline__ bool bwd_load(const FrameDev &f, const Item &it, const BwdIn &in, const ItemView &iv,
+                                         WarpBlock &wb, BwdPixel &b) {
+    constexpr bool XN = (XM & kXNrm) != 0, XD = (XM & kXDist) != 0;
+    const DevCam &cam = f.views[iv.view];
+    const PixelRay p = pixel_ray(cam, iv.tile, it.blk, wb);
+    if (wb.smask == 0) return false;
+    b.p = p;
+    const int beg = it.beg;
+    const bool split = it.slot != kNoSlot;
+    const int lane = threadIdx.x & 31;
+    const size_t HW = (size_t)cam.W * cam.H;
+    const size_t px = (size_t)p.y * cam.W + p.x;
+    const size_t o = (size_t)cam.pix_base + px;
+
+    PixelGrad g = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    float Tfin = 1.f;
+    int last = beg - 1;
+    if (p.inside) {
+        if (in.d_rgb) {
+            const float *gr = in.d_rgb + 3 * (size_t)cam.pix_base + px;
+            g.gC0 = gr[0];
+            g.gC1 = gr[HW];
+            g.gC2 = gr[2 * HW];
+        }
+        if (in.d_depth) g.gD = in.d_depth[o];
+        if (XN && in.d_normal) {
+            const float *gn = in.d_normal + 3 * (size_t)cam.pix_base + px;
+            g.gN0 = gn[0];
+            g.gN1 = gn[HW];
+            g.gN2 = gn[2 * HW];
+        }
+        Tfin = in.T[o];
+        if (in.d_alpha) g.gAT = in.d_alpha[o] * Tfin;
+        if (XD && in.d_dist) {
+            g.gL = in.d_dist[o];
+            g.Wtot = 1.f - Tfin;
+            g.Stot = in.dist[2 * (size_t)cam.pix_base + HW + px];
+        }
+        last = max(beg - 1, min(in.last[o], it.end - 1));   // stay inside the tile's list
+    }
+    // The part of the list this item covers and the state behind it: the
+    // whole list behind which lies T_final bg, or one segment of a split
+    // tile with the forward's sums behind it and transmittance around it.
+    int idx0 = beg;
+    float T_after = Tfin, T_before = 1.f;
+    float SC0 = Tfin * f.bg[0], SC1 = Tfin * f.bg[1], SC2 = Tfin * f.bg[2], SD = 0.f;
+    NrmSums SN = {0.f, 0.f, 0.f};
+    DistSums DS = {0.f, 0.f, 0.f};
+    // every tile takes the hit masks of this sort's forward; a split tile
+    // also starts from its segment sums, which must include the normal image
+    // and the distortion sums when their gradients are asked for
+    {
+        const unsigned done = f.status->fwd_done;
+        if (done == 0 || (split && ((XN && in.d_normal && !(done & 2u)) || (XD && in.d_dist && !(done & 4u))))) {
+            if (lane == 0) atomicOr(&f.status->flags, SVR_FLAG_NO_FORWARD);
+            return false;
+        }
+    }
+    if (split) {
+        idx0 = beg + it.seg * kSegLen;
+        const float *q = seg_fields(f, it.slot, it.blk);
+        SC0 = q[0];
+        SC1 = q[32];
+        SC2 = q[2 * 32];
+        SD = q[3 * 32];
+        T_after = q[4 * 32];
+        T_before = q[5 * 32];
+        if (XN) {
+            SN.x = q[8 * 32];
+            SN.y = q[9 * 32];
+            SN.z = q[10 * 32];
+        }
+        if (XD && in.d_dist) {
+            DS.W = q[11 * 32];
+            DS.S = q[12 * 32];
+            DS.R = q[13 * 32];
+        }
+    }
+    b.g = g;
+    b.last = last;
+    b.idx0 = idx0;
+    b.T_after = T_after;
+    b.T_before = T_before;
+    b.SC0 = SC0;
+    b.SC1 = SC1;
+    b.SC2 = SC2;
+    b.SD = SD;
+    b.SN = SN;
+    b.DS = DS;
+    b.has = p.inside && last >= idx0;
+    b.fallback = b.has && T_after < 1e-30f;
+    return true;
+}
+
 // Front-to-back gradients for the pixels of an item whose transmittance
 // behind their part of the list underflowed (the back-to-front recovery
 // T_i = T_(i+1) / (1 - alpha_i) would lose precision): sweep 1 sums the
 // part's colour, depth (and normal) from the transmittance in front of it,
 // sweep 2 takes the gradients with the sums behind each voxel as total minus
 // prefix.
+// Rare, and a function of its own that loads the item again, so that nothing
+// it needs weighs on the main path's registers.
 template <int K, int XM>
-__device__ __noinline__ void bwd_front_to_back(const FrameDev &f, const ItemList L, int p0, int p1, int idx0,
-                                               int last, bool fallback, float T_before, float SC0, float SC1, float SC2,
-                                               float SD, NrmSums SN, DistSums DSb, const ViewData vd,
-                                               const WarpBlock wb, const PixelRay p, const PixelGrad g, Entry *st,
-                                               RecSmem &rs, const BwdIn &in, float4 *dcol) {
+__device__ __noinline__ void bwd_front_to_back(const FrameDev &f, unsigned w, Entry *st, RecSmem &rs, const BwdIn &in) {
     constexpr bool XN = (XM & kXNrm) != 0, XD = (XM & kXDist) != 0, XS = (XM & kXStat) != 0;
     const int lane = threadIdx.x & 31;
-    const int n_fb = lower_pos(L.list, p0, p1, __reduce_max_sync(0xffffffffu, fallback ? last + 1 : idx0));
+    const Item it = load_item(f, w);
+    const ItemView iv = item_view(f, it.g);
+    const ViewData &vd = iv.vd;
+    WarpBlock wb;
+    BwdPixel bp;
+    if (!bwd_load<XM>(f, it, in, iv, wb, bp)) return;
+    float4 *dcol = f.dcol + (size_t)iv.view * f.n_vox;
+    const PixelRay &p = bp.p;
+    const PixelGrad &g = bp.g;
+    const int last = bp.last;
+    const bool fallback = bp.fallback;
+    const float T_before = bp.T_before, SC0 = bp.SC0, SC1 = bp.SC1, SC2 = bp.SC2, SD = bp.SD;
+    const NrmSums SN = bp.SN;
+    const DistSums DSb = bp.DS;
+    const uint2 *list = it.list;
+    const int n_fb = lower_pos(list, 0, it.n, __reduce_max_sync(0xffffffffu, fallback ? last + 1 : bp.idx0));
     // sweep 1: this part's own sums, from the transmittance in front of it
     // (distortion: the part's internal loss and sums of w, w m)
     float T = T_before, Ct0 = 0.f, Ct1 = 0.f, Ct2 = 0.f, Dt = 0.f;
     NrmSums Nt = {0.f, 0.f, 0.f};
     FwdState dp = {};
-    for (int base = p0; base < n_fb; base += kBatch) {
+    for (int base = 0; base < n_fb; base += kBatch) {
         Lookahead cur;
-        fetch_vi(cur, L.list, base + lane, base + lane < n_fb);
+        fetch_vi(cur, list, base + lane, base + lane < n_fb);
         fetch_box(cur, vd);
         const unsigned cand = warp_transpose(entry_pixels(cur.valid, cur.vi.x, cur.box, wb));
         stage_ahead(st, vd, cur);
@@ -1538,9 +1697,9 @@ __device__ __noinline__ void bwd_front_to_back(const FrameDev &f, const ItemList
     float Tf = T_before, PC0 = 0.f, PC1 = 0.f, PC2 = 0.f, PD = 0.f;
     NrmSums PN = {0.f, 0.f, 0.f};
     float PW = 0.f, PS = 0.f, PR = 0.f;
-    for (int base = p0; base < n_fb; base += kBatch) {
+    for (int base = 0; base < n_fb; base += kBatch) {
         Lookahead cur;
-        fetch_vi(cur, L.list, base + lane, base + lane < n_fb);
+        fetch_vi(cur, list, base + lane, base + lane < n_fb);
         fetch_box(cur, vd);
         const unsigned cand = warp_transpose(entry_pixels(cur.valid, cur.vi.x, cur.box, wb));
         stage_ahead(st, vd, cur);
@@ -1616,118 +1775,52 @@ __device__ __noinline__ void bwd_front_to_back(const FrameDev &f, const ItemList
 }
 
 template <int K, int XM>
-__device__ __forceinline__ void bwd_item(const FrameDev &f, const Item &it, Entry *st, RecSmem &rs,
-                                         const BwdIn &in) {
+__device__ __forceinline__ void bwd_item(const FrameDev &f, unsigned w, Entry *st, RecSmem &rs, const BwdIn &in) {
     constexpr bool XN = (XM & kXNrm) != 0, XD = (XM & kXDist) != 0, XS = (XM & kXStat) != 0;
-    const ItemView iv = item_view(f, it.g);
-    const DevCam &cam = f.views[iv.view];
-    const ViewData &vd = iv.vd;
-    float4 *dcol = f.dcol + (size_t)iv.view * f.n_vox;
-    WarpBlock wb;
-    const PixelRay p = pixel_ray(cam, iv.tile, it.blk, wb);
-    if (wb.smask == 0) return;
-    const ItemList L = item_list(f, it.g, it.blk);
-    {
-        // a block with no entries in this item's part of the list has no hit
-        int q0 = 0, q1 = L.n_list;
-        if (L.ts.x > 1) seg_range(L, f.blocks_per_tile, it.seg, q0, q1);
-        if (q1 <= q0) return;
-    }
-    const int beg = L.beg;
+    const Item it = load_item(f, w);
+    if (it.n == 0) return;
+    const bool split = it.slot != kNoSlot;
     const int lane = threadIdx.x & 31;
-    const size_t HW = (size_t)cam.W * cam.H;
-    const size_t px = (size_t)p.y * cam.W + p.x;
-    const size_t o = (size_t)cam.pix_base + px;
+    const ItemView iv = item_view(f, it.g);
+    const ViewData &vd = iv.vd;
+    WarpBlock wb;
+    BwdPixel bp;
+    if (!bwd_load<XM>(f, it, in, iv, wb, bp)) return;
+    float4 *dcol = f.dcol + (size_t)iv.view * f.n_vox;
+    const PixelRay &p = bp.p;
+    const PixelGrad &g = bp.g;
+    const int last = bp.last;
+    float T_after = bp.T_after, SC0 = bp.SC0, SC1 = bp.SC1, SC2 = bp.SC2, SD = bp.SD;
+    NrmSums SN = bp.SN;
+    DistSums DS = bp.DS;
+    const bool active = bp.has && !bp.fallback;
 
-    PixelGrad g = {0.f, 0.f, 0.f, 0.f, 0.f, 1.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    int last = beg - 1;
-    if (p.inside) {
-        if (in.d_rgb) {
-            const float *gr = in.d_rgb + 3 * (size_t)cam.pix_base + px;
-            g.gC0 = gr[0];
-            g.gC1 = gr[HW];
-            g.gC2 = gr[2 * HW];
-        }
-        if (in.d_depth) g.gD = in.d_depth[o];
-        if (in.d_alpha) g.gA = in.d_alpha[o];
-        if (XN && in.d_normal) {
-            const float *gn = in.d_normal + 3 * (size_t)cam.pix_base + px;
-            g.gN0 = gn[0];
-            g.gN1 = gn[HW];
-            g.gN2 = gn[2 * HW];
-        }
-        g.Tfin = in.T[o];
-        if (XD && in.d_dist) {
-            g.gL = in.d_dist[o];
-            g.Wtot = 1.f - g.Tfin;
-            g.Stot = in.dist[2 * (size_t)cam.pix_base + HW + px];
-        }
-        last = max(beg - 1, min(in.last[o], L.end - 1));   // stay inside the tile's list
-    }
-    // The part of the list this item covers and the state behind it: the
-    // whole list behind which lies T_final bg, or one segment of a split
-    // tile with the forward's sums behind it and transmittance around it.
-    int p0 = 0, p1 = L.n_list, idx0 = beg;
-    float T_after = g.Tfin, T_before = 1.f;
-    float SC0 = g.Tfin * f.bg[0], SC1 = g.Tfin * f.bg[1], SC2 = g.Tfin * f.bg[2], SD = 0.f;
-    NrmSums SN = {0.f, 0.f, 0.f};
-    DistSums DS = {0.f, 0.f, 0.f};
-    // every tile takes the hit masks of this sort's forward; a split tile
-    // also starts from its segment sums, which must include the normal image
-    // and the distortion sums when their gradients are asked for
+    // ---- back to front, over the forward's batches [32 k, 32 k + 32): each
+    // pixel's hits in a batch are the forward's hit mask (which tested every
+    // candidate of the batch before the pixel stopped) restricted to the
+    // entries up to its last voxel.  No pixel's last voxel lies beyond the
+    // batches that the forward walked; in a split list it may lie well before
+    // them (the segment was walked from T = 1), so its place is searched.
     {
-        const unsigned done = f.status->fwd_done;
-        if (done == 0 || (L.ts.x > 1 && ((XN && in.d_normal && !(done & 2u)) || (XD && in.d_dist && !(done & 4u))))) {
-            if (lane == 0) atomicOr(&f.status->flags, SVR_FLAG_NO_FORWARD);
-            return;
-        }
-    }
-    if (L.ts.x > 1) {
-        seg_range(L, f.blocks_per_tile, it.seg, p0, p1);
-        idx0 = beg + it.seg * kSegLen;
-        const float *q = seg_fields(f, L.ts.y + it.seg, it.blk);
-        SC0 = q[0];
-        SC1 = q[32];
-        SC2 = q[2 * 32];
-        SD = q[3 * 32];
-        T_after = q[4 * 32];
-        T_before = q[5 * 32];
-        if (XN) {
-            SN.x = q[8 * 32];
-            SN.y = q[9 * 32];
-            SN.z = q[10 * 32];
-        }
-        if (XD && in.d_dist) {
-            DS.W = q[11 * 32];
-            DS.S = q[12 * 32];
-            DS.R = q[13 * 32];
-        }
-    }
-    const bool has = p.inside && last >= idx0;
-    const bool fallback = has && T_after < 1e-30f;
-    const bool active = has && !fallback;
-
-    // ---- back to front, over the forward's batches [p0 + 32 k, p0 + 32 k + 32):
-    // each pixel's hits in a batch are the forward's hit mask (which tested
-    // every candidate of the batch before the pixel stopped) restricted to
-    // the entries up to its last voxel
-    {
-        const int top_all = lower_pos(L.list, p0, p1, __reduce_max_sync(0xffffffffu, active ? last + 1 : idx0));
-        const uint32_t *hm = hit_masks(f, L, it);
-        int base = p0 + (((top_all - 1 - p0) >> 5) << 5);   // the batch of position top_all - 1
+        int top_all = 0;
+        if (__any_sync(0xffffffffu, active))
+            top_all = !split ? min((int)it.walked, it.n)
+                             : lower_pos(it.list, 0, it.n, __reduce_max_sync(0xffffffffu, active ? last + 1 : bp.idx0));
+        const uint32_t *hm = it.hm;
+        int base = ((top_all - 1) >> 5) << 5;   // the batch of position top_all - 1
         Lookahead la;
         unsigned m_next = 0u;
         la.valid = false;
-        if (top_all > p0) {
-            fetch_vi(la, L.list, base + kBatch - 1 - lane, base + kBatch - 1 - lane < top_all);
+        if (top_all > 0) {
+            fetch_vi(la, it.list, base + kBatch - 1 - lane, base + kBatch - 1 - lane < top_all);
             m_next = __ldg(hm + base + lane);
         }
         prefetch_record(la, vd);
-        for (; top_all > p0 && base >= p0; base -= kBatch) {
+        for (; top_all > 0 && base >= 0; base -= kBatch) {
             const Lookahead cur = la;
             const unsigned m = m_next;
-            if (base - kBatch >= p0) {
-                fetch_vi(la, L.list, base - 1 - lane, true);
+            if (base - kBatch >= 0) {
+                fetch_vi(la, it.list, base - 1 - lane, true);
                 m_next = __ldg(hm + base - kBatch + lane);
             } else {
                 la.valid = false;
@@ -1804,11 +1897,8 @@ __device__ __forceinline__ void bwd_item(const FrameDev &f, const Item &it, Entr
         }
     }
 
-    // ---- front to back for pixels whose transmittance underflowed (rare:
-    // kept out of line so that it does not weigh on the main path's registers)
-    if (__any_sync(0xffffffffu, fallback))
-        bwd_front_to_back<K, XM>(f, L, p0, p1, idx0, last, fallback, T_before, SC0, SC1, SC2, SD, SN, DS, vd, wb,
-                                    p, g, st, rs, in, dcol);
+    // ---- front to back for pixels whose transmittance underflowed
+    if (__any_sync(0xffffffffu, bp.fallback)) bwd_front_to_back<K, XM>(f, w, st, rs, in);
 }
 
 template <int K, int XM>
@@ -1817,11 +1907,10 @@ __global__ void __launch_bounds__(kBwdThreads, kBwdMinBlocks) k_render_bwd(Frame
     __shared__ RecSmem recs[kBwdWarps];
     const int warp = threadIdx.x >> 5;
     Entry *st = stage[warp];
-    const unsigned bpt = (unsigned)f.blocks_per_tile;
-    const unsigned n_items = f.status->n_listed * bpt;  // an empty tile has no gradient
-    Item it;
-    while (next_item(&f.status->bwd_next, n_items, bpt, f.order, it)) {
-        bwd_item<K, XM>(f, it, st, recs[warp], in);
+    const unsigned n_items = f.status->n_listed * (unsigned)f.blocks_per_tile;   // an empty tile has no gradient
+    unsigned w;
+    while (next_work(&f.status->bwd_next, n_items, w)) {
+        bwd_item<K, XM>(f, w, st, recs[warp], in);
         __syncwarp();
     }
 }
@@ -1945,14 +2034,21 @@ cudaError_t launch_block_lists(const FrameDev &f, int sorted_alt, cudaStream_t s
     return cudaGetLastError();
 }
 
-// Grid size from a lower bound on the work items (every tile has at least
-// one segment); the kernels read the exact count from the device.
+// Bound on the render items: every tile's blocks, and those of the segments
+// of split lists if a list can be that long (every voxel with every sign
+// pattern).  The kernels read the exact counts from the device; a grid sized
+// for the tiles alone left a third of the chip idle on a 320 x 210 preview
+// of 2M voxels, whose few tiles have up to 88 segments each.
+static int64_t max_items(const FrameDev &f) {
+    return (f.total_tiles + (8 * f.n_vox > kSegLen ? f.seg_slots : 0)) * (int64_t)f.blocks_per_tile;
+}
+
 template <int K, int MODE>
 static cudaError_t fwd_k(const FrameDev &f, const FwdOut &out, cudaStream_t s) {
     static DeviceCache cache;
     const unsigned grid = device_cached(cache, [] { return persistent_grid(k_render_fwd<K, MODE>, kThreads); });
-    const unsigned items = (unsigned)f.total_tiles * (unsigned)f.blocks_per_tile;
-    const unsigned g = tmin<unsigned>(grid, (items + kWarps - 1) / kWarps);
+    const int64_t items = max_items(f);
+    const unsigned g = (unsigned)tmin<int64_t>(grid, (items + kWarps - 1) / kWarps);
     k_render_fwd<K, MODE><<<g, kThreads, 0, s>>>(f, out);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || MODE != kModeExtra || !out.max_weight) return e;
@@ -1964,7 +2060,7 @@ static cudaError_t fwd_k(const FrameDev &f, const FwdOut &out, cudaStream_t s) {
     FwdOut wout = out;
     wout.normal = nullptr;
     wout.dist = nullptr;
-    k_render_maxw<K><<<tmin<unsigned>(grid_w, (items + kWarps - 1) / kWarps), kThreads, 0, s>>>(f, wout);
+    k_render_maxw<K><<<(unsigned)tmin<int64_t>(grid_w, (items + kWarps - 1) / kWarps), kThreads, 0, s>>>(f, wout);
     return cudaGetLastError();
 }
 
@@ -1973,8 +2069,8 @@ static cudaError_t bwd_k(const FrameDev &f, const BwdIn &in, cudaStream_t s) {
     static DeviceCache cache;
     const unsigned grid =
         device_cached(cache, [] { return persistent_grid(k_render_bwd<K, XM>, kBwdThreads); });
-    const unsigned items = (unsigned)f.total_tiles * (unsigned)f.blocks_per_tile;
-    const unsigned g = tmin<unsigned>(grid, (items + kBwdWarps - 1) / kBwdWarps);
+    const int64_t items = max_items(f);
+    const unsigned g = (unsigned)tmin<int64_t>(grid, (items + kBwdWarps - 1) / kBwdWarps);
     k_render_bwd<K, XM><<<g, kBwdThreads, 0, s>>>(f, in);
     return cudaGetLastError();
 }

@@ -389,7 +389,7 @@ __global__ void __cluster_dims__(kMergeCluster, 1, 1) __launch_bounds__(kMergeTh
                     if ((t & 31) == 0) split[warp] = c;
                 }
                 __syncthreads();
-                const int a0 = split[0], a1 = split[1], b0 = d0 - a0, b1 = d1 - a1;
+                const int a0 = split[0], a1 = split[1], b0 = d0 - a0;
                 const int ca = a1 - a0, n = d1 - d0;
                 for (int i = t; i < n; i += kMergeThreads) {
                     const int64_t from = i < ca ? p0 + a0 + i : mid + b0 + (i - ca);

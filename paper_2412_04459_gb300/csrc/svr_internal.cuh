@@ -85,6 +85,23 @@ struct Status {
     unsigned pad[2];
 };
 
+// A work item of the render kernels: the 8x4 block `blk` of a tile and its
+// block list, or the part of it in one segment of a split tile's list.
+// k_block_lists writes those of every work-order entry e with a non-empty list
+// at e B + blk, so a warp has all it needs about its work one load after it
+// was given its number (the order, ranges, segments and lengths were four
+// dependent loads).
+struct __align__(16) RenderItem {
+    uint32_t tile;     // global tile
+    uint32_t blkseg;   // block | segment << 8
+    uint32_t n;        // entries of the block list (in this segment)
+    uint32_t beg, end; // the tile's range in the sorted pairs
+    uint32_t slot;     // segment slot of a split tile, else kNoSlot
+    uint32_t walked;   // entries the forward's first walk took (written by it)
+    uint32_t pad;
+};
+constexpr uint32_t kNoSlot = 0xFFFFFFFFu;
+
 // Groups of the render work order: floor(log2(length)) + 1 of a tile's list,
 // one more for a split list, so that every split list (longer than kSegLen)
 // precedes every unsplit one; a split list's first segment goes to group
@@ -297,7 +314,7 @@ struct FrameDev {
     int64_t seg_slots;       // slots the workspace holds
     uint2 *blist;            // per (tile, 8x4 block) lists of (value, sorted index): block b of a tile
                              // whose list is [beg, end) owns [B beg + b (end - beg), ...)
-    uint32_t *blen;          // [total_tiles * B] entries in each block list
+    RenderItem *items;       // [(total_tiles + seg slots) * B]
     uint32_t *hmask;         // the forward's hit masks: block b of tile g (list [beg, end)) owns the
                              // words from B beg + b (end - beg) + 32 (g B + b); word p of it is, for
                              // p in batch [32 k, 32 k + 32) of the block's walk, the mask of the
