@@ -522,9 +522,9 @@ __device__ __forceinline__ void hit_fwd(const Entry &e, const PixelRay &p, float
     for (int k = 0; k < K; ++k) {
         const float v = trilerp(e.g0, e.g1, fmaf(t, rx, -e.c.x), fmaf(t, ry, -e.c.y), fmaf(t, rz, -e.c.z));
         const float xk = xs * explin(v);
-        const float ek = ex2(-xk);
-        d = fmaf(P * (1.f - ek), t, d);
-        P *= ek;
+        const float Pn = P * ex2(-xk);
+        d = fmaf(P - Pn, t, d);
+        P = Pn;
         X += xk;
         t += step;
     }
@@ -676,9 +676,9 @@ __device__ __forceinline__ void hit_fwd_slot(const FwdSlot &e, const PixelRay &p
     for (int k = 0; k < K; ++k) {
         const float v = trilerp(g0, g1, fmaf(t, rx, -cx), fmaf(t, ry, -cy), fmaf(t, rz, -cz));
         const float xk = xs * explin(v);
-        const float ek = ex2(-xk);
-        d = fmaf(P * (1.f - ek), t, d);
-        P *= ek;
+        const float Pn = P * ex2(-xk);
+        d = fmaf(P - Pn, t, d);
+        P = Pn;
         X += xk;
         t += step;
     }
@@ -1234,30 +1234,32 @@ __device__ __forceinline__ void hit_grad(const Entry &e, const PixelRay &p, cons
     const float step = seg * inv_k;
     const float inv_size = e.b.w;
     const float rx = p.rd.x * inv_size, ry = p.rd.y * inv_size, rz = p.rd.z * inv_size;
-    float tk[K], ek[K], qx[K], qy[K], qz[K], dsig[K];
+    // of each sample: its place, the transmittance up to it, and d x_k / d v_k
+    // (explin' is 1 above 1.1, else explin / 1.1)
+    float tk[K], Pk[K + 1], qx[K], qy[K], qz[K], dx[K];
     float t = fmaf(0.5f, step, a);
-    float trans = 1.f, d = 0.f, X = 0.f;
+    float d = 0.f, X = 0.f;
+    Pk[0] = 1.f;
 #pragma unroll
     for (int k = 0; k < K; ++k) {
         qx[k] = fmaf(t, rx, -e.c.x);
         qy[k] = fmaf(t, ry, -e.c.y);
         qz[k] = fmaf(t, rz, -e.c.z);
         const float v = trilerp(e.g0, e.g1, qx[k], qy[k], qz[k]);
-        const float sig = explin(v);
-        dsig[k] = v > 1.1f ? 1.f : sig * 0.909090909f;
-        const float xk = xs2 * sig;
-        ek[k] = ex2(-xk);
+        const float xk = xs2 * explin(v);
+        dx[k] = v > 1.1f ? xs : xk * (kLn2 * 0.909090909f);
+        Pk[k + 1] = Pk[k] * ex2(-xk);
         X += xk;
         tk[k] = t;
-        d = fmaf(trans * (1.f - ek[k]), t, d);
-        trans *= ek[k];
+        d = fmaf(Pk[k] - Pk[k + 1], t, d);
         t += step;
     }
+    const float trans = Pk[K];
     if (B2F) {
         // T_known >= 1e-30 here (smaller goes front to back) and T_i <= 1, so
-        // trans >= 1e-30 lies in the fast division's 2-ulp range
+        // trans >= 1e-30 is far from the reciprocal's flushed range
         T_after = T_known;
-        T_i = __fdividef(T_known, trans);
+        T_i = T_known * rcp(trans);
     } else {
         T_i = T_known;
         T_after = T_known * trans;
@@ -1299,10 +1301,6 @@ __device__ __forceinline__ void hit_grad(const Entry &e, const PixelRay &p, cons
     }
     if (XS) prio = fabsf(gx * al / fmaxf(trans, 1e-30f));
     // per-sample depth term, suffix Q_k = sum_{m>k} P_m (1 - e_m) t_m
-    float Pk[K + 1];
-    Pk[0] = 1.f;
-#pragma unroll
-    for (int k = 0; k < K; ++k) Pk[k + 1] = Pk[k] * ek[k];
     float Q = 0.f;
 #pragma unroll
     for (int c = 0; c < 8; ++c) dgeo[c] = 0.f;
@@ -1310,7 +1308,7 @@ __device__ __forceinline__ void hit_grad(const Entry &e, const PixelRay &p, cons
 #pragma unroll
     for (int k = K - 1; k >= 0; --k) {
         const float gxk = fmaf(gdT, fmaf(Pk[k + 1], tk[k], -Q), gx);
-        const float dv = gxk * xs * dsig[k];
+        const float dv = gxk * dx[k];
         // adjoint of the polynomial's coefficients (trilerp)
         const float ax = dv * qx[k], ay = dv * qy[k], axy = ax * qy[k];
         dgeo[0] += dv;
@@ -1321,7 +1319,7 @@ __device__ __forceinline__ void hit_grad(const Entry &e, const PixelRay &p, cons
         dgeo[5] = fmaf(ax, qz[k], dgeo[5]);
         dgeo[6] += axy;
         dgeo[7] = fmaf(axy, qz[k], dgeo[7]);
-        Q = fmaf(Pk[k] * (1.f - ek[k]), tk[k], Q);
+        Q = fmaf(Pk[k] - Pk[k + 1], tk[k], Q);
     }
     // normal: dL/dn = w g_N, through the normalisation (I - n n^T) / |grad|
     // to the linear coefficients (Eq. interp_grad_grad)

@@ -250,6 +250,13 @@ __device__ __forceinline__ float ex2(float x) {
 }
 constexpr float kLog2e = 1.44269504f, kLn2 = 0.693147181f;
 
+// 1 / x to 1 ulp, the hardware instruction on its own.
+__device__ __forceinline__ float rcp(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
 // explin (Eq. explin): x above 1.1, else exp(x / 1.1 - 1 + ln 1.1), whose
 // exponent in base 2 is (x / 1.1 - 1 + ln 1.1) log2(e).
 __device__ __forceinline__ float explin(float x) { return x > 1.1f ? x : ex2(fmaf(x, 1.31154095f, -1.30519153f)); }
