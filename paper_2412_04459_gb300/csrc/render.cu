@@ -1923,6 +1923,11 @@ __global__ void __launch_bounds__(kBwdThreads, kBwdMinBlocks) k_render_bwd(Frame
 constexpr int kVoxBwdThreads = 128;
 constexpr int kShRow = 52;
 
+// A batch's views are taken VIEWS = 4 at a time, their loads in flight
+// together (0.82 -> 0.59 ms for 8 views of 8M voxels, 191 -> 133 us for 16 of
+// 1M); a single view by its own instantiation, which needs fewer registers (40
+// us for 1M voxels, 45 with four).
+template <int VIEWS>
 __global__ void __launch_bounds__(kVoxBwdThreads) k_voxel_bwd(FrameDev f, float *__restrict__ d_sh,
                                                               float *__restrict__ priority) {
     __shared__ __align__(16) float rows[kVoxBwdThreads * kShRow];
@@ -1933,23 +1938,32 @@ __global__ void __launch_bounds__(kVoxBwdThreads) k_voxel_bwd(FrameDev f, float 
 #pragma unroll
         for (int i = 0; i < 48; ++i) o[i] = 0.f;
         float prio = 0.f;
-        for (int view = 0; view < f.n_views; ++view) {
-            const int64_t iv = (int64_t)view * f.n_vox + v;
-            if (f.count[iv] == 0) continue;
-            const DevCam &cam = f.views[view];
-            const float4 g = f.dcol[iv];
-            prio += g.w;
-            float dx = f.centre[3 * v + 0] - cam.ro[0];
-            float dy = f.centre[3 * v + 1] - cam.ro[1];
-            float dz = f.centre[3 * v + 2] - cam.ro[2];
-            const float inv = 1.0f / sqrtf(dx * dx + dy * dy + dz * dz);
-            float Y[16];
-            sh_basis(dx * inv, dy * inv, dz * inv, Y);
+        for (int view0 = 0; view0 < f.n_views; view0 += VIEWS) {
+            bool seen[VIEWS];
+            float4 g[VIEWS];
 #pragma unroll
-            for (int n = 0; n < 16; ++n) {
-                o[3 * n + 0] = fmaf(Y[n], g.x, o[3 * n + 0]);
-                o[3 * n + 1] = fmaf(Y[n], g.y, o[3 * n + 1]);
-                o[3 * n + 2] = fmaf(Y[n], g.z, o[3 * n + 2]);
+            for (int i = 0; i < VIEWS; ++i)
+                seen[i] = view0 + i < f.n_views && f.count[(int64_t)(view0 + i) * f.n_vox + v] != 0;
+#pragma unroll
+            for (int i = 0; i < VIEWS; ++i)
+                if (seen[i]) g[i] = f.dcol[(int64_t)(view0 + i) * f.n_vox + v];
+#pragma unroll
+            for (int i = 0; i < VIEWS; ++i) {
+                if (!seen[i]) continue;
+                const DevCam &cam = f.views[view0 + i];
+                prio += g[i].w;
+                float dx = f.centre[3 * v + 0] - cam.ro[0];
+                float dy = f.centre[3 * v + 1] - cam.ro[1];
+                float dz = f.centre[3 * v + 2] - cam.ro[2];
+                const float inv = 1.0f / sqrtf(dx * dx + dy * dy + dz * dz);
+                float Y[16];
+                sh_basis(dx * inv, dy * inv, dz * inv, Y);
+#pragma unroll
+                for (int n = 0; n < 16; ++n) {
+                    o[3 * n + 0] = fmaf(Y[n], g[i].x, o[3 * n + 0]);
+                    o[3 * n + 1] = fmaf(Y[n], g[i].y, o[3 * n + 1]);
+                    o[3 * n + 2] = fmaf(Y[n], g[i].z, o[3 * n + 2]);
+                }
             }
         }
         float4 *row = reinterpret_cast<float4 *>(rows + threadIdx.x * kShRow);
@@ -2133,7 +2147,8 @@ cudaError_t launch_render_bwd(const FrameDev &f, const float *d_rgb, const float
         const unsigned blocks = (unsigned)((f.n_vox + kVoxBwdThreads - 1) / kVoxBwdThreads);
         const int64_t per = kGridThreads * kGridIlp / 8;
         k_grid_bwd<<<(unsigned)((f.n_vox + per - 1) / per), kGridThreads, 0, s>>>(f, d_grid);
-        k_voxel_bwd<<<blocks, kVoxBwdThreads, 0, s>>>(f, d_sh, priority);
+        if (f.n_views == 1) k_voxel_bwd<1><<<blocks, kVoxBwdThreads, 0, s>>>(f, d_sh, priority);
+        else k_voxel_bwd<4><<<blocks, kVoxBwdThreads, 0, s>>>(f, d_sh, priority);
         e = cudaGetLastError();
     }
     return e;
