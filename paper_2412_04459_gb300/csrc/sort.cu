@@ -189,17 +189,17 @@ __device__ __forceinline__ void group_sort(uint64_t (&x)[VT], uint64_t *s, int t
     sort_network<VT>(x, less);
     const int o = t * VT;
     bool wide = false;   // whether the last merge read other warps' words
-    for (int w = VT;; w *= 2) {
-        const bool next_wide = 2 * w > 32 * VT;
+    for (int m = 1;; m *= 2) {   // runs of m threads' words
+        const bool next_wide = m > 16;
         if (wide) group_sync(gt, g);
         else __syncwarp();
 #pragma unroll
         for (int i = 0; i < VT; ++i) s[pad(o + i)] = x[i];
-        const bool last = w >= gt * VT;
+        const bool last = m >= gt;
         if (next_wide || last) group_sync(gt, g);
         else __syncwarp();
         if (last) return;
-        const int p0 = o & ~(2 * w - 1);
+        const int p0 = (t & ~(2 * m - 1)) * VT, w = m * VT;
         merge_out<VT>(s, p0, p0 + w, p0 + w, p0 + 2 * w, o - p0, x, less);
         wide = next_wide;
     }
@@ -274,42 +274,55 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_sort_lists(FrameDev f) {
         __syncthreads();
         unsigned u = unit;
         __syncthreads();
+        // the group's list or chunk: n pairs from c0
+        int gt = kSortThreads, n, dst = -1;
+        unsigned tile;
+        uint32_t c0;
         if (u < n_chunks) {
             const uint2 q = f.chunks[u];
             const uint2 rg = f.ranges[q.x];
             if (!SVR_IN_BOUNDS(f.debug, kDbgRange, rg.y, f.capacity + 1)) continue;
-            const int L = (int)(rg.y - rg.x), c0 = (int)q.y * kSortCap;
+            const int L = (int)(rg.y - rg.x), first = (int)q.y * kSortCap;
             const int r = merge_rounds(list_chunks(L));
-            // the merge rounds alternate between the buffers and end in the first
-            sort_list<MODE, kSortVT>(f, smem, threadIdx.x, kSortThreads, 0, (int)q.x, rg.x + c0, min(kSortCap, L - c0),
-                                     r ? (r & 1) : -1);
-            continue;
-        }
-        u -= n_chunks;
-        int c = kSortClasses - 1;
-        for (; c >= 0; --c) {
-            const int per = 16 >> (c > 0 ? c - 1 : 0);
-            const unsigned units = (plan->count[c] + per - 1) / per;
-            if (u < units) break;
-            u -= units;
-        }
-        if (c < 0) return;
-        const int gt = 32 << (c > 0 ? c - 1 : 0);
-        const int g = threadIdx.x / gt, t = threadIdx.x & (gt - 1);
-        const unsigned e = u * (kSortThreads / gt) + g;
-        if (e >= plan->count[c]) continue;
-        const unsigned tile = f.order[plan->first[c] + e].x;
-        const uint2 rg = f.ranges[tile];
-        if (!SVR_IN_BOUNDS(f.debug, kDbgRange, rg.y, f.capacity + 1)) continue;
-        const int n = (int)(rg.y - rg.x);
-        if (n > gt * kSortVT) continue;   // not reached: the class's longest list fits
-        uint64_t *s = smem + (size_t)g * (gt / 16 * 17 * kSortVT);
-        if (n <= 32) {
-            if (n > 1 || MODE == kWords) sort_list<MODE, 1>(f, s, t, gt, g, (int)tile, rg.x, n, -1);
-        } else if (n <= 128) {
-            sort_list<MODE, 4>(f, s, t, gt, g, (int)tile, rg.x, n, -1);
+            if (r) dst = r & 1;   // the merge rounds alternate between the buffers and end in the first
+            tile = q.x;
+            c0 = rg.x + first;
+            n = min(kSortCap, L - first);
         } else {
-            sort_list<MODE, kSortVT>(f, s, t, gt, g, (int)tile, rg.x, n, -1);
+            u -= n_chunks;
+            int c = kSortClasses - 1;
+            for (; c >= 0; --c) {
+                const int per = 16 >> (c > 0 ? c - 1 : 0);
+                const unsigned units = (plan->count[c] + per - 1) / per;
+                if (u < units) break;
+                u -= units;
+            }
+            if (c < 0) return;
+            gt = 32 << (c > 0 ? c - 1 : 0);
+            const unsigned e = u * (kSortThreads / gt) + threadIdx.x / gt;
+            if (e >= plan->count[c]) continue;
+            tile = f.order[plan->first[c] + e].x;
+            const uint2 rg = f.ranges[tile];
+            if (!SVR_IN_BOUNDS(f.debug, kDbgRange, rg.y, f.capacity + 1)) continue;
+            c0 = rg.x;
+            n = (int)(rg.y - rg.x);
+            if (n > gt * kSortVT) continue;   // not reached: the class's longest list fits
+        }
+        const int g = threadIdx.x / gt, t = threadIdx.x & (gt - 1);
+        uint64_t *s = smem + (size_t)g * (gt / 16 * 17 * kSortVT);
+        // as few words per thread as hold the list: a class's lists are half
+        // to wholly as long as its longest, a long list's last chunk may be
+        // short
+        if (n <= gt) {
+            if (n > 1 || MODE == kWords || dst >= 0) sort_list<MODE, 1>(f, s, t, gt, g, (int)tile, c0, n, dst);
+        } else if (n <= 4 * gt) {
+            sort_list<MODE, 4>(f, s, t, gt, g, (int)tile, c0, n, dst);
+        } else if (n <= 8 * gt) {
+            sort_list<MODE, 8>(f, s, t, gt, g, (int)tile, c0, n, dst);
+        } else if (n <= 12 * gt) {
+            sort_list<MODE, 12>(f, s, t, gt, g, (int)tile, c0, n, dst);
+        } else {
+            sort_list<MODE, kSortVT>(f, s, t, gt, g, (int)tile, c0, n, dst);
         }
     }
 }
