@@ -65,9 +65,10 @@ Layout make_layout(int64_t n_vox, int n_views, int64_t cap, int64_t ntiles, int 
     take(kOctpath, 8 * N);
     take(kRect, 8 * VN);
     take(kCount, 4 * VN);
-    take(kTileCount, 4 * 2 * svr::kTileSub * (size_t)ntiles);
+    const size_t subs = (size_t)ntiles << svr::tile_sub_log2(ntiles);
+    take(kTileCount, 4 * 2 * subs);
     take(kRecord, sizeof(svr::Record) * VN);
-    take(kScanBlocks, 4 * (((size_t)ntiles * svr::kTileSub + svr::kScanTile - 1) / svr::kScanTile + 1));
+    take(kScanBlocks, 4 * ((subs + svr::kScanTile - 1) / svr::kScanTile + 1));
     take(kKeys0, 8 * C);
     take(kKeys1, 8 * C);
     take(kVals0, 4 * C);
@@ -173,6 +174,7 @@ svr::FrameDev frame_dev(const svr_frame *f) {
     memset(&d, 0, sizeof(d));
     d.n_views = f->n_views;
     d.total_tiles = (int)f->total_tiles;
+    d.sub_log2 = svr::tile_sub_log2(f->total_tiles);
     d.key_shift = f->key_shift;
     for (int v = 0; v < f->n_views; ++v) {
         const svr_camera &c = f->cams[v];
@@ -202,7 +204,7 @@ svr::FrameDev frame_dev(const svr_frame *f) {
     d.rect = (short4 *)(ws + o[kRect]);
     d.count = (uint32_t *)(ws + o[kCount]);
     d.tile_cnt = (uint32_t *)(ws + o[kTileCount]);
-    d.cursor = d.tile_cnt + (size_t)svr::kTileSub * f->total_tiles;
+    d.cursor = d.tile_cnt + ((size_t)f->total_tiles << d.sub_log2);
     d.rec = (svr::Record *)(ws + o[kRecord]);
     d.box = (ushort4 *)(ws + o[kBox]);
     d.scan_blocks = (uint32_t *)(ws + o[kScanBlocks]);

@@ -13,7 +13,7 @@
 //                 one thread per voxel, reading its densities and SH once
 //   k_scan_*      exclusive scan of the tiles' pair counts (block sums, then
 //                 each block scans its part after summing the earlier blocks;
-//                 kTileSub sub-buckets per tile, adjacent): each sub-bucket's
+//                 the sub-buckets of a tile are adjacent): each sub-bucket's
 //                 start, each tile's range and segments, the work order's
 //                 group counts, the total, the capacity check
 //   k_emit        writes each (voxel, tile, sign pattern s) pair into its
@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(kMaskThreads) k_tile_mask(FrameDev f) {
     const int lane = threadIdx.x & 31;
     const int n_threads = gridDim.x * kMaskThreads, n_warps = n_threads / 32;
     const int warp = blockIdx.x * (kMaskThreads / 32) + (threadIdx.x >> 5);
-    for (int64_t i = blockIdx.x * kMaskThreads + threadIdx.x; i < (int64_t)kTileSub * f.total_tiles; i += n_threads)
+    for (int64_t i = blockIdx.x * kMaskThreads + threadIdx.x; i < ((int64_t)f.total_tiles << f.sub_log2); i += n_threads)
         f.tile_cnt[i] = 0u;
     const int B = f.blocks_per_tile;
     for (int base = 0; base + warp < f.total_tiles; base += 8 * n_warps) {
@@ -261,7 +261,7 @@ __device__ __forceinline__ uint32_t count_pairs(const FrameDev &f, const DevCam 
     const int lane = threadIdx.x & 31;
     const uint8_t *mask = f.tile_mask + cam.tile_base;
     uint32_t *cnt = f.tile_cnt + cam.tile_base;
-    const int sub = (int)(v & (kTileSub - 1));
+    const int sub = (int)(v & ((1 << f.sub_log2) - 1));
     const bool coop = rect_tiles(rc) > kCoopTiles;
     uint32_t n = 0;
     if (!coop) {
@@ -465,10 +465,10 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t x, uint32_t *w
     return wpre + inc - x;
 }
 
-// Scan position i is sub-bucket i % kTileSub of tile i / kTileSub, stored
+// Scan position i is sub-bucket i mod 2^sub_log2 of tile i / 2^sub_log2, stored
 // sub-bucket-major (count[sub * ntiles + tile]).
-__device__ __forceinline__ int64_t sub_index(int64_t i, int64_t ntiles) {
-    return (i % kTileSub) * ntiles + i / kTileSub;
+__device__ __forceinline__ int64_t sub_index(const FrameDev &f, int64_t i) {
+    return (i & ((1 << f.sub_log2) - 1)) * (int64_t)f.total_tiles + (i >> f.sub_log2);
 }
 
 // Also clears the counters of the work order and the sort for k_scan_down.
@@ -478,9 +478,9 @@ __global__ void __launch_bounds__(256) k_scan_reduce(FrameDev f) {
         for (int i = threadIdx.x; i < (int)(sizeof(SortPlan) / 4); i += 256) reinterpret_cast<unsigned *>(f.plan)[i] = 0u;
         if (threadIdx.x == 0) f.status->slots_used = 0;
     }
-    const int64_t ntiles = f.total_tiles, n = ntiles * kTileSub;
+    const int64_t n = (int64_t)f.total_tiles << f.sub_log2;
     const int64_t i = (int64_t)blockIdx.x * kScanTile + threadIdx.x;
-    const uint64_t acc = i < n ? f.tile_cnt[sub_index(i, ntiles)] : 0u;
+    const uint64_t acc = i < n ? f.tile_cnt[sub_index(f, i)] : 0u;
     uint32_t tot;
     // a block sum beyond 2^32 saturates; the capacity check on the 64-bit
     // total catches it
@@ -525,17 +525,18 @@ __global__ void __launch_bounds__(256) k_scan_down(FrameDev f, int nb) {
         all += wall[w];
     }
     const bool over = all > (unsigned long long)f.capacity;
-    const int64_t ntiles = f.total_tiles, n = ntiles * kTileSub;
+    const int64_t n = (int64_t)f.total_tiles << f.sub_log2;
     const int64_t i = (int64_t)blockIdx.x * kScanTile + t;
-    const uint32_t x = i < n ? f.tile_cnt[sub_index(i, ntiles)] : 0u;
+    const uint32_t x = i < n ? f.tile_cnt[sub_index(f, i)] : 0u;
     uint32_t tot;
     const uint32_t ex = block_exclusive_scan(x, ws, tot);
     const uint32_t c = (uint32_t)tmin<unsigned long long>(pre + ex, 0xFFFFFFFFull);
     const uint32_t e = (uint32_t)tmin<unsigned long long>(pre + ex + x, 0xFFFFFFFFull);
-    if (i < n) f.cursor[sub_index(i, ntiles)] = c;
-    // the kTileSub lanes of a tile: the first one takes the tile
-    const uint32_t end = __shfl_sync(0xffffffffu, e, lane | (kTileSub - 1));
-    const bool tile = i < n && i % kTileSub == 0;
+    if (i < n) f.cursor[sub_index(f, i)] = c;
+    // the lanes of a tile's sub-buckets: the first one takes the tile
+    const int last_sub = (1 << f.sub_log2) - 1;
+    const uint32_t end = __shfl_sync(0xffffffffu, e, lane | last_sub);
+    const bool tile = i < n && (i & last_sub) == 0;
     const uint2 r = over || end == c ? make_uint2(0u, 0u) : make_uint2(c, end);
     const unsigned len = r.y - r.x;
     unsigned nseg = len > (unsigned)kSegLen ? (len + kSegLen - 1) / kSegLen : 1u, base = 0;
@@ -555,8 +556,8 @@ __global__ void __launch_bounds__(256) k_scan_down(FrameDev f, int nb) {
         } else {
             atomicAdd(&group_cnt[bk], 1u);
         }
-        f.ranges[i / kTileSub] = r;
-        f.tile_seg[i / kTileSub] = make_uint2(nseg, base);
+        f.ranges[i >> f.sub_log2] = r;
+        f.tile_seg[i >> f.sub_log2] = make_uint2(nseg, base);
     }
     __syncthreads();
     if (t < 2 * kOrderGroups && group_cnt[t]) atomicAdd(&f.plan->cnt[t], group_cnt[t]);
@@ -606,7 +607,7 @@ __global__ void __launch_bounds__(kEmitThreads) k_emit(FrameDev f) {
         rc = f.rect[iv];
         code = f.octpath[v];
     }
-    const int sub = (int)(v & (kTileSub - 1));
+    const int sub = (int)(v & ((1 << f.sub_log2) - 1));
     uint32_t *cur = f.cursor + (size_t)sub * f.total_tiles;
     const bool coop = rect_tiles(rc) > kCoopTiles;
     // the rectangle's tiles in row-major batches of kEmitBatch: a batch's
@@ -677,8 +678,7 @@ cudaError_t launch_preprocess(const FrameDev &f, cudaStream_t s) {
 }
 
 cudaError_t launch_scan(const FrameDev &f, cudaStream_t s) {
-    const int64_t T = f.total_tiles;
-    const int nb = (int)((T * kTileSub + kScanTile - 1) / kScanTile);
+    const int nb = (int)((((int64_t)f.total_tiles << f.sub_log2) + kScanTile - 1) / kScanTile);
     static_assert(kScanTile == 256, "one entry per thread");
     k_scan_reduce<<<nb, 256, 0, s>>>(f);
     k_scan_down<<<nb, 256, 0, s>>>(f, nb);

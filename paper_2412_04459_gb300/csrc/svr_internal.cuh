@@ -30,10 +30,16 @@ constexpr int kScanTile = 256;             // entries per block of the count sca
 // loss sums (11..13).
 constexpr int kSegLen = 1024;
 constexpr int kSegFields = 14;
-// A tile's pairs are counted and emitted through kTileSub sub-buckets (by
-// voxel id), so that the atomics on a busy tile spread over separate cache
-// lines; the sub-buckets of a tile are adjacent in its range.
-constexpr int kTileSub = 8;
+// A tile's pairs are counted and emitted through sub-buckets (by voxel id), so
+// that the atomics on a busy tile spread over separate cache lines; the
+// sub-buckets of a tile are adjacent in its range.  Fewer tiles are busier,
+// and the scan's cost grows with all of them: 32 up to 8192 tiles (emission of
+// a 2M-voxel preview over 280 tiles 99 -> 60 us against 8, 1M voxels over
+// 4,240 tiles 33.8 -> 32.5 us), 16 up to 131,072 (16 mixed views, 75,080 tiles:
+// 547 -> 497 us), else 8.
+__host__ __device__ __forceinline__ int tile_sub_log2(int64_t ntiles) {
+    return ntiles <= 8192 ? 5 : ntiles <= 131072 ? 4 : 3;
+}
 
 // A tile list up to kSortCap pairs is sorted by one group of threads in shared
 // memory; a longer one as chunks of at most kSortCap pairs, merged afterwards.
@@ -293,6 +299,7 @@ struct FrameDev {
     DevCam views[kMaxViews];
     int n_views;
     int total_tiles;         // sum of the views' tile counts
+    int sub_log2;            // log2 of a tile's sub-buckets
     int key_shift;           // Morton bits kept in the key; the tile id sits above them
     Status *status;
     uint8_t *tile_mask;      // [total_tiles]
@@ -300,11 +307,11 @@ struct FrameDev {
     uint64_t *octpath;       // [N]
     short4 *rect;            // [V * N] tile rectangle tx0, tx1, ty0, ty1
     uint32_t *count;         // [V * N] pairs of each (view, voxel)
-    uint32_t *tile_cnt;      // [kTileSub][total_tiles] pairs of each tile's sub-buckets (k_preprocess)
-    uint32_t *cursor;        // [kTileSub][total_tiles] next free slot of each sub-bucket
+    uint32_t *tile_cnt;      // [2^sub_log2][total_tiles] pairs of each tile's sub-buckets (k_preprocess)
+    uint32_t *cursor;        // [2^sub_log2][total_tiles] next free slot of each sub-bucket
     Record *rec;             // [V * N]
     ushort4 *box;            // [V * N] inclusive pixel range x0, x1, y0, y1 a hit can fall in
-    uint32_t *scan_blocks;   // [ceil(kTileSub total_tiles / kScanTile) + 1]
+    uint32_t *scan_blocks;   // [ceil(2^sub_log2 total_tiles / kScanTile) + 1]
     uint64_t *keys[2];
     uint32_t *vals[2];
     SortPlan *plan;
