@@ -51,6 +51,7 @@ constexpr int kMaskThreads = 128;
 constexpr int kMaskWarps = 4096;
 
 __global__ void __launch_bounds__(kMaskThreads) k_tile_mask(FrameDev f) {
+    begin_kernel();
     // also starts the frame: status cleared (no smallest invalid voxel yet)
     // and the tiles' pair counters zeroed, before k_preprocess counts
     if (blockIdx.x == 0 && threadIdx.x < sizeof(Status) / 4)
@@ -346,6 +347,7 @@ __device__ __forceinline__ void write_octpath(const FrameDev &f, int64_t v, int 
 // One view (grid.y = view): one thread per (view, voxel).  No thread leaves
 // before the pair count, which the warp takes together.
 __global__ void __launch_bounds__(128, 8) k_preprocess(FrameDev f) {
+    begin_kernel();
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const bool in = v < f.n_vox;
     const int view = blockIdx.y;
@@ -394,6 +396,7 @@ __global__ void __launch_bounds__(128, 8) k_preprocess(FrameDev f) {
 // records' colour words); then each view's projection, tile counts and the
 // rest of its record.
 __global__ void __launch_bounds__(128) k_preprocess_views(FrameDev f) {
+    begin_kernel();
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const bool in = v < f.n_vox;
     float c0 = 0.f, c1 = 0.f, c2 = 0.f, vs = 0.f;
@@ -473,6 +476,7 @@ __device__ __forceinline__ int64_t sub_index(const FrameDev &f, int64_t i) {
 
 // Also clears the counters of the work order and the sort for k_scan_down.
 __global__ void __launch_bounds__(256) k_scan_reduce(FrameDev f) {
+    begin_kernel();
     __shared__ uint32_t ws[8];
     if (blockIdx.x == 0) {
         for (int i = threadIdx.x; i < (int)(sizeof(SortPlan) / 4); i += 256) reinterpret_cast<unsigned *>(f.plan)[i] = 0u;
@@ -496,6 +500,7 @@ __global__ void __launch_bounds__(256) k_scan_reduce(FrameDev f) {
 // ranges are empty).  A start beyond 2^32 saturates; the capacity flag covers
 // it.
 __global__ void __launch_bounds__(256) k_scan_down(FrameDev f, int nb) {
+    begin_kernel();
     __shared__ uint32_t ws[8];
     __shared__ unsigned long long wpre[8], wall[8];
     __shared__ unsigned group_cnt[2 * kOrderGroups], slots, slot0;
@@ -596,6 +601,7 @@ __device__ __forceinline__ void write_pairs(const FrameDev &f, int g, unsigned m
 
 // grid.y = view.  A voxel over more than kCoopTiles tiles is left to the warp.
 __global__ void __launch_bounds__(kEmitThreads) k_emit(FrameDev f) {
+    begin_kernel();
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (f.status->flags & SVR_FLAG_CAPACITY) return;   // not raised here while the pairs fit
     const int view = blockIdx.y, lane = threadIdx.x & 31;
@@ -663,34 +669,26 @@ __global__ void __launch_bounds__(kEmitThreads) k_emit(FrameDev f) {
 
 cudaError_t launch_tile_mask(const FrameDev &f, cudaStream_t s) {
     const int warps = tmin(f.total_tiles, kMaskWarps), per = kMaskThreads / 32;
-    k_tile_mask<<<(unsigned)((warps + per - 1) / per), kMaskThreads, 0, s>>>(f);
-    return cudaGetLastError();
+    return launch(k_tile_mask, dim3((unsigned)((warps + per - 1) / per)), kMaskThreads, 0, s, f);
 }
 
 cudaError_t launch_preprocess(const FrameDev &f, cudaStream_t s) {
     if (f.n_vox == 0) return cudaSuccess;
-    if (f.n_views == 1) {
-        k_preprocess<<<(unsigned)((f.n_vox + 127) / 128), 128, 0, s>>>(f);
-    } else {
-        k_preprocess_views<<<(unsigned)((f.n_vox + 127) / 128), 128, 0, s>>>(f);
-    }
-    return cudaGetLastError();
+    return launch(f.n_views == 1 ? k_preprocess : k_preprocess_views, dim3((unsigned)((f.n_vox + 127) / 128)), 128, 0, s,
+                  f);
 }
 
 cudaError_t launch_scan(const FrameDev &f, cudaStream_t s) {
     const int nb = (int)((((int64_t)f.total_tiles << f.sub_log2) + kScanTile - 1) / kScanTile);
     static_assert(kScanTile == 256, "one entry per thread");
-    k_scan_reduce<<<nb, 256, 0, s>>>(f);
-    k_scan_down<<<nb, 256, 0, s>>>(f, nb);
-    return cudaGetLastError();
+    const cudaError_t e = launch(k_scan_reduce, dim3(nb), 256, 0, s, f);
+    return e != cudaSuccess ? e : launch(k_scan_down, dim3(nb), 256, 0, s, f, nb);
 }
 
 cudaError_t launch_emit(const FrameDev &f, cudaStream_t s) {
-    if (f.n_vox > 0) {
-        const dim3 grid((unsigned)((f.n_vox + kEmitThreads - 1) / kEmitThreads), (unsigned)f.n_views);
-        k_emit<<<grid, kEmitThreads, 0, s>>>(f);
-    }
-    return cudaGetLastError();
+    if (f.n_vox == 0) return cudaSuccess;
+    const dim3 grid((unsigned)((f.n_vox + kEmitThreads - 1) / kEmitThreads), (unsigned)f.n_views);
+    return launch(k_emit, grid, kEmitThreads, 0, s, f);
 }
 
 }  // namespace svr

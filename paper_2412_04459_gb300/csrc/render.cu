@@ -339,6 +339,7 @@ __device__ __forceinline__ void block_lists_entry(const FrameDev &f, const uint3
 // A persistent grid of CTAs takes the work-order entries in turn (the count
 // is the device's).
 __global__ void __launch_bounds__(kListThreads) k_block_lists(FrameDev f, const uint32_t *__restrict__ vals) {
+    begin_kernel();
     __shared__ uint32_t sval[kListChunk];
     __shared__ uint32_t smsk[kListChunk];
     __shared__ uint32_t scnt[32];
@@ -1124,6 +1125,7 @@ __device__ __forceinline__ void fwd_item(const FrameDev &f, const Item &it, uint
 // kModeDist: the distortion loss alone (the training step's extra).
 template <int K, int MODE>
 __global__ void __launch_bounds__(kThreads, kFwdMinBlocks) k_render_fwd(FrameDev f, FwdOut out) {
+    begin_kernel();
     __shared__ FwdSmem smem[kWarps];
     FwdSmem &ws = smem[threadIdx.x >> 5];
     // the items, then the empty tiles (the last work-order entries), a tile
@@ -1162,6 +1164,7 @@ __global__ void __launch_bounds__(kThreads, kFwdMinBlocks) k_render_fwd(FrameDev
 // over the items, so each weight is the true T_i alpha_i.
 template <int K>
 __global__ void __launch_bounds__(kThreads, kFwdMinBlocks) k_render_maxw(FrameDev f, FwdOut out) {
+    begin_kernel();
     __shared__ FwdSmem smem[kWarps];
     FwdSmem &ws = smem[threadIdx.x >> 5];
     const unsigned n_items = f.status->n_listed * (unsigned)f.blocks_per_tile;
@@ -2042,8 +2045,7 @@ cudaError_t launch_block_lists(const FrameDev &f, int sorted_alt, cudaStream_t s
     const int64_t grid = (int64_t)f.total_tiles + f.seg_slots;
     static DeviceCache cache;
     const unsigned resident = device_cached(cache, [] { return persistent_grid(k_block_lists, kListThreads); });
-    k_block_lists<<<(unsigned)tmin<int64_t>(grid, resident), kListThreads, 0, s>>>(f, f.vals[sorted_alt]);
-    return cudaGetLastError();
+    return launch(k_block_lists, dim3((unsigned)tmin<int64_t>(grid, resident)), kListThreads, 0, s, f, f.vals[sorted_alt]);
 }
 
 // Bound on the render items: every tile's blocks, and those of the segments
@@ -2061,8 +2063,7 @@ static cudaError_t fwd_k(const FrameDev &f, const FwdOut &out, cudaStream_t s) {
     const unsigned grid = device_cached(cache, [] { return persistent_grid(k_render_fwd<K, MODE>, kThreads); });
     const int64_t items = max_items(f);
     const unsigned g = (unsigned)tmin<int64_t>(grid, (items + kWarps - 1) / kWarps);
-    k_render_fwd<K, MODE><<<g, kThreads, 0, s>>>(f, out);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch(k_render_fwd<K, MODE>, dim3(g), kThreads, 0, s, f, out);
     if (e != cudaSuccess || MODE != kModeExtra || !out.max_weight) return e;
     // the later segments of split lists, from their true transmittance
     static DeviceCache cache_w;
@@ -2072,8 +2073,8 @@ static cudaError_t fwd_k(const FrameDev &f, const FwdOut &out, cudaStream_t s) {
     FwdOut wout = out;
     wout.normal = nullptr;
     wout.dist = nullptr;
-    k_render_maxw<K><<<(unsigned)tmin<int64_t>(grid_w, (items + kWarps - 1) / kWarps), kThreads, 0, s>>>(f, wout);
-    return cudaGetLastError();
+    return launch(k_render_maxw<K>, dim3((unsigned)tmin<int64_t>(grid_w, (items + kWarps - 1) / kWarps)), kThreads, 0, s, f,
+                  wout);
 }
 
 template <int K, int XM>

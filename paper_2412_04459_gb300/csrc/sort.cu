@@ -38,6 +38,7 @@ constexpr int kOrderThreads = 256;
 // 4,240 tiles of a 1280 x 840 view and 118 us for 115,200 tiles.  CTA 0 also
 // writes the queue's counts and the sort classes.
 __global__ void __launch_bounds__(kOrderThreads) k_order(FrameDev f) {
+    begin_kernel();
     constexpr int G = 2 * kOrderGroups;
     __shared__ unsigned cnt[G], start[G], mine[G];
     const int t = threadIdx.x, i = blockIdx.x * kOrderThreads + t;
@@ -264,6 +265,7 @@ __device__ __forceinline__ void sort_list(const FrameDev &f, uint64_t *s, int t,
 // the short ones fill the tail.
 template <int MODE>
 __global__ void __launch_bounds__(kSortThreads, 2) k_sort_lists(FrameDev f) {
+    begin_kernel();
     extern __shared__ __align__(16) unsigned char dyn[];
     uint64_t *smem = reinterpret_cast<uint64_t *>(dyn);
     __shared__ unsigned unit;
@@ -373,6 +375,7 @@ __device__ __forceinline__ int merge_split(const uint64_t *ak, const uint32_t *a
 // lists of up to 90,564.
 template <bool WORDS>
 __global__ void __cluster_dims__(kMergeCluster, 1, 1) __launch_bounds__(kMergeThreads, 2) k_merge_long(FrameDev f) {
+    begin_kernel();
     __shared__ uint64_t sk[kPiece / 16 * 17];
     __shared__ uint32_t sv[WORDS ? 1 : kPiece];
     __shared__ int split[2];
@@ -469,8 +472,7 @@ static unsigned sm_count() {
 }
 
 cudaError_t launch_order(const FrameDev &f, cudaStream_t s) {
-    k_order<<<(unsigned)((f.total_tiles + kOrderThreads - 1) / kOrderThreads), kOrderThreads, 0, s>>>(f);
-    return cudaGetLastError();
+    return launch(k_order, dim3((unsigned)((f.total_tiles + kOrderThreads - 1) / kOrderThreads)), kOrderThreads, 0, s, f);
 }
 
 template <int MODE>
@@ -491,15 +493,13 @@ static cudaError_t sort_lists(const FrameDev &f, cudaStream_t s) {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sort_lists<MODE>, kSortThreads, kSortSmemBytes);
         return sm_count() * (unsigned)(per_sm > 0 ? per_sm : 1);
     });
-    k_sort_lists<MODE><<<(unsigned)tmin<int64_t>(units, resident), kSortThreads, kSortSmemBytes, s>>>(f);
-    e = cudaGetLastError();
+    e = launch(k_sort_lists<MODE>, dim3((unsigned)tmin<int64_t>(units, resident)), kSortThreads, kSortSmemBytes, s, f);
     // no list can be longer than every voxel with every sign pattern
     if (e != cudaSuccess || f.capacity <= kSortCap || 8 * f.n_vox <= kSortCap) return e;
     // clusters: one per possible long list, at most two CTAs per SM
     const int64_t lists = f.capacity / kSortCap;
     const unsigned clusters = (unsigned)tmin<int64_t>(lists, tmin<int64_t>(f.total_tiles, sm_count() / (kMergeCluster / 2)));
-    k_merge_long<MODE == kWords><<<(clusters ? clusters : 1u) * kMergeCluster, kMergeThreads, 0, s>>>(f);
-    return cudaGetLastError();
+    return launch(k_merge_long<MODE == kWords>, dim3((clusters ? clusters : 1u) * kMergeCluster), kMergeThreads, 0, s, f);
 }
 
 cudaError_t launch_tile_sort(const FrameDev &f, cudaStream_t s) {

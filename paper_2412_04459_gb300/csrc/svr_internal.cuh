@@ -409,6 +409,37 @@ unsigned device_cached(DeviceCache &c, F compute) {
     return x;
 }
 
+// Programmatic dependent launch: a kernel launched with launch() may start
+// while the stream's kernel before it still runs; it first lets the next one
+// do the same and then waits for all of the kernel before (and so, that one
+// having waited too, for everything before it), before it reads or writes
+// memory.  So the ten kernels from the tile masks to the forward do not wait
+// for one another's launch: 742 -> 718 us for the 1M-voxel step, 183 -> 174 us
+// for the smallest view.  The backward's kernels are launched plainly: with
+// them the step took 773 us.  Nor do the kernels of a large batch gain (16
+// mixed views, 75,080 tiles: 8.34 ms without, 8.37 with).
+constexpr int kOverlapTiles = 16384;
+
+__device__ __forceinline__ void begin_kernel() {
+    asm volatile("griddepcontrol.launch_dependents;\ngriddepcontrol.wait;" ::: "memory");
+}
+
+template <class... Params, class... Args>
+cudaError_t launch(void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s,
+                   const FrameDev &f, Args... args) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = f.total_tiles <= kOverlapTiles ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, f, args...);
+}
+
 // Records a printf-style message for svr_last_error() and returns code.
 int set_error(int code, const char *fmt, ...);
 
