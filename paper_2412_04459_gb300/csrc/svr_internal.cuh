@@ -78,7 +78,7 @@ struct Status {
     unsigned n_pairs_hi;
     int bad_voxel;        // smallest invalid voxel id (all bits set: none)
     unsigned fwd_next;    // next work item of the forward render (the last warp of a launch resets it)
-    unsigned bwd_next;    // next work item of the backward render (reset before each launch)
+    unsigned bwd_next;    // next work item of the backward render (k_grid_bwd resets it)
     unsigned n_queue;     // (tile, segment) entries of the render work order
     unsigned slots_used;  // segment slots taken by the split tiles
     unsigned fwd_done;    // bit 0: a forward filled the segment sums of the current sort; bit 1: with
