@@ -331,7 +331,6 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_sort_lists(FrameDev f) {
 
 // ------------------------------------------------------------ long lists
 
-constexpr int kMergeCluster = 8;
 constexpr int kMergeThreads = 512;
 constexpr int kMergeVT = 8;
 constexpr int kPiece = kMergeThreads * kMergeVT;   // outputs merged at a time by a CTA
@@ -367,23 +366,23 @@ __device__ __forceinline__ int merge_split(const uint64_t *ak, const uint32_t *a
 
 // Lists of more than kSortCap pairs: their sorted chunks are merged pairwise
 // in rounds between the two buffers, the last round into the first.  A
-// cluster of eight CTAs takes one list at a time; a round's outputs are cut
+// cluster takes one list at a time; a round's outputs are cut
 // into pieces of 4096, each merged in shared memory by one CTA (two searches
 // for its ends, coalesced loads and stores), and the cluster barrier
 // separates the rounds.  One CTA per list, merging in global memory by
 // itself, took 48 us for a single list of 8,714 pairs and 3.1 ms for 46
 // lists of up to 90,564.
-template <bool WORDS>
-__global__ void __cluster_dims__(kMergeCluster, 1, 1) __launch_bounds__(kMergeThreads, 2) k_merge_long(FrameDev f) {
+template <bool WORDS, int CLUSTER>
+__global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(kMergeThreads, 2) k_merge_long(FrameDev f) {
     begin_kernel();
     __shared__ uint64_t sk[kPiece / 16 * 17];
     __shared__ uint32_t sv[WORDS ? 1 : kPiece];
     __shared__ int split[2];
     const int t = threadIdx.x, warp = t >> 5;
-    const int rank = (int)(blockIdx.x % kMergeCluster);
+    const int rank = (int)(blockIdx.x % CLUSTER);
     const unsigned n_huge = f.plan->n_huge;
     const Less<kWords> less = {nullptr};
-    for (unsigned e = blockIdx.x / kMergeCluster; e < n_huge; e += gridDim.x / kMergeCluster) {
+    for (unsigned e = blockIdx.x / CLUSTER; e < n_huge; e += gridDim.x / CLUSTER) {
         const unsigned tile = f.order[e].x;
         const uint2 rg = f.ranges[tile];
         if (!SVR_IN_BOUNDS(f.debug, kDbgRange, rg.y, f.capacity + 1)) continue;   // the whole cluster alike
@@ -395,7 +394,7 @@ __global__ void __cluster_dims__(kMergeCluster, 1, 1) __launch_bounds__(kMergeTh
             const uint64_t *k0 = f.keys[src] + rg.x;
             const uint32_t *v0 = f.vals[src] + rg.x;
             const int64_t w = (int64_t)kSortCap << r;
-            for (int64_t o = (int64_t)rank * kPiece; o < L; o += (int64_t)kMergeCluster * kPiece) {
+            for (int64_t o = (int64_t)rank * kPiece; o < L; o += (int64_t)CLUSTER * kPiece) {
                 const int64_t p0 = o / (2 * w) * (2 * w);
                 const int64_t mid = tmin<int64_t>(L, p0 + w), end = tmin<int64_t>(L, p0 + 2 * w);
                 const int na = (int)(mid - p0), nb = (int)(end - mid);
@@ -475,6 +474,20 @@ cudaError_t launch_order(const FrameDev &f, cudaStream_t s) {
     return launch(k_order, dim3((unsigned)((f.total_tiles + kOrderThreads - 1) / kOrderThreads)), kOrderThreads, 0, s, f);
 }
 
+// Clusters: one per possible long list, at most two CTAs per SM.  Few tiles
+// make few and longer lists, which take eight CTAs each (a preview of 280
+// tiles: 71 us, 133 with four); many tiles make many lists of two or three
+// chunks, whose rounds have work for fewer (8 x 2560x1440 views: 555 us with
+// eight CTAs, 292 with four, 189 with two; 16 mixed views: 113, 61 and 56).
+constexpr int kFewTiles = 8192;
+
+template <bool WORDS, int CLUSTER>
+static cudaError_t merge_long(const FrameDev &f, cudaStream_t s) {
+    const int64_t lists = tmin<int64_t>(f.capacity / kSortCap, f.total_tiles);
+    const unsigned clusters = (unsigned)tmin<int64_t>(lists > 0 ? lists : 1, 2 * sm_count() / CLUSTER);
+    return launch(k_merge_long<WORDS, CLUSTER>, dim3(clusters * CLUSTER), kMergeThreads, 0, s, f);
+}
+
 template <int MODE>
 static cudaError_t sort_lists(const FrameDev &f, cudaStream_t s) {
     // at most one CTA per possible unit, at most as many as are resident at
@@ -496,10 +509,7 @@ static cudaError_t sort_lists(const FrameDev &f, cudaStream_t s) {
     e = launch(k_sort_lists<MODE>, dim3((unsigned)tmin<int64_t>(units, resident)), kSortThreads, kSortSmemBytes, s, f);
     // no list can be longer than every voxel with every sign pattern
     if (e != cudaSuccess || f.capacity <= kSortCap || 8 * f.n_vox <= kSortCap) return e;
-    // clusters: one per possible long list, at most two CTAs per SM
-    const int64_t lists = f.capacity / kSortCap;
-    const unsigned clusters = (unsigned)tmin<int64_t>(lists, tmin<int64_t>(f.total_tiles, sm_count() / (kMergeCluster / 2)));
-    return launch(k_merge_long<MODE == kWords>, dim3((clusters ? clusters : 1u) * kMergeCluster), kMergeThreads, 0, s, f);
+    return f.total_tiles <= kFewTiles ? merge_long<MODE == kWords, 8>(f, s) : merge_long<MODE == kWords, 2>(f, s);
 }
 
 cudaError_t launch_tile_sort(const FrameDev &f, cudaStream_t s) {

@@ -44,3 +44,21 @@ def test_list_lengths(n, level):
     fr, out, ins = run_gpu(scene, cam)
     assert ins["n_pairs"] == n
     compare_integers(scene, cam, ins)
+
+
+# eyes whose view holds the cells in its middle tile and not the far cells
+EYES = {10: (-1.2, -1.1, -1.4), 15: (0.85, 0.2, 0.2)}
+
+
+@pytest.mark.parametrize("n", (8193, 16385, 40001))
+@pytest.mark.parametrize("level", sorted(EYES))
+def test_long_list_among_many_tiles(n, level):
+    """Images of more than 8192 tiles merge their long lists with smaller
+    clusters."""
+    require_gpu()
+    scene = lattice_scene(n, level, n + level)
+    # 91 x 91 tiles, the cells a few pixels wide
+    cam = synth.look_at(EYES[level], (0.5, 0.5, 0.5), (0.0, 1.0, 0.0), 150.0, 1456, 1456)
+    fr, out, ins = run_gpu(scene, cam)
+    assert (ins["ranges"][:, 1].astype(np.int64) - ins["ranges"][:, 0]).max() == n
+    compare_integers(scene, cam, ins)
