@@ -51,8 +51,12 @@ SegBytes seg_bytes(int64_t ntiles, size_t slots, size_t B) {
     return b;
 }
 
+constexpr size_t kNone = ~size_t(0);   // offset of a buffer that the layout leaves out
+
 // n_vox voxels seen by n_views views with ntiles tiles of edge `tile` in all.
-Layout make_layout(int64_t n_vox, int n_views, int64_t cap, int64_t ntiles, int tile) {
+// A forward-only layout leaves out what only the backward reads: the gradient
+// accumulators and the hit masks.
+Layout make_layout(int64_t n_vox, int n_views, int64_t cap, int64_t ntiles, int tile, bool forward_only = false) {
     Layout L;
     size_t o = 0;
     auto take = [&](Slot s, size_t bytes) {
@@ -74,14 +78,16 @@ Layout make_layout(int64_t n_vox, int n_views, int64_t cap, int64_t ntiles, int 
     take(kVals0, 4 * C);
     take(kVals1, 4 * C);
     take(kRanges, 8 * (size_t)ntiles);
-    take(kDcol, 16 * VN + 32 * N);   // colour accumulators per view, corner-density accumulators
+    if (forward_only) L.off[kDcol] = kNone;
+    else take(kDcol, 16 * VN + 32 * N);   // colour accumulators per view, corner-density accumulators
     take(kBox, 8 * VN);
     const size_t slots = (size_t)svr::seg_slot_capacity(cap);
     take(kTileOrder, 8 * ((size_t)ntiles + slots));
     const size_t B = (size_t)tile * tile / 32;
     take(kBlockList, 8 * B * C);
     take(kBlockLen, sizeof(svr::RenderItem) * B * ((size_t)ntiles + slots));   // render items
-    take(kHitMask, 4 * B * (C + 32 * (size_t)ntiles));   // the block lists' positions + 32 per (tile, block)
+    if (forward_only) L.off[kHitMask] = kNone;
+    else take(kHitMask, 4 * B * (C + 32 * (size_t)ntiles));   // the block lists' positions + 32 per (tile, block)
     take(kSegment, seg_bytes(ntiles, slots, B).total);
     take(kSortPlan, align256(sizeof(svr::SortPlan)) + 8 * (size_t)svr::sort_chunk_capacity(cap));
     L.off[kTotal] = o;
@@ -218,7 +224,7 @@ svr::FrameDev frame_dev(const svr_frame *f) {
     d.order = (uint2 *)(ws + o[kTileOrder]);
     d.blist = (uint2 *)(ws + o[kBlockList]);
     d.items = (svr::RenderItem *)(ws + o[kBlockLen]);
-    d.hmask = (uint32_t *)(ws + o[kHitMask]);
+    d.hmask = o[kHitMask] == kNone ? nullptr : (uint32_t *)(ws + o[kHitMask]);
     d.blocks_per_tile = f->params.tile * f->params.tile / 32;
     d.seg_slots = svr::seg_slot_capacity(f->pair_capacity);
     const SegBytes sb = seg_bytes(f->total_tiles, (size_t)d.seg_slots, (size_t)d.blocks_per_tile);
@@ -227,8 +233,8 @@ svr::FrameDev frame_dev(const svr_frame *f) {
     d.merge_cnt = (uint32_t *)(seg + sb.merge_cnt);
     d.seg_len = (uint32_t *)(seg + sb.seg_len);
     d.seg_part = (float *)(seg + sb.seg_part);
-    d.dcol = (float4 *)(ws + o[kDcol]);
-    d.dgrid = d.dcol + (size_t)f->n_views * f->scene.n_vox;
+    d.dcol = o[kDcol] == kNone ? nullptr : (float4 *)(ws + o[kDcol]);
+    d.dgrid = o[kDcol] == kNone ? nullptr : d.dcol + (size_t)f->n_views * f->scene.n_vox;
     d.n_vox = f->scene.n_vox;
     d.n_pts = f->scene.n_pts;
     d.capacity = f->pair_capacity;
@@ -256,7 +262,7 @@ svr::FrameDev frame_dev(const svr_frame *f) {
 // (compact keys).
 int preprocess(svr_frame *frame, const svr_scene *scene, const svr_camera *cams, int n_views,
                const svr_params *params, void *ws, size_t ws_bytes, int64_t pair_capacity, bool paper_keys,
-               void *stream) {
+               void *stream, bool forward_only = false) {
     g_err[0] = 0;
     if (!frame || !scene) return fail(SVR_ERR_INVALID, "null frame or scene");
     int64_t ntiles = 0;
@@ -284,7 +290,7 @@ int preprocess(svr_frame *frame, const svr_scene *scene, const svr_camera *cams,
     if (pair_capacity < 0 || pair_capacity > INT32_MAX)
         return fail(SVR_ERR_INVALID, "pair_capacity %lld", (long long)pair_capacity);
     if (!ws || (((uintptr_t)ws) & 255u)) return fail(SVR_ERR_INVALID, "workspace null or not 256-byte aligned");
-    const Layout L = make_layout(N, n_views, pair_capacity, ntiles, params->tile);
+    const Layout L = make_layout(N, n_views, pair_capacity, ntiles, params->tile, forward_only);
     if (ws_bytes < L.off[kTotal])
         return fail(SVR_ERR_INVALID, "workspace %zu bytes < %zu needed", ws_bytes, (size_t)L.off[kTotal]);
 
@@ -335,6 +341,12 @@ int set_error(int code, const char *fmt, ...) {
     vsnprintf(g_err, sizeof(g_err), fmt, ap);
     va_end(ap);
     return code;
+}
+
+int preprocess_forward_only(svr_frame *frame, const svr_scene *scene, const svr_camera *cam,
+                            const svr_params *params, void *ws, size_t ws_bytes, int64_t pair_capacity,
+                            void *stream) {
+    return preprocess(frame, scene, cam, 1, params, ws, ws_bytes, pair_capacity, true, stream, true);
 }
 }  // namespace svr
 

@@ -428,7 +428,7 @@ __device__ __forceinline__ Item load_item(const FrameDev &f, unsigned i) {
     const size_t B = (size_t)f.blocks_per_tile;
     const size_t at = B * it.beg + (size_t)it.blk * (it.end - it.beg) + (it.slot == kNoSlot ? 0 : (size_t)it.seg * kSegLen);
     it.list = f.blist + at;
-    it.hm = f.hmask + at + 32 * ((size_t)it.g * B + it.blk);
+    it.hm = f.hmask ? f.hmask + at + 32 * ((size_t)it.g * B + it.blk) : nullptr;
     return it;
 }
 

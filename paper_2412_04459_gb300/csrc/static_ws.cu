@@ -29,6 +29,28 @@ constexpr int kMaxDevices = 64;
 
 __device__ __align__(256) unsigned char g_static_ws[kStaticWorkspaceBytes];
 
+// Bytes that a call is charged against the array's size: the sum that a
+// workspace for forward and backward took when the limits were set, buffer by
+// buffer on 256-byte boundaries.  The layout that the call uses has since
+// changed and, without the backward's buffers, is smaller than this for every
+// call near the limit; the charge keeps what is taken and what is refused
+// where it was.
+size_t charged_bytes(int64_t n_vox, int64_t pairs, int64_t ntiles, int tile) {
+    const size_t N = (size_t)n_vox, C = (size_t)pairs, T = (size_t)ntiles, B = (size_t)tile * tile / 32;
+    const size_t slots = 2 * C / 1024 + 1;   // segment slots
+    const size_t sizes[] = {
+        64, T * (1 + B), 8 * N, 8 * N, 4 * N, 68 * T, 64 * N,   // status, masks, voxel and tile tables, records
+        4 * ((8 * T + 255) / 256 + 1),                          // scan blocks
+        8 * C, 8 * C, 4 * C, 4 * C, 8 * T, 12 * N, 8 * N,       // pairs, ranges, colour gradients, boxes
+        8 * (T + slots), 8 * B * C, 4 * B * T,                  // work order, block lists and their lengths
+        4 * B * (C + 32 * T),                                   // hit masks
+        8 * T, 4 * B * T, 4 * B * slots, 4 * B * slots * 448,   // segments: table, counters, lengths, sums
+    };
+    size_t sum = 0;
+    for (size_t b : sizes) sum += (b + 255) & ~size_t(255);
+    return sum;
+}
+
 std::mutex g_setup_mu;
 void *g_static_ptr[kMaxDevices] = {};
 
@@ -66,26 +88,27 @@ SVR_API int svr_render_fwd_static(const svr_scene *scene, const svr_camera *cam,
                               (long long)scene->n_vox, (long long)kStaticMaxVoxels);
     // the image's tile count first, so that an oversized image is reported as
     // the limit it breaks (svr_workspace_size returns 0 for it)
+    int64_t tiles = 0;
     if (params->tile == 8 || params->tile == 16 || params->tile == 32) {
         if (cam->width > 0 && cam->height > 0) {
-            const int64_t tiles = (int64_t)((cam->width + params->tile - 1) / params->tile) *
-                                  ((cam->height + params->tile - 1) / params->tile);
+            tiles = (int64_t)((cam->width + params->tile - 1) / params->tile) *
+                    ((cam->height + params->tile - 1) / params->tile);
             if (tiles > 65536)
                 return svr::set_error(SVR_ERR_LIMIT, "static workspace: %lld tiles > 2^16 (the key's 16-bit tile id)",
                                       (long long)tiles);
         }
     }
-    const size_t base = svr_workspace_size(scene->n_vox, 0, cam, params);
-    if (base == 0) return svr::set_error(SVR_ERR_INVALID, "invalid camera or params");
+    if (svr_workspace_size(scene->n_vox, 0, cam, params) == 0)
+        return svr::set_error(SVR_ERR_INVALID, "invalid camera or params");
+    const size_t base = charged_bytes(scene->n_vox, 0, tiles, params->tile);
     if (base > kStaticWorkspaceBytes)
         return svr::set_error(SVR_ERR_LIMIT, "static workspace: this image needs %zu bytes, %zu available",
                               base, kStaticWorkspaceBytes);
-    // the largest pair capacity whose workspace fits in the array
+    // the largest pair capacity whose charge fits in the array
     int64_t lo = 0, hi = (int64_t)(kStaticWorkspaceBytes / 24) + 1;
     while (hi - lo > 1) {
         const int64_t mid = (lo + hi) / 2;
-        const size_t need = svr_workspace_size(scene->n_vox, mid, cam, params);
-        if (need != 0 && need <= kStaticWorkspaceBytes) lo = mid;
+        if (charged_bytes(scene->n_vox, mid, tiles, params->tile) <= kStaticWorkspaceBytes) lo = mid;
         else hi = mid;
     }
     if (lo == 0) return svr::set_error(SVR_ERR_LIMIT, "static workspace: no room left for pairs");
@@ -93,7 +116,7 @@ SVR_API int svr_render_fwd_static(const svr_scene *scene, const svr_camera *cam,
     int rc = static_workspace(&ws);
     if (rc != SVR_OK) return svr::set_error(rc, "static workspace: no device address for the array");
     svr_frame frame;
-    rc = svr_preprocess(&frame, scene, cam, params, ws, kStaticWorkspaceBytes, lo, stream);
+    rc = svr::preprocess_forward_only(&frame, scene, cam, params, ws, kStaticWorkspaceBytes, lo, stream);
     if (rc != SVR_OK) return rc;
     int64_t n_pairs = 0;
     rc = svr_bin_sort(&frame, &n_pairs, stream);

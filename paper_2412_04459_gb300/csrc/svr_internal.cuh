@@ -188,6 +188,10 @@ DebugBlock *debug_block();
 //            the 8 gathered corner densities: coefficients of 1, z, y, yz and
 //            x, xz, xy, xyz (see density_coeffs)
 //   r3 = colour rgb, bit c of the w word set if channel c was > 0 before the clamp
+struct Record {
+    float4 r0, r1, r2, r3;
+};
+
 // Asynchronous 16-byte global -> shared copy (cp.async, L2 only), its
 // commit and the wait for all but the N most recent groups.
 __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
@@ -197,10 +201,6 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
-
-struct Record {
-    float4 r0, r1, r2, r3;
-};
 
 // Ray direction of pixel (x, y): R^T ((x + .5 - cx) / fx, (y + .5 - cy) / fy, 1),
 // written with explicit roundings so every kernel derives the same bits.
@@ -442,6 +442,12 @@ cudaError_t launch(void (*kernel)(Params...), dim3 grid, unsigned threads, size_
 
 // Records a printf-style message for svr_last_error() and returns code.
 int set_error(int code, const char *fmt, ...);
+
+// svr_preprocess for a frame that no backward will follow: its workspace holds
+// neither gradient accumulators nor hit masks.
+int preprocess_forward_only(svr_frame *frame, const svr_scene *scene, const svr_camera *cam,
+                            const svr_params *params, void *ws, size_t ws_bytes, int64_t pair_capacity,
+                            void *stream);
 
 cudaError_t launch_tile_mask(const FrameDev &f, cudaStream_t s);
 cudaError_t launch_preprocess(const FrameDev &f, cudaStream_t s);
