@@ -575,9 +575,15 @@ __global__ void __launch_bounds__(256) k_scan_down(FrameDev f, int nb) {
 
 // --------------------------------------------------------------------- emit
 
-constexpr int kEmitBatch = 8;
-constexpr int kEmitCoop = 4;   // tiles per lane of a cooperative batch
-constexpr int kEmitThreads = 256;
+// Bound by the round trips of the counts, rectangles and atomics, so by the
+// warps that are resident: batches of four tiles take 48 registers, of eight
+// 58.  8 views of 8M voxels 1502 -> 1185 us, 16 mixed views 492 -> 430, one view
+// of 1M 45 -> 40 (batches of two: 1199, 438, 42); CTAs of 128 threads instead
+// of 256: 1158, 423, 39, and a camera inside the scene 77 -> 73.  32 registers
+// by launch bounds spill: 1440, 484, 50.
+constexpr int kEmitBatch = 4;
+constexpr int kEmitCoop = 4;   // tiles per lane of a cooperative batch (two: 1144 and 417, but 84 inside)
+constexpr int kEmitThreads = 128;
 
 // Writes the pairs of voxel v in tile g, whose sign patterns are m, from slot o.
 __device__ __forceinline__ void write_pairs(const FrameDev &f, int g, unsigned m, uint32_t o, uint64_t code,
