@@ -147,7 +147,7 @@ typedef struct svr_buffers {
     const int16_t *rect;      /* [V][N][4] tx0, tx1, ty0, ty1 (empty: tx0 > tx1) */
     const uint32_t *count;    /* [V][N] pairs emitted per (view, voxel) */
     const uint32_t *offset;   /* NULL: pairs are written per tile, not at per-voxel offsets */
-    const float *record;      /* [V][N][16] per-voxel record of each view */
+    const float *record;      /* [V][N][16] per-voxel record of each view: min corner and size, density polynomial, colour */
     const uint64_t *keys;     /* [pair_capacity] sorted keys: tile << key_shift | Morton order */
     const uint32_t *values;   /* [pair_capacity] sorted values: s << 29 | voxel id */
     const uint32_t *ranges;   /* [total_tiles][2] begin, end of each tile's list */
@@ -172,8 +172,8 @@ SVR_API size_t svr_workspace_size_views(int64_t n_vox, int64_t pair_capacity,
  *     rectangle of the 2-D bounding box of its 8 projected corners (all
  *     corners at camera depth <= 1e-3: culled; some: whole image); the pair
  *     count = sum over the rectangle's tiles of the number of sign patterns
- *     in the tile mask; its colour (Eq. vox_color) and its 8 gathered corner
- *     densities.
+ *     in the tile mask; its colour (Eq. vox_color) and its density, from the
+ *     8 gathered corner densities, as a polynomial about its centre.
  * Fills *frame.  pair_capacity: pairs the workspace was sized for.
  * Errors: SVR_ERR_INVALID (null pointer, K not in 1..3, tile != 16, bad
  * camera, misaligned sh or workspace, workspace too small, max_level outside
@@ -207,8 +207,9 @@ SVR_API int svr_preprocess_views(svr_frame *frame, const svr_scene *scene, const
  * direction-dependent Morton order of Sec. B.2), value = s << 29 | voxel id;
  * then a sort of each tile's range by the Morton bits that can differ (the
  * top 3 (max_level + 1) of the 48; with max_level = 16 all of them and the
- * value first), done tile by tile in shared memory: stable LSD radix sorts of
- * 1024-pair chunks, whose runs are merged per tile.  The result equals a sort
+ * value first), done tile by tile: merge sorts in shared memory, of chunks of
+ * 8192 pairs in longer lists, whose chunks are then merged by clusters of
+ * CTAs.  The result equals a sort
  * of all pairs by (key, value): within a tile distinct pairs have distinct
  * (key, value).  Also builds the render work order and the per-block lists.
  * n_pairs_out: if not NULL, the call synchronises the stream, stores the
@@ -360,7 +361,8 @@ SVR_API int svr_render_stats(const svr_frame *frame, float *rgb, float *depth, f
  * array compiled into the library, which every GPU that loads the library
  * keeps until the process exits.
  * Limits: at most 65536 voxels, at most 2^16 tiles, and as many pairs as fit
- * in the array next to the voxel buffers; beyond them the call returns
+ * in 16 MiB next to the voxel, tile and backward buffers of a workspace (by a
+ * fixed count of bytes per voxel, tile and pair); beyond them the call returns
  * SVR_ERR_LIMIT (voxels, tiles or image) or SVR_ERR_CAPACITY (pairs; the
  * render is skipped and *n_pairs_out holds the true count).
  * The first call on a device looks up the array's device address (once per
