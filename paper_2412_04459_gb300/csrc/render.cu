@@ -231,9 +231,10 @@ __device__ __forceinline__ bool slab(const Entry &e, const PixelRay &p, float &a
 // items of its blocks, in the work order's place.  The warp of segment 0 also
 // clears the tile's merge counters for the next forward.  The warps form a
 // persistent grid that strides over the entries.  A CTA per entry, with the
-// masks in shared memory and two barriers per 1024 entries, took 28 us for
-// the 1M-voxel frame and 1.55 ms for 8 views of 8M voxels: it waited for
-// itself.
+// masks in shared memory and two barriers per 1024 entries, took 30.5 us for
+// the 1M-voxel frame and 422 us for 16 mixed views against 25.7 and 267: it
+// waited for itself.  8 views of 8M voxels take 1.56 ms either way, waiting for
+// their boxes.  Two or eight groups in flight: 293 and 297 us (mixed views).
 
 constexpr int kListThreads = 128;
 constexpr int kListUnroll = 4;
@@ -1968,8 +1969,8 @@ __global__ void __launch_bounds__(kVoxBwdThreads) k_voxel_bwd(FrameDev f, float 
 // instruction.  Bound by the latency of its two dependent loads and the
 // scattered atomics: kGridIlp corners per thread are in flight.  A kernel of
 // its own, before k_voxel_bwd while the accumulators are in L2: inside it,
-// 79 us (1M voxels) and 1.28 ms (8M, 8 views) for both against 37 + 37 us and
-// 0.31 + 0.72 ms; as other CTAs of one launch, 116 us and 1.54 ms.
+// 79 us (1M voxels) and 1.28 ms (8M, 8 views) for both against 31 + 40 us and
+// 0.29 + 0.60 ms; as other CTAs of one launch, 116 us and 1.54 ms.
 constexpr int kGridThreads = 256, kGridIlp = 4;
 
 __global__ void __launch_bounds__(kGridThreads) k_grid_bwd(FrameDev f, float *__restrict__ d_grid) {
