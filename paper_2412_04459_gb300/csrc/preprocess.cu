@@ -230,11 +230,13 @@ __device__ __forceinline__ short4 project_voxel(const DevCam &cam, float c0, flo
         box = fx0 <= fx1 && fy0 <= fy1 ? make_ushort4((unsigned short)fx0, (unsigned short)fx1, (unsigned short)fy0,
                                                       (unsigned short)fy1)
                                        : make_ushort4(1, 0, 1, 0);
-        const float T = (float)cam.tile;
-        const int tx0 = umin < 0.f ? 0 : min(cam.ntx - 1, (int)floorf(umin / T));
-        const int tx1 = umax >= (float)cam.W ? cam.ntx - 1 : min(cam.ntx - 1, (int)floorf(umax / T));
-        const int ty0 = vmin < 0.f ? 0 : min(cam.nty - 1, (int)floorf(vmin / T));
-        const int ty1 = vmax >= (float)cam.H ? cam.nty - 1 : min(cam.nty - 1, (int)floorf(vmax / T));
+        // a power of two, so its inverse is exact (four divisions were 2 % of
+        // the kernel: 8 views of 8M voxels 2671 -> 2618 us)
+        const float inv_T = 1.0f / (float)cam.tile;
+        const int tx0 = umin < 0.f ? 0 : min(cam.ntx - 1, (int)floorf(umin * inv_T));
+        const int tx1 = umax >= (float)cam.W ? cam.ntx - 1 : min(cam.ntx - 1, (int)floorf(umax * inv_T));
+        const int ty0 = vmin < 0.f ? 0 : min(cam.nty - 1, (int)floorf(vmin * inv_T));
+        const int ty1 = vmax >= (float)cam.H ? cam.nty - 1 : min(cam.nty - 1, (int)floorf(vmax * inv_T));
         rc = make_short4((short)tx0, (short)tx1, (short)ty0, (short)ty1);
     }
     return rc;
