@@ -136,8 +136,8 @@ __device__ __forceinline__ bool voxel_valid(const FrameDev &f, int64_t v, float 
     }
     // corner indices must name grid points
     const int4 *ci = reinterpret_cast<const int4 *>(f.corner_idx + 8 * v);
-    i0 = __ldg(ci);
-    i1 = __ldg(ci + 1);
+    i0 = ci[0];
+    i1 = ci[1];
     const int64_t np = f.n_pts;
     const int lo = min(min(min(i0.x, i0.y), min(i0.z, i0.w)), min(min(i1.x, i1.y), min(i1.z, i1.w)));
     const int hi = max(max(max(i0.x, i0.y), max(i0.z, i0.w)), max(max(i1.x, i1.y), max(i1.z, i1.w)));
@@ -324,7 +324,7 @@ __device__ __forceinline__ void load_sh(const FrameDev &f, int64_t v, float sh[4
     const float4 *shv = reinterpret_cast<const float4 *>(f.sh + 48 * v);
 #pragma unroll
     for (int q = 0; q < 12; ++q) {
-        const float4 s4 = __ldg(shv + q);
+        const float4 s4 = shv[q];
         sh[4 * q + 0] = s4.x;
         sh[4 * q + 1] = s4.y;
         sh[4 * q + 2] = s4.z;
@@ -335,8 +335,8 @@ __device__ __forceinline__ void load_sh(const FrameDev &f, int64_t v, float sh[4
 // A voxel's density polynomial from its gathered corner densities.
 __device__ __forceinline__ void gather_density(const FrameDev &f, const int4 &i0, const int4 &i1, float4 &r1,
                                                float4 &r2) {
-    float g[8] = {__ldg(f.grid + i0.x), __ldg(f.grid + i0.y), __ldg(f.grid + i0.z), __ldg(f.grid + i0.w),
-                  __ldg(f.grid + i1.x), __ldg(f.grid + i1.y), __ldg(f.grid + i1.z), __ldg(f.grid + i1.w)};
+    float g[8] = {f.grid[i0.x], f.grid[i0.y], f.grid[i0.z], f.grid[i0.w],
+                  f.grid[i1.x], f.grid[i1.y], f.grid[i1.z], f.grid[i1.w]};
     density_coeffs(g);
     r1 = make_float4(g[0], g[1], g[2], g[3]);
     r2 = make_float4(g[4], g[5], g[6], g[7]);

@@ -239,7 +239,7 @@ __device__ __forceinline__ bool slab(const Entry &e, const PixelRay &p, float &a
 constexpr int kListThreads = 128;
 constexpr int kListUnroll = 4;
 
-__device__ __forceinline__ void block_lists_entry(const FrameDev &f, const uint32_t *__restrict__ vals, unsigned e) {
+__device__ __forceinline__ void block_lists_entry(const FrameDev &f, const uint32_t *vals, unsigned e) {
     const uint2 gs = f.order[e];
     const int g = (int)gs.x, sg = (int)gs.y;
     const uint2 rg = f.ranges[g];
@@ -277,13 +277,13 @@ __device__ __forceinline__ void block_lists_entry(const FrameDev &f, const uint3
 #pragma unroll
         for (int u = 0; u < kListUnroll; ++u) {
             const int i = c0 + 32 * u + lane;
-            val[u] = i < stop ? __ldg(vals + i) : 0u;
+            val[u] = i < stop ? __ldcg(vals + i) : 0u;
         }
         ushort4 bx[kListUnroll];
 #pragma unroll
         for (int u = 0; u < kListUnroll; ++u)
             bx[u] = c0 + 32 * u + lane < stop
-                        ? __ldg(boxes + checked(f.debug, kDbgVoxel, val[u] & 0x1FFFFFFFu, f.n_vox))
+                        ? __ldcg(boxes + checked(f.debug, kDbgVoxel, val[u] & 0x1FFFFFFFu, f.n_vox))
                         : make_ushort4(1, 0, 1, 0);
 #pragma unroll
         for (int u = 0; u < kListUnroll; ++u) {
@@ -319,7 +319,7 @@ __device__ __forceinline__ void block_lists_entry(const FrameDev &f, const uint3
     }
 }
 
-__global__ void __launch_bounds__(kListThreads) k_block_lists(FrameDev f, const uint32_t *__restrict__ vals) {
+__global__ void __launch_bounds__(kListThreads) k_block_lists(FrameDev f, const uint32_t *vals) {
     begin_kernel();
     const unsigned nq = f.status->n_listed;  // empty lists have no block lists
     const unsigned warps = gridDim.x * (kListThreads / 32);
@@ -349,13 +349,13 @@ struct Lookahead {
     bool valid;
 };
 
-__device__ __forceinline__ void fetch_vi(Lookahead &la, const uint2 *__restrict__ list, int pos, bool valid) {
+__device__ __forceinline__ void fetch_vi(Lookahead &la, const uint2 *list, int pos, bool valid) {
     la.valid = valid;
-    la.vi = valid ? __ldg(list + pos) : make_uint2(0u, 0u);
+    la.vi = valid ? __ldcg(list + pos) : make_uint2(0u, 0u);
 }
 
 __device__ __forceinline__ void fetch_box(Lookahead &la, const ViewData &vd) {
-    la.box = la.valid ? __ldg(vd.box + vid_of(vd, la.vi.x)) : make_ushort4(0, 0, 0, 0);
+    la.box = la.valid ? __ldcg(vd.box + vid_of(vd, la.vi.x)) : make_ushort4(0, 0, 0, 0);
 }
 
 // Ask for the looked-ahead entry's 64-byte record in L1 (the backward stages
@@ -744,7 +744,7 @@ __device__ __forceinline__ void fwd_hits_parallel(const FwdSlot *st, const uint2
 // Returns the position at which every pixel had stopped (p1 or beyond if the
 // walk went to the end).
 template <int K, int MODE>
-__device__ __forceinline__ int fwd_walk(const uint2 *__restrict__ list, int p0, int p1, const ViewData &vd,
+__device__ __forceinline__ int fwd_walk(const uint2 *list, int p0, int p1, const ViewData &vd,
                                          const PixelRay &p, const WarpBlock &wb, FwdSmem &ws, float t_stop,
                                          FwdState &s, const FwdOut &out, bool true_weights, uint32_t *hm) {
     constexpr bool STATS = MODE == kModeStats, FN = MODE == kModeExtra, FD = FN || MODE == kModeDist;

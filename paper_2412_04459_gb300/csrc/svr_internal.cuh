@@ -418,6 +418,10 @@ unsigned device_cached(DeviceCache &c, F compute) {
 // for the smallest view.  The backward's kernels are launched plainly: with
 // them the step took 773 us.  Nor do the kernels of a large batch gain (16
 // mixed views, 75,080 tiles: 8.34 ms without, 8.37 with).
+// Such a kernel is resident while the ones before it still write, so what it
+// reads is not constant for its lifetime: it loads with ordinary or L2 loads
+// only, which the wait orders, never through __ldg or const __restrict__
+// pointers (ld.global.nc).
 constexpr int kOverlapTiles = 16384;
 
 __device__ __forceinline__ void begin_kernel() {
