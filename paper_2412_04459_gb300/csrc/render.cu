@@ -1949,7 +1949,9 @@ __global__ void __launch_bounds__(kVoxBwdThreads) k_voxel_bwd(FrameDev f, float 
         float4 *row = reinterpret_cast<float4 *>(rows + threadIdx.x * kShRow);
 #pragma unroll
         for (int q = 0; q < 12; ++q) row[q] = make_float4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
-        if (priority && prio != 0.f) priority[v] += prio;
+        // atomic: backwards of other frames may add to the same priorities on
+        // other streams
+        if (priority && prio != 0.f) atomicAdd(priority + v, prio);
     }
     __syncthreads();
     const int nv = (int)tmin<int64_t>(kVoxBwdThreads, f.n_vox - v0);
