@@ -29,7 +29,9 @@
 // Forward (Sec. 3.1.2, Eq. alpha_blend, Eq. supp_alpha_comp, Sec. A.4):
 //   K samples per segment, trilinear raw density, explin, per-sample
 //   e_k = exp(-(l/K) explin(v_k)); 1 - alpha = prod_k e_k; local depth
-//   d = sum_k prod_{j<k} e_j (1 - e_k) t_k; C += T alpha c, D += T d,
+//   d = sum_k prod_{j<k} e_j (1 - e_k) t_k, P (1 - e) as the multiply-add P - P e
+//   (the difference of two rounded transmittances put depths up to 16 % further
+//   from 64 bits); C += T alpha c, D += T d,
 //   T *= 1 - alpha; a pixel stops after the voxel that leaves T < t_stop and
 //   the warp leaves the list once all its pixels stopped.
 //
@@ -500,9 +502,9 @@ __device__ __forceinline__ void hit_fwd(const Entry &e, const PixelRay &p, float
     for (int k = 0; k < K; ++k) {
         const float v = trilerp(e.g0, e.g1, fmaf(t, rx, -e.c.x), fmaf(t, ry, -e.c.y), fmaf(t, rz, -e.c.z));
         const float xk = xs * explin(v);
-        const float Pn = P * ex2(-xk);
-        d = fmaf(P - Pn, t, d);
-        P = Pn;
+        const float ek = ex2(-xk);
+        d = fmaf(fmaf(-P, ek, P), t, d);
+        P *= ek;
         X += xk;
         t += step;
     }
@@ -654,9 +656,9 @@ __device__ __forceinline__ void hit_fwd_slot(const FwdSlot &e, const PixelRay &p
     for (int k = 0; k < K; ++k) {
         const float v = trilerp(g0, g1, fmaf(t, rx, -cx), fmaf(t, ry, -cy), fmaf(t, rz, -cz));
         const float xk = xs * explin(v);
-        const float Pn = P * ex2(-xk);
-        d = fmaf(P - Pn, t, d);
-        P = Pn;
+        const float ek = ex2(-xk);
+        d = fmaf(fmaf(-P, ek, P), t, d);
+        P *= ek;
         X += xk;
         t += step;
     }
@@ -1216,7 +1218,7 @@ __device__ __forceinline__ void hit_grad(const Entry &e, const PixelRay &p, cons
     const float rx = p.rd.x * inv_size, ry = p.rd.y * inv_size, rz = p.rd.z * inv_size;
     // of each sample: its place, the transmittance up to it, and d x_k / d v_k
     // (explin' is 1 above 1.1, else explin / 1.1)
-    float tk[K], Pk[K + 1], qx[K], qy[K], qz[K], dx[K];
+    float tk[K], Pk[K + 1], wk[K], qx[K], qy[K], qz[K], dx[K];
     float t = fmaf(0.5f, step, a);
     float d = 0.f, X = 0.f;
     Pk[0] = 1.f;
@@ -1228,10 +1230,12 @@ __device__ __forceinline__ void hit_grad(const Entry &e, const PixelRay &p, cons
         const float v = trilerp(e.g0, e.g1, qx[k], qy[k], qz[k]);
         const float xk = xs2 * explin(v);
         dx[k] = v > 1.1f ? xs : xk * (kLn2 * 0.909090909f);
-        Pk[k + 1] = Pk[k] * ex2(-xk);
+        const float ek = ex2(-xk);
+        Pk[k + 1] = Pk[k] * ek;
+        wk[k] = fmaf(-Pk[k], ek, Pk[k]);
         X += xk;
         tk[k] = t;
-        d = fmaf(Pk[k] - Pk[k + 1], t, d);
+        d = fmaf(wk[k], t, d);
         t += step;
     }
     const float trans = Pk[K];
@@ -1299,7 +1303,7 @@ __device__ __forceinline__ void hit_grad(const Entry &e, const PixelRay &p, cons
         dgeo[5] = fmaf(ax, qz[k], dgeo[5]);
         dgeo[6] += axy;
         dgeo[7] = fmaf(axy, qz[k], dgeo[7]);
-        Q = fmaf(Pk[k] - Pk[k + 1], tk[k], Q);
+        Q = fmaf(wk[k], tk[k], Q);
     }
     // normal: dL/dn = w g_N, through the normalisation (I - n n^T) / |grad|
     // to the linear coefficients (Eq. interp_grad_grad)
