@@ -43,8 +43,7 @@
 //   dC/dc_i = T_i alpha_i,
 //   dd_i/dx_ik = P_{k+1} t_k - sum_{m>k} P_m (1 - e_m) t_m  (P_k = prod_{j<k} e_j;
 //                the general form of the K <= 3 closed forms of Sec. A.4),
-//   dx_ik/dv_k = (l/K) explin'(v_k), dv_k/da_m = monomial m of the density
-//   polynomial (its adjoint takes the sums to the corners).
+//   dx_ik/dv_k = (l/K) explin'(v_k), dv_k/dV_c = corner c's trilinear weight.
 // T_i is recovered as T_{i+1} / exp(-x_i).  Pixels whose T_final is below
 // 1e-30 (where that division loses precision) take a front-to-back phase
 // instead, with SC_i, SD_i from totals recomputed in a first sweep.  The
@@ -75,7 +74,7 @@ constexpr int kBatch = 32;
 struct Entry {
     float4 a;    // entry plane (near corner) relative to r_o, clamp bits of the colour channels (uint)
     float4 b;    // exit plane (far corner) relative to r_o, 1 / size
-    float4 c;    // (centre - r_o) / size, index in the sorted list (int)
+    float4 c;    // (min corner - r_o) / size, index in the sorted list (int)
     float4 g0;   // density polynomial: 1, z, y, yz
     float4 g1;   // x, xz, xy, xyz
     float4 col;  // colour, voxel id (int)
@@ -91,7 +90,7 @@ __device__ __forceinline__ void stage_entry(Entry &e, uint32_t val, int idx, con
     const float hx = lx + size, hy = ly + size, hz = lz + size;
     const float inv = 1.0f / size;
     e.b = make_float4((s & 4) ? lx : hx, (s & 2) ? ly : hy, (s & 1) ? lz : hz, inv);
-    e.c = make_float4(fmaf(lx, inv, 0.5f), fmaf(ly, inv, 0.5f), fmaf(lz, inv, 0.5f), __int_as_float(idx));
+    e.c = make_float4(lx * inv, ly * inv, lz * inv, __int_as_float(idx));
     e.g0 = __ldg(&r->r1);
     e.g1 = __ldg(&r->r2);
     const float4 c3 = __ldg(&r->r3);
@@ -500,7 +499,8 @@ __device__ __forceinline__ void hit_fwd(const Entry &e, const PixelRay &p, float
     float P = 1.f, d = 0.f, X = 0.f;
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-        const float v = trilerp(e.g0, e.g1, fmaf(t, rx, -e.c.x), fmaf(t, ry, -e.c.y), fmaf(t, rz, -e.c.z));
+        const float v = trilerp(e.g0, e.g1, fmaf(t, rx, -e.c.x) - 0.5f, fmaf(t, ry, -e.c.y) - 0.5f,
+                                fmaf(t, rz, -e.c.z) - 0.5f);
         const float xk = xs * explin(v);
         const float ek = ex2(-xk);
         d = fmaf(fmaf(-P, ek, P), t, d);
@@ -1216,7 +1216,7 @@ __device__ __forceinline__ void hit_grad(const Entry &e, const PixelRay &p, cons
     const float step = seg * inv_k;
     const float inv_size = e.b.w;
     const float rx = p.rd.x * inv_size, ry = p.rd.y * inv_size, rz = p.rd.z * inv_size;
-    // of each sample: its place, the transmittance up to it, and d x_k / d v_k
+    // of each sample: its place in [0, 1]^3, the transmittance up to it, and d x_k / d v_k
     // (explin' is 1 above 1.1, else explin / 1.1)
     float tk[K], Pk[K + 1], wk[K], qx[K], qy[K], qz[K], dx[K];
     float t = fmaf(0.5f, step, a);
@@ -1227,7 +1227,7 @@ __device__ __forceinline__ void hit_grad(const Entry &e, const PixelRay &p, cons
         qx[k] = fmaf(t, rx, -e.c.x);
         qy[k] = fmaf(t, ry, -e.c.y);
         qz[k] = fmaf(t, rz, -e.c.z);
-        const float v = trilerp(e.g0, e.g1, qx[k], qy[k], qz[k]);
+        const float v = trilerp(e.g0, e.g1, qx[k] - 0.5f, qy[k] - 0.5f, qz[k] - 0.5f);
         const float xk = xs2 * explin(v);
         dx[k] = v > 1.1f ? xs : xk * (kLn2 * 0.909090909f);
         const float ek = ex2(-xk);
@@ -1293,34 +1293,42 @@ __device__ __forceinline__ void hit_grad(const Entry &e, const PixelRay &p, cons
     for (int k = K - 1; k >= 0; --k) {
         const float gxk = fmaf(gdT, fmaf(Pk[k + 1], tk[k], -Q), gx);
         const float dv = gxk * dx[k];
-        // adjoint of the polynomial's coefficients (trilerp)
-        const float ax = dv * qx[k], ay = dv * qy[k], axy = ax * qy[k];
-        dgeo[0] += dv;
-        dgeo[1] = fmaf(dv, qz[k], dgeo[1]);
-        dgeo[2] += ay;
-        dgeo[3] = fmaf(ay, qz[k], dgeo[3]);
-        dgeo[4] += ax;
-        dgeo[5] = fmaf(ax, qz[k], dgeo[5]);
-        dgeo[6] += axy;
-        dgeo[7] = fmaf(axy, qz[k], dgeo[7]);
+        // each corner's share by its trilinear weight, axis by axis (1 - q inside
+        // the multiply-add), so that a corner with a small share keeps its
+        // relative precision.  Sums of the polynomial's coefficients, taken to
+        // the corners at the end, cost 4 operations a sample less and left every
+        // corner the rounding of the whole.
+        const float ax0 = fmaf(-dv, qx[k], dv), ax1 = dv * qx[k];
+        const float b00 = fmaf(-ax0, qy[k], ax0), b01 = ax0 * qy[k];
+        const float b10 = fmaf(-ax1, qy[k], ax1), b11 = ax1 * qy[k];
+        const float z0 = 1.f - qz[k], z1 = qz[k];
+        dgeo[0] = fmaf(b00, z0, dgeo[0]);
+        dgeo[1] = fmaf(b00, z1, dgeo[1]);
+        dgeo[2] = fmaf(b01, z0, dgeo[2]);
+        dgeo[3] = fmaf(b01, z1, dgeo[3]);
+        dgeo[4] = fmaf(b10, z0, dgeo[4]);
+        dgeo[5] = fmaf(b10, z1, dgeo[5]);
+        dgeo[6] = fmaf(b11, z0, dgeo[6]);
+        dgeo[7] = fmaf(b11, z1, dgeo[7]);
         Q = fmaf(wk[k], tk[k], Q);
     }
     // normal: dL/dn = w g_N, through the normalisation (I - n n^T) / |grad|
-    // to the linear coefficients (Eq. interp_grad_grad)
+    // and Eq. interp_grad_grad: dgrad/dV_c = (2 x_c - 1, 2 y_c - 1, 2 z_c - 1) / 4
     if (XN && nlen > 0.f) {
         const float dnx = w * g.gN0, dny = w * g.gN1, dnz = w * g.gN2;
         const float dot = dnx * nrm.x + dny * nrm.y + dnz * nrm.z;
-        const float il = 1.0f / nlen;
-        dgeo[4] += (dnx - nrm.x * dot) * il;
-        dgeo[2] += (dny - nrm.y * dot) * il;
-        dgeo[1] += (dnz - nrm.z * dot) * il;
+        const float il = 0.25f / nlen;
+        const float gx_ = (dnx - nrm.x * dot) * il, gy_ = (dny - nrm.y * dot) * il, gz_ = (dnz - nrm.z * dot) * il;
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            dgeo[c] += ((c & 4) ? gx_ : -gx_) + ((c & 2) ? gy_ : -gy_) + ((c & 1) ? gz_ : -gz_);
     }
 }
 
 // ------------------------------------------------------- gradient records
 //
 // The gradients of one batch's hits go to per-hit records of 12 floats (8
-// density coefficients, 3 colour channels, the priority term) laid out entry by
+// corner densities, 3 colour channels, the priority term) laid out entry by
 // entry: the hits of staged entry j get consecutive slots, in pixel order, so
 // a lane writes each of its hits' records to a slot of its own with no
 // coordination.  At most kRecCap records are held at a time: a batch with
@@ -1329,9 +1337,9 @@ __device__ __forceinline__ void hit_grad(const Entry &e, const PixelRay &p, cons
 //
 // Once a run's hits are done, the lanes sum its records: lane l takes the
 // kRecLane slots from kRecLane l, and adds each stretch of one entry to the
-// voxel's accumulators in global memory with three 16-byte atomics (density
-// coefficients per voxel, colour and priority per view and voxel; k_voxel_bwd
-// takes them on to d_grid, d_sh and the priorities).  So the work is even
+// voxel's accumulators in global memory with three 16-byte atomics (corner
+// densities per voxel, colour and priority per view and voxel; k_grid_bwd and
+// k_voxel_bwd take them on to d_grid, d_sh and the priorities).  So the work is even
 // over the lanes whatever the entries' hit counts; with lane j summing entry
 // j's records, the warp waited for the entry with most hits (30 % of the
 // kernel, 16 mixed views: 4.99 ms in all), and each entry took 11 scalar
@@ -1374,7 +1382,7 @@ __device__ __forceinline__ int rec_slot(const RecSmem &rs, int k, int base) {
     return rs.off[k] + __popc(rs.pix[k] & lt) - base;
 }
 
-// Record of a hit on entry k: 8 coefficient gradients, 3 colour gradients
+// Record of a hit on entry k: 8 corner-density gradients, 3 colour gradients
 // and the subdivision priority term (extras; 0 otherwise).
 __device__ __forceinline__ void rec_write(RecSmem &rs, int slot, int k, const float dgeo[8], const float dcol[3],
                                           float prio) {
@@ -1967,42 +1975,31 @@ __global__ void __launch_bounds__(kVoxBwdThreads) k_voxel_bwd(FrameDev f, float 
     }
 }
 
-// The voxels' density gradients, summed over all hits in all views, taken
-// from the polynomial's coefficients to the corners and added to the grid
-// points (a voxel that no pixel hit has none).  Eight lanes take a voxel's
-// eight corners, so that the corner indices are read coalesced and the
-// adjacent grid points of corners 2 i and 2 i + 1 share a sector of one
-// instruction.  Bound by the latency of its two dependent loads and the
-// scattered atomics: kGridIlp corners per thread are in flight.  A kernel of
-// its own, before k_voxel_bwd while the accumulators are in L2: inside it,
-// 79 us (1M voxels) and 1.28 ms (8M, 8 views) for both against 31 + 40 us and
-// 0.29 + 0.60 ms; as other CTAs of one launch, 116 us and 1.54 ms.
+// The voxels' corner-density gradients, summed over all hits in all views,
+// added to the grid points (zeros are not: most voxels of a sparse view have no
+// hit).  Eight lanes take a voxel's eight corners, so that the sums and the
+// corner indices are read coalesced and the adjacent grid points of corners 2 i
+// and 2 i + 1 share a sector of one instruction.  Bound by the latency of its
+// two dependent loads and the scattered atomics: kGridIlp corners per thread are
+// in flight.  A kernel of its own, before k_voxel_bwd while the accumulators are
+// in L2: inside it, 79 us (1M voxels) and 1.28 ms (8M, 8 views) for both against
+// 31 + 40 us and 0.29 + 0.60 ms; as other CTAs of one launch, 116 us and 1.54 ms.
 constexpr int kGridThreads = 256, kGridIlp = 4;
 
 __global__ void __launch_bounds__(kGridThreads) k_grid_bwd(FrameDev f, float *__restrict__ d_grid) {
     if (blockIdx.x == 0 && threadIdx.x == 0) f.status->bwd_next = 0;   // for the next backward
-    const int c = threadIdx.x & 7;
-    const float sz = (c & 1) ? 1.f : -1.f, sy = (c & 2) ? 1.f : -1.f, sx = (c & 4) ? 1.f : -1.f;
     const int64_t n = f.n_vox * 8;
     const int64_t i0 = (int64_t)blockIdx.x * (kGridThreads * kGridIlp) + threadIdx.x;   // corners of all voxels
+    const float *acc = reinterpret_cast<const float *>(f.dgrid);
     float d[kGridIlp];
-    float4 g0[kGridIlp], g1[kGridIlp];
 #pragma unroll
     for (int r = 0; r < kGridIlp; ++r) {
         const int64_t i = i0 + r * kGridThreads;
-        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-        g0[r] = i < n ? __ldg(f.dgrid + 2 * (i >> 3)) : zero;
-        g1[r] = i < n ? __ldg(f.dgrid + 2 * (i >> 3) + 1) : zero;
+        d[r] = i < n ? __ldg(acc + i) : 0.f;
     }
     int p[kGridIlp];
 #pragma unroll
-    for (int r = 0; r < kGridIlp; ++r) {
-        // corner c's share: half a mean plus or minus a difference, per axis
-        const float a = fmaf(0.5f, g0[r].x, sx * g1[r].x), b = fmaf(0.5f, g0[r].y, sx * g1[r].y);
-        const float e = fmaf(0.5f, g0[r].z, sx * g1[r].z), h = fmaf(0.5f, g0[r].w, sx * g1[r].w);
-        d[r] = fmaf(0.5f, fmaf(0.5f, a, sy * e), sz * fmaf(0.5f, b, sy * h));
-        p[r] = d[r] != 0.f ? __ldg(f.corner_idx + i0 + r * kGridThreads) : 0;
-    }
+    for (int r = 0; r < kGridIlp; ++r) p[r] = d[r] != 0.f ? __ldg(f.corner_idx + i0 + r * kGridThreads) : 0;
 #pragma unroll
     for (int r = 0; r < kGridIlp; ++r)
         if (d[r] != 0.f && SVR_IN_BOUNDS(f.debug, kDbgGradPoint, p[r], f.n_pts)) atomicAdd(d_grid + p[r], d[r]);

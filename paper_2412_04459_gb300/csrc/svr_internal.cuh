@@ -335,7 +335,7 @@ struct FrameDev {
                              // batch's entries (bit i: position 32 k + i) that pixel p mod 32 hit
     int blocks_per_tile;     // B = tile * tile / 32
     float4 *dcol;            // [V * N] colour gradient and priority accumulators
-    float4 *dgrid;           // [N][2] density-coefficient gradient accumulators (after dcol)
+    float4 *dgrid;           // [N][2] corner-density gradient accumulators (after dcol)
     int64_t n_vox;
     int64_t n_pts;
     int64_t capacity;

@@ -38,3 +38,47 @@ def test_depth(name, K):
     transmittances: 1.3 to 9 % more for two and three samples)."""
     require_gpu()
     assert image_error(name, K, "depth") <= 1.015 * DEPTH[name, K]
+
+
+def test_small_shares_of_the_density_gradient():
+    """A corner's gradient is its trilinear weight's share of the voxel's.  One
+    voxel, one pixel, one sample near a corner: shares down to 1e-7 keep their
+    relative precision.  The place q in the voxel is t r / size - c with |t r /
+    size|, |c| <= 4, from operands of relative error below 2^-22: off by at
+    most 3e-6 per axis, so a share with distance w to the far faces' weights 0 by
+    3e-6 sum 1 / w, plus the products' roundings.  (Sums of polynomial
+    coefficients taken to the corners are off by 2^-24 of the whole gradient.)"""
+    require_gpu()
+    import torch
+    from paper_2412_04459_gb300 import DeviceScene, Frame
+    scene = synth.scenes.subscene(synth.dense_scene(1, seed=3), np.array([7]))
+    dev = DeviceScene.from_host(scene)
+    lo, size = np.asarray(scene.centre[0], np.float64) - 0.25, 0.5
+    rng = np.random.default_rng(11)
+    smallest, done = 1.0, 0
+    for _ in range(150):
+        w = np.exp(rng.uniform(np.log(0.004), np.log(0.1), 3))
+        corner = rng.integers(0, 2, 3)
+        target = lo + size * np.where(corner, 1 - w, w)
+        d = rng.normal(size=3)
+        d /= np.linalg.norm(d)
+        cam = synth.look_at(target - 1.2 * d, target, (0.0, 1.0, 0.0) if abs(d[1]) < 0.9 else (1.0, 0.0, 0.0), 40.0,
+                            1, 1)
+        w2c = np.asarray(cam.w2c, np.float64)
+        origin, ray = -w2c[:, :3].T @ w2c[:, 3], w2c[2, :3]   # the pixel's centre is the principal point
+        t = np.sort(np.stack([(lo - origin) / ray, (lo + size - origin) / ray]), 0)
+        a, b = t[0].max(), t[1].min()
+        q = (origin + 0.5 * (a + b) * ray - lo) / size
+        near = np.minimum(q, 1 - q)
+        if not (b - a > 1e-3 and near.max() < 0.2 and near.min() > 2e-3):
+            continue
+        fr = Frame(dev, cam, K=1)
+        out = fr.render()
+        d_grid, _ = fr.backward(torch.ones(3, 1, 1, device="cuda"), torch.zeros(1, 1, device="cuda"),
+                                torch.ones(1, 1, device="cuda"), out)
+        g = d_grid.double().cpu().numpy()[np.asarray(scene.corner_idx[0])]
+        share = np.array([np.prod(np.where(np.array([c >> 2 & 1, c >> 1 & 1, c & 1]), q, 1 - q)) for c in range(8)])
+        rel = np.abs(g / g.sum() / share - 1).max()
+        assert rel <= 3e-6 * (1 / near).sum() + 1e-6, (rel, share.min())
+        smallest, done = min(smallest, share.min()), done + 1
+    assert done >= 10 and smallest < 1e-5
