@@ -82,3 +82,15 @@ def test_small_shares_of_the_density_gradient():
         assert rel <= 3e-6 * (1 / near).sum() + 1e-6, (rel, share.min())
         smallest, done = min(smallest, share.min()), done + 1
     assert done >= 10 and smallest < 1e-5
+
+
+# the corner form's errors: alpha, one sample
+ALPHA = {"mixed": 5.00171e-07, "dense": 1.91148e-06}
+
+
+@pytest.mark.parametrize("name", sorted(ALPHA))
+def test_alpha(name):
+    """explin's exponent takes log2(e) as a factor of its own (folded into its
+    two constants: 0.6 to 1 % more).  The forward is deterministic."""
+    require_gpu()
+    assert image_error(name, 1, "alpha") <= 1.004 * ALPHA[name]
