@@ -94,3 +94,56 @@ def test_alpha(name):
     two constants: 0.6 to 1 % more).  The forward is deterministic."""
     require_gpu()
     assert image_error(name, 1, "alpha") <= 1.004 * ALPHA[name]
+
+
+def single_voxel(value):
+    scene = synth.scenes.subscene(synth.dense_scene(1, seed=3, grid_fn=synth.constant_grid(value)), np.array([7]))
+    centre = np.asarray(scene.centre[0], np.float64)
+    cam = synth.look_at(centre + np.array([0.4, 0.3, -2.0]), centre, (0.0, 1.0, 0.0), 20.0, 24, 16)
+    w2c = np.asarray(cam.w2c, np.float64)
+    origin = -w2c[:, :3].T @ w2c[:, 3]
+    x, y = np.meshgrid((np.arange(24) + 0.5 - float(cam.cx)) / float(cam.fx),
+                       (np.arange(16) + 0.5 - float(cam.cy)) / float(cam.fy))
+    rays = np.stack([x, y, np.ones_like(x)], -1) @ w2c[:, :3]
+    t = np.sort(np.stack([(centre - 0.25 - origin) / rays, (centre + 0.25 - origin) / rays]), 0)
+    length = np.maximum(t[1].min(-1) - t[0].max(-1), 0.0) * np.linalg.norm(rays, axis=-1)
+    return scene, cam, length
+
+
+TINY = 2.0 ** -149   # spacing of the subnormals
+
+
+@pytest.mark.parametrize("K", (1, 2, 3))
+@pytest.mark.parametrize("value", (-90.0, -97.0, -100.0, -104.0))
+def test_densities_below_the_normal_range(value, K):
+    """A voxel of density explin(v) < 2^-126 (v < -95.2) has a weight.  The
+    exponent, about -140, is off by three roundings of 2^-18 each at most, and
+    each of some ten subnormal products and sums by one spacing.  (Gradients
+    that small are flushed by the global atomics in any case.)"""
+    require_gpu()
+    import torch
+    from paper_2412_04459_gb300 import DeviceScene, Frame
+    scene, cam, length = single_voxel(value)
+    fr = Frame(DeviceScene.from_host(scene), cam, K=K)
+    fr.preprocess()
+    fr.bin_sort()
+    weight = torch.zeros(1, device="cuda")
+    fr.forward_ex(max_weight=weight)
+    sigma = 1.1 * np.exp(value / 1.1 - 1.0)
+    want = length.max() * sigma
+    assert abs(float(weight) - want) <= 1e-4 * want + 10 * TINY
+
+
+def test_transmittance_below_the_normal_range():
+    """exp(-x) for optical depths from 87.3 (2^-126) to 103 (2^-149) is not
+    flushed: relative error below that of x, 103 x 2^-21, plus one spacing."""
+    require_gpu()
+    from paper_2412_04459_gb300 import DeviceScene, Frame
+    scene, cam, length = single_voxel(0.0)
+    depth = 95.0 / length.max()
+    scene, cam, length = single_voxel(float(np.float32(depth)))
+    T = Frame(DeviceScene.from_host(scene), cam, K=1).render()["T_final"].double().cpu().numpy()
+    want = np.exp(-length * float(np.float32(depth)))
+    sel = (want < 2.0 ** -126) & (length > 0)
+    assert sel.sum() > 20
+    assert (np.abs(T - want)[sel] <= 1e-4 * want[sel] + 2 * TINY).all()
