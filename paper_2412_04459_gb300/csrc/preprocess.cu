@@ -332,11 +332,24 @@ __device__ __forceinline__ void load_sh(const FrameDev &f, int64_t v, float sh[4
     }
 }
 
+// Corner densities beyond this are taken as it: their voxels are as empty or as
+// opaque, and the differences of the polynomial stay finite.  (The lowest float,
+// or minus infinity, as the density of points that are to hold nothing gave
+// infinite differences of both signs, and NaN images.)  NaN stays NaN.
+constexpr float kDensityMost = 1e36f;
+
 // A voxel's density polynomial from its gathered corner densities.
 __device__ __forceinline__ void gather_density(const FrameDev &f, const int4 &i0, const int4 &i1, float4 &r1,
                                                float4 &r2) {
     float g[8] = {f.grid[i0.x], f.grid[i0.y], f.grid[i0.z], f.grid[i0.w],
                   f.grid[i1.x], f.grid[i1.y], f.grid[i1.z], f.grid[i1.w]};
+    float most = 0.f;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) most = fmaxf(most, fabsf(g[c]));
+    if (most > kDensityMost) {
+#pragma unroll
+        for (int c = 0; c < 8; ++c) g[c] = g[c] > kDensityMost ? kDensityMost : g[c] < -kDensityMost ? -kDensityMost : g[c];
+    }
     density_coeffs(g);
     r1 = make_float4(g[0], g[1], g[2], g[3]);
     r2 = make_float4(g[4], g[5], g[6], g[7]);
