@@ -72,7 +72,7 @@ Layout make_layout(int64_t n_vox, int n_views, int64_t cap, int64_t ntiles, int 
     const size_t subs = (size_t)ntiles << svr::tile_sub_log2(ntiles);
     take(kTileCount, 4 * 2 * subs);
     take(kRecord, sizeof(svr::Record) * VN);
-    take(kScanBlocks, 4 * ((subs + svr::kScanTile - 1) / svr::kScanTile + 1));
+    take(kScanBlocks, 8 * (size_t)svr::scan_blocks((int64_t)subs));
     take(kKeys0, 8 * C);
     take(kKeys1, 8 * C);
     take(kVals0, 4 * C);
@@ -213,7 +213,7 @@ svr::FrameDev frame_dev(const svr_frame *f) {
     d.cursor = d.tile_cnt + ((size_t)f->total_tiles << d.sub_log2);
     d.rec = (svr::Record *)(ws + o[kRecord]);
     d.box = (ushort4 *)(ws + o[kBox]);
-    d.scan_blocks = (uint32_t *)(ws + o[kScanBlocks]);
+    d.scan_blocks = (unsigned long long *)(ws + o[kScanBlocks]);
     d.keys[0] = (uint64_t *)(ws + o[kKeys0]);
     d.keys[1] = (uint64_t *)(ws + o[kKeys1]);
     d.vals[0] = (uint32_t *)(ws + o[kVals0]);

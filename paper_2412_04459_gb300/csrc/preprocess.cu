@@ -489,95 +489,98 @@ __device__ __forceinline__ int64_t sub_index(const FrameDev &f, int64_t i) {
     return (i & ((1 << f.sub_log2) - 1)) * (int64_t)f.total_tiles + (i >> f.sub_log2);
 }
 
-// Also clears the counters of the work order and the sort for k_scan_down.
-__global__ void __launch_bounds__(256) k_scan_reduce(FrameDev f) {
+// Sum of one 64-bit value per thread over the CTA (256 threads), in every thread.
+__device__ __forceinline__ unsigned long long block_sum(unsigned long long x, unsigned long long *warp_sums) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if ((threadIdx.x & 31) == 0) warp_sums[threadIdx.x >> 5] = x;
+    __syncthreads();
+    x = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) x += warp_sums[w];
+    return x;
+}
+
+// Sums of the scan blocks, `rounds` times 256 entries each (scan_rounds).  Also
+// clears the counters of the work order and the sort for k_scan_down.
+__global__ void __launch_bounds__(256) k_scan_reduce(FrameDev f, int rounds) {
     begin_kernel();
-    __shared__ uint32_t ws[8];
+    __shared__ unsigned long long ws[8];
     if (blockIdx.x == 0) {
         for (int i = threadIdx.x; i < (int)(sizeof(SortPlan) / 4); i += 256) reinterpret_cast<unsigned *>(f.plan)[i] = 0u;
         if (threadIdx.x == 0) f.status->slots_used = 0;
     }
     const int64_t n = (int64_t)f.total_tiles << f.sub_log2;
-    const int64_t i = (int64_t)blockIdx.x * kScanTile + threadIdx.x;
-    const uint64_t acc = i < n ? f.tile_cnt[sub_index(f, i)] : 0u;
-    uint32_t tot;
-    // a block sum beyond 2^32 saturates; the capacity check on the 64-bit
-    // total catches it
-    block_exclusive_scan((uint32_t)tmin<uint64_t>(acc, 0xFFFFFFFFull), ws, tot);
-    if (threadIdx.x == 0) f.scan_blocks[blockIdx.x] = tot;
+    unsigned long long acc = 0;
+    for (int r = 0; r < rounds; ++r) {
+        const int64_t i = ((int64_t)blockIdx.x * rounds + r) * kScanTile + threadIdx.x;
+        if (i < n) acc += f.tile_cnt[sub_index(f, i)];
+    }
+    acc = block_sum(acc, ws);
+    if (threadIdx.x == 0) f.scan_blocks[blockIdx.x] = acc;
 }
 
 // Sub-bucket starts (the emission cursors) from the counts, and per tile its
 // range, its segments (with slots for a split list's) and its work-order
-// group's count.  Each CTA first sums the block sums of all earlier CTAs
-// (64-bit), so no separate top-level scan is launched, and of all CTAs, so
-// that every one knows whether the pairs exceed the capacity (then all
-// ranges are empty).  A start beyond 2^32 saturates; the capacity flag covers
-// it.
-__global__ void __launch_bounds__(256) k_scan_down(FrameDev f, int nb) {
+// group's count.  Each CTA first sums the block sums of all earlier CTAs, so no
+// separate top-level scan is launched, and of all CTAs, so that every one
+// knows whether the pairs exceed the capacity: then all ranges are empty and
+// nothing is emitted, so it does not matter that the starts, 32-bit sums, wrap.
+__global__ void __launch_bounds__(256) k_scan_down(FrameDev f, int nb, int rounds) {
     begin_kernel();
     __shared__ uint32_t ws[8];
     __shared__ unsigned long long wpre[8], wall[8];
     __shared__ unsigned group_cnt[2 * kOrderGroups], slots, slot0;
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int t = threadIdx.x, lane = t & 31;
     if (t < 2 * kOrderGroups) group_cnt[t] = 0u;
     if (t == 0) slots = 0u;
     unsigned long long pre = 0, all = 0;
     for (int j = t; j < nb; j += 256) {
-        const unsigned x = f.scan_blocks[j];
+        const unsigned long long x = f.scan_blocks[j];
         all += x;
         if (j < (int)blockIdx.x) pre += x;
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        pre += __shfl_xor_sync(0xffffffffu, pre, o);
-        all += __shfl_xor_sync(0xffffffffu, all, o);
-    }
-    if (lane == 0) {
-        wpre[warp] = pre;
-        wall[warp] = all;
-    }
-    __syncthreads();
-    pre = all = 0;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) {
-        pre += wpre[w];
-        all += wall[w];
-    }
+    pre = block_sum(pre, wpre);
+    all = block_sum(all, wall);
     const bool over = all > (unsigned long long)f.capacity;
     const int64_t n = (int64_t)f.total_tiles << f.sub_log2;
-    const int64_t i = (int64_t)blockIdx.x * kScanTile + t;
-    const uint32_t x = i < n ? f.tile_cnt[sub_index(f, i)] : 0u;
-    uint32_t tot;
-    const uint32_t ex = block_exclusive_scan(x, ws, tot);
-    const uint32_t c = (uint32_t)tmin<unsigned long long>(pre + ex, 0xFFFFFFFFull);
-    const uint32_t e = (uint32_t)tmin<unsigned long long>(pre + ex + x, 0xFFFFFFFFull);
-    if (i < n) f.cursor[sub_index(f, i)] = c;
-    // the lanes of a tile's sub-buckets: the first one takes the tile
-    const int last_sub = (1 << f.sub_log2) - 1;
-    const uint32_t end = __shfl_sync(0xffffffffu, e, lane | last_sub);
-    const bool tile = i < n && (i & last_sub) == 0;
-    const uint2 r = over || end == c ? make_uint2(0u, 0u) : make_uint2(c, end);
-    const unsigned len = r.y - r.x;
-    unsigned nseg = len > (unsigned)kSegLen ? (len + kSegLen - 1) / kSegLen : 1u, base = 0;
-    if (tile && nseg > 1) base = atomicAdd(&slots, nseg);
-    __syncthreads();
-    if (t == 0) slot0 = slots ? atomicAdd(&f.status->slots_used, slots) : 0u;
-    __syncthreads();
-    if (tile) {
-        if (nseg > 1) {
-            base += slot0;
-            if ((int64_t)base + nseg > f.seg_slots) nseg = 1, base = 0;  // only past the pair capacity
+    uint32_t carry = (uint32_t)pre;
+    for (int r = 0; r < rounds; ++r) {
+        const int64_t i = ((int64_t)blockIdx.x * rounds + r) * kScanTile + t;
+        const uint32_t x = i < n ? f.tile_cnt[sub_index(f, i)] : 0u;
+        uint32_t tot;
+        const uint32_t c = carry + block_exclusive_scan(x, ws, tot);
+        if (i < n) f.cursor[sub_index(f, i)] = c;
+        carry += tot;
+        // the lanes of a tile's sub-buckets: the first one takes the tile
+        const int last_sub = (1 << f.sub_log2) - 1;
+        const uint32_t end = __shfl_sync(0xffffffffu, c + x, lane | last_sub);
+        const bool tile = i < n && (i & last_sub) == 0;
+        const uint2 rg = over || end == c ? make_uint2(0u, 0u) : make_uint2(c, end);
+        const unsigned len = rg.y - rg.x;
+        unsigned nseg = len > (unsigned)kSegLen ? (len + kSegLen - 1) / kSegLen : 1u, base = 0;
+        if (tile && nseg > 1) base = atomicAdd(&slots, nseg);
+        __syncthreads();
+        if (t == 0) {
+            slot0 = slots ? atomicAdd(&f.status->slots_used, slots) : 0u;
+            slots = 0u;
         }
-        const int bk = order_bucket(len, nseg);
-        if (nseg > 1) {
-            atomicAdd(&group_cnt[kFirstSeg + bk], 1u);
-            atomicAdd(&group_cnt[bk], nseg - 1);
-        } else {
-            atomicAdd(&group_cnt[bk], 1u);
+        __syncthreads();
+        if (tile) {
+            if (nseg > 1) {
+                base += slot0;
+                if ((int64_t)base + nseg > f.seg_slots) nseg = 1, base = 0;  // only past the pair capacity
+            }
+            const int bk = order_bucket(len, nseg);
+            if (nseg > 1) {
+                atomicAdd(&group_cnt[kFirstSeg + bk], 1u);
+                atomicAdd(&group_cnt[bk], nseg - 1);
+            } else {
+                atomicAdd(&group_cnt[bk], 1u);
+            }
+            f.ranges[i >> f.sub_log2] = rg;
+            f.tile_seg[i >> f.sub_log2] = make_uint2(nseg, base);
         }
-        f.ranges[i >> f.sub_log2] = r;
-        f.tile_seg[i >> f.sub_log2] = make_uint2(nseg, base);
     }
     __syncthreads();
     if (t < 2 * kOrderGroups && group_cnt[t]) atomicAdd(&f.plan->cnt[t], group_cnt[t]);
@@ -700,10 +703,11 @@ cudaError_t launch_preprocess(const FrameDev &f, cudaStream_t s) {
 }
 
 cudaError_t launch_scan(const FrameDev &f, cudaStream_t s) {
-    const int nb = (int)((((int64_t)f.total_tiles << f.sub_log2) + kScanTile - 1) / kScanTile);
-    static_assert(kScanTile == 256, "one entry per thread");
-    const cudaError_t e = launch(k_scan_reduce, dim3(nb), 256, 0, s, f);
-    return e != cudaSuccess ? e : launch(k_scan_down, dim3(nb), 256, 0, s, f, nb);
+    const int64_t n = (int64_t)f.total_tiles << f.sub_log2;
+    const int rounds = scan_rounds(n), nb = scan_blocks(n);
+    static_assert(kScanTile == 256, "one entry per thread and round");
+    const cudaError_t e = launch(k_scan_reduce, dim3(nb), 256, 0, s, f, rounds);
+    return e != cudaSuccess ? e : launch(k_scan_down, dim3(nb), 256, 0, s, f, nb, rounds);
 }
 
 cudaError_t launch_emit(const FrameDev &f, cudaStream_t s) {

@@ -41,6 +41,21 @@ __host__ __device__ __forceinline__ int tile_sub_log2(int64_t ntiles) {
     return ntiles <= 8192 ? 5 : ntiles <= 131072 ? 4 : 3;
 }
 
+// Blocks of the scan over n sub-buckets, at most kScanBlocks: every block sums
+// the sums of all, so without a bound the loads grow with the square of the
+// tiles (svr_bin_sort of a few pairs over 115,200 tiles 301 us without the bound,
+// 281 with it; 460,800: 906 and 841; 4.2 M: 7.7 and 3.7 ms).  Beyond 2^18
+// sub-buckets a block then takes several rounds of kScanTile.
+constexpr int kScanBlocks = 1024;
+__host__ __device__ __forceinline__ int scan_rounds(int64_t n) {
+    const int64_t most = (int64_t)kScanTile * kScanBlocks;
+    return (int)((n + most - 1) / most);
+}
+__host__ __device__ __forceinline__ int scan_blocks(int64_t n) {
+    const int64_t per = (int64_t)kScanTile * scan_rounds(n);
+    return (int)((n + per - 1) / per);
+}
+
 // A tile list up to kSortCap pairs is sorted by one group of threads in shared
 // memory; a longer one as chunks of at most kSortCap pairs, merged afterwards.
 constexpr int kSortCap = 8192;
@@ -315,7 +330,7 @@ struct FrameDev {
     uint32_t *cursor;        // [2^sub_log2][total_tiles] next free slot of each sub-bucket
     Record *rec;             // [V * N]
     ushort4 *box;            // [V * N] inclusive pixel range x0, x1, y0, y1 a hit can fall in
-    uint32_t *scan_blocks;   // [ceil(2^sub_log2 total_tiles / kScanTile) + 1]
+    unsigned long long *scan_blocks;   // [scan_blocks(2^sub_log2 total_tiles)] their sums
     uint64_t *keys[2];
     uint32_t *vals[2];
     SortPlan *plan;
