@@ -344,7 +344,7 @@ def run_native(args, rank, world, local_rank):
                      "unit": "T FP32 lane-ops/s", "frac": achieved_bwd / alu_peak, "traffic": traffic,
                      "traffic_from": traffic_from,
                      "work": {"hits": n_hit, "ops_per_hit": OPS_CAND + OPS_HIT_BWD[K]},
-                     "timed": "svr_render_bwd call: memset + k_render_bwd + k_grid_bwd + k_voxel_bwd",
+                     "timed": "svr_render_bwd call: k_clear_acc + k_render_bwd + k_grid_bwd + k_voxel_bwd",
                      "peak_from": f"{sm} SMs x {FP32_LANES_PER_SM} FP32 lanes x {sm_mhz:.0f} MHz"},
         "roofline_fwd": {"bound": "alu", "kernel": "k_render_fwd", "achieved": achieved, "peak": alu_peak,
                          "unit": "T FP32 lane-ops/s", "frac": achieved / alu_peak,
@@ -775,9 +775,9 @@ def frame_algorithmic_bytes(scene, P, H, W):
 def launches_per_step(fr):
     """Kernels of ours launched per step (fills/memsets excluded): tile masks,
     preprocess, 2 tile-count scan kernels, work order, emission, list sort,
-    long-list merge, block lists, forward, backward, its density scatter, its
-    SH gradients."""
-    return 2 + 2 + 1 + 1 + 2 + 1 + 1 + 1 + 2
+    long-list merge, block lists, forward, the accumulators' clearing, backward,
+    its density scatter, its SH gradients."""
+    return 2 + 2 + 1 + 1 + 2 + 1 + 1 + 1 + 1 + 2
 
 
 def sources_sha1(paths=KERNEL_SOURCES):

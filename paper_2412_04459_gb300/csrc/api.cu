@@ -29,7 +29,7 @@ inline size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 enum Slot {
     kStatus, kTileMask, kOctpath, kRect, kCount, kTileCount, kRecord, kScanBlocks,
     kKeys0, kKeys1, kVals0, kVals1, kRanges, kDcol, kBox, kTileOrder, kBlockList, kBlockLen,
-    kHitMask, kSegment, kSortPlan, kTotal, kNumSlots
+    kHitMask, kSegment, kSortPlan, kMayHit, kTotal, kNumSlots
 };
 
 struct Layout {
@@ -55,7 +55,10 @@ constexpr size_t kNone = ~size_t(0);   // offset of a buffer that the layout lea
 
 // n_vox voxels seen by n_views views with ntiles tiles of edge `tile` in all.
 // A forward-only layout leaves out what only the backward reads: the gradient
-// accumulators and the hit masks.
+// accumulators and the hit masks.  The accumulators lie where the sort had its
+// second pair buffer, which nothing reads after the sort (12 bytes per pair, of
+// which a caller usually takes 4 per voxel and view, against 16 per voxel and
+// view and 32 per voxel).
 Layout make_layout(int64_t n_vox, int n_views, int64_t cap, int64_t ntiles, int tile, bool forward_only = false) {
     Layout L;
     size_t o = 0;
@@ -74,13 +77,19 @@ Layout make_layout(int64_t n_vox, int n_views, int64_t cap, int64_t ntiles, int 
     take(kRecord, sizeof(svr::Record) * VN);
     take(kScanBlocks, 8 * (size_t)svr::scan_blocks((int64_t)subs));
     take(kKeys0, 8 * C);
-    take(kKeys1, 8 * C);
     take(kVals0, 4 * C);
+    take(kKeys1, 8 * C);
     take(kVals1, 4 * C);
+    L.off[kDcol] = kNone;
+    if (!forward_only) {
+        // colour accumulators per view, corner-density accumulators
+        L.off[kDcol] = L.off[kKeys1];
+        const size_t end = L.off[kDcol] + 16 * VN + 32 * N;
+        if (end > o) o = align256(end);
+    }
     take(kRanges, 8 * (size_t)ntiles);
-    if (forward_only) L.off[kDcol] = kNone;
-    else take(kDcol, 16 * VN + 32 * N);   // colour accumulators per view, corner-density accumulators
     take(kBox, 8 * VN);
+    take(kMayHit, n_views == 1 ? 4 * svr::hit_words(n_vox) : 0);
     const size_t slots = (size_t)svr::seg_slot_capacity(cap);
     take(kTileOrder, 8 * ((size_t)ntiles + slots));
     const size_t B = (size_t)tile * tile / 32;
@@ -213,6 +222,7 @@ svr::FrameDev frame_dev(const svr_frame *f) {
     d.cursor = d.tile_cnt + ((size_t)f->total_tiles << d.sub_log2);
     d.rec = (svr::Record *)(ws + o[kRecord]);
     d.box = (ushort4 *)(ws + o[kBox]);
+    d.may_hit = (uint32_t *)(ws + o[kMayHit]);
     d.scan_blocks = (unsigned long long *)(ws + o[kScanBlocks]);
     d.keys[0] = (uint64_t *)(ws + o[kKeys0]);
     d.keys[1] = (uint64_t *)(ws + o[kKeys1]);

@@ -386,6 +386,10 @@ __global__ void __launch_bounds__(128, 8) k_preprocess(FrameDev f) {
             mark_invalid(f.status, v);
         }
     }
+    // which of the warp's voxels a pixel can hit: those with a tile rectangle
+    // (and so with pairs) and a box that is not empty
+    const unsigned hit = __ballot_sync(0xffffffffu, rc.x <= rc.y && box.x <= box.y);
+    if (in && (threadIdx.x & 31) == 0) f.may_hit[v >> 5] = hit;
     const uint32_t cnt = count_pairs(f, cam, v, rc);
     if (!in) return;
     f.rect[iv] = rc;

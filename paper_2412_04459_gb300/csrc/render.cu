@@ -1905,6 +1905,27 @@ __global__ void __launch_bounds__(kBwdThreads, kBwdMinBlocks) k_render_bwd(Frame
     }
 }
 
+// Single view: clears the accumulators of the voxels that a pixel can hit
+// (may_hit); the others' are neither cleared nor read.  On a small image most
+// voxels of a large scene fall between the pixels' centres (94 % of 8.7M at 320 x
+// 210), and a memset of all accumulators made that backward slower than scattering
+// every hit's gradients had been: 8M voxels at 320 x 210 690 us, 659 with the
+// scatter, 528 so; at 640 x 420 825, 804 and 734.  The 1M-voxel step at 1280 x 840,
+// where every voxel can be hit, pays 0.3 %.  Batches keep the memset: there the
+// backward was faster than the scatter at every size tried (8 views of 8M voxels at
+// 320 x 210 2.72 against 3.48 ms, 4 of 2M at 640 x 420 0.79 against 0.87), a bit per view
+// gains 1 % of the former and costs 3 % of the latter and 4 % of every batch's preprocess.
+constexpr int kClearThreads = 256;
+
+__global__ void __launch_bounds__(kClearThreads) k_clear_acc(FrameDev f) {
+    const int64_t v = (int64_t)blockIdx.x * kClearThreads + threadIdx.x;
+    if (v >= f.n_vox || !((__ldg(f.may_hit + (v >> 5)) >> (v & 31)) & 1u)) return;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    f.dcol[v] = zero;
+    f.dgrid[2 * v] = zero;
+    f.dgrid[2 * v + 1] = zero;
+}
+
 // Per voxel: dL/dsh[n][c] = sum over views of Y_n(d_v) * dL/dc_{v,c}, over
 // the views where the voxel is in view (dL/dc_{v,c} holds only the channels
 // that were > 0 before the clamp, Eq. vox_color); zero for a voxel in no view;
@@ -1920,7 +1941,7 @@ constexpr int kShRow = 52;
 // 1M); a single view by its own instantiation, which needs fewer registers (40
 // us for 1M voxels, 45 with four).
 template <int VIEWS>
-__global__ void __launch_bounds__(kVoxBwdThreads) k_voxel_bwd(FrameDev f, float *__restrict__ d_sh,
+__global__ void __launch_bounds__(kVoxBwdThreads, VIEWS == 1 ? 7 : 5) k_voxel_bwd(FrameDev f, float *__restrict__ d_sh,
                                                               float *__restrict__ priority) {
     __shared__ __align__(16) float rows[kVoxBwdThreads * kShRow];
     const int64_t v0 = (int64_t)blockIdx.x * kVoxBwdThreads;
@@ -1935,7 +1956,8 @@ __global__ void __launch_bounds__(kVoxBwdThreads) k_voxel_bwd(FrameDev f, float 
             float4 g[VIEWS];
 #pragma unroll
             for (int i = 0; i < VIEWS; ++i)
-                seen[i] = view0 + i < f.n_views && f.count[(int64_t)(view0 + i) * f.n_vox + v] != 0;
+                seen[i] = VIEWS == 1 ? ((__ldg(f.may_hit + (v >> 5)) >> (v & 31)) & 1u) != 0u
+                                     : view0 + i < f.n_views && f.count[(int64_t)(view0 + i) * f.n_vox + v] != 0;
 #pragma unroll
             for (int i = 0; i < VIEWS; ++i)
                 if (seen[i]) g[i] = f.dcol[(int64_t)(view0 + i) * f.n_vox + v];
@@ -1984,25 +2006,43 @@ __global__ void __launch_bounds__(kVoxBwdThreads) k_voxel_bwd(FrameDev f, float 
 // in flight.  A kernel of its own, before k_voxel_bwd while the accumulators are
 // in L2: inside it, 79 us (1M voxels) and 1.28 ms (8M, 8 views) for both against
 // 31 + 40 us and 0.29 + 0.60 ms; as other CTAs of one launch, 116 us and 1.54 ms.
+// A warp takes 32 voxels and, ONE (a single view), skips those that no pixel can
+// hit.
 constexpr int kGridThreads = 256, kGridIlp = 4;
 
+template <bool ONE>
 __global__ void __launch_bounds__(kGridThreads) k_grid_bwd(FrameDev f, float *__restrict__ d_grid) {
     if (blockIdx.x == 0 && threadIdx.x == 0) f.status->bwd_next = 0;   // for the next backward
-    const int64_t n = f.n_vox * 8;
-    const int64_t i0 = (int64_t)blockIdx.x * (kGridThreads * kGridIlp) + threadIdx.x;   // corners of all voxels
-    const float *acc = reinterpret_cast<const float *>(f.dgrid);
-    float d[kGridIlp];
+    const size_t words = hit_words(f.n_vox);
+    const size_t w = (size_t)blockIdx.x * (kGridThreads / 32) + (threadIdx.x >> 5);
+    if (w >= words) return;
+    unsigned m = 0xffffffffu >> (32 - (int)tmin<int64_t>(32, f.n_vox - 32 * (int64_t)w));
+    if (ONE) m = __ldg(f.may_hit + w);
+    const float *acc = reinterpret_cast<const float *>(f.dgrid) + 256 * w;
+    const int32_t *corner = f.corner_idx + 256 * w;
+    const int c = threadIdx.x & 7, sub = (threadIdx.x >> 3) & 3;
+    while (m) {
+        // voxel sub of the next 4 kGridIlp with a bit, four at a time
+        int at[kGridIlp];
 #pragma unroll
-    for (int r = 0; r < kGridIlp; ++r) {
-        const int64_t i = i0 + r * kGridThreads;
-        d[r] = i < n ? __ldg(acc + i) : 0.f;
+        for (int r = 0; r < kGridIlp; ++r) {
+            at[r] = -1;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (q == sub && m) at[r] = 8 * (__ffs(m) - 1) + c;
+                m &= m - 1u;
+            }
+        }
+        float d[kGridIlp];
+        int p[kGridIlp];
+#pragma unroll
+        for (int r = 0; r < kGridIlp; ++r) d[r] = at[r] >= 0 ? __ldg(acc + at[r]) : 0.f;
+#pragma unroll
+        for (int r = 0; r < kGridIlp; ++r) p[r] = d[r] != 0.f ? __ldg(corner + at[r]) : 0;
+#pragma unroll
+        for (int r = 0; r < kGridIlp; ++r)
+            if (d[r] != 0.f && SVR_IN_BOUNDS(f.debug, kDbgGradPoint, p[r], f.n_pts)) atomicAdd(d_grid + p[r], d[r]);
     }
-    int p[kGridIlp];
-#pragma unroll
-    for (int r = 0; r < kGridIlp; ++r) p[r] = d[r] != 0.f ? __ldg(f.corner_idx + i0 + r * kGridThreads) : 0;
-#pragma unroll
-    for (int r = 0; r < kGridIlp; ++r)
-        if (d[r] != 0.f && SVR_IN_BOUNDS(f.debug, kDbgGradPoint, p[r], f.n_pts)) atomicAdd(d_grid + p[r], d[r]);
 }
 
 // ---------------------------------------------------------------- launchers
@@ -2102,8 +2142,12 @@ cudaError_t launch_render_bwd(const FrameDev &f, const float *d_rgb, const float
     // the work counter is zero here: cleared with the status block, then by
     // the k_grid_bwd of every backward
     cudaError_t e = cudaSuccess;
-    if (f.n_vox > 0)
+    if (f.n_vox > 0 && f.n_views == 1) {
+        k_clear_acc<<<(unsigned)((f.n_vox + kClearThreads - 1) / kClearThreads), kClearThreads, 0, s>>>(f);
+        e = cudaGetLastError();
+    } else if (f.n_vox > 0) {
         e = cudaMemsetAsync(f.dcol, 0, sizeof(float4) * (size_t)f.n_vox * (f.n_views + 2), s);  // dcol and dgrid
+    }
     if (e != cudaSuccess) return e;
     const BwdIn in = {d_rgb, d_depth, d_alpha, T_final, last, d_normal, d_dist, dist, max_weight};
     // extras: none; the distortion gradient alone (the training step's); it
@@ -2129,10 +2173,14 @@ cudaError_t launch_render_bwd(const FrameDev &f, const float *d_rgb, const float
     if (e != cudaSuccess) return e;
     if (f.n_vox > 0) {
         const unsigned blocks = (unsigned)((f.n_vox + kVoxBwdThreads - 1) / kVoxBwdThreads);
-        const int64_t per = kGridThreads * kGridIlp / 8;
-        k_grid_bwd<<<(unsigned)((f.n_vox + per - 1) / per), kGridThreads, 0, s>>>(f, d_grid);
-        if (f.n_views == 1) k_voxel_bwd<1><<<blocks, kVoxBwdThreads, 0, s>>>(f, d_sh, priority);
-        else k_voxel_bwd<4><<<blocks, kVoxBwdThreads, 0, s>>>(f, d_sh, priority);
+        const unsigned grid = (unsigned)((f.n_vox + kGridThreads - 1) / kGridThreads);   // 32 voxels a warp
+        if (f.n_views == 1) {
+            k_grid_bwd<true><<<grid, kGridThreads, 0, s>>>(f, d_grid);
+            k_voxel_bwd<1><<<blocks, kVoxBwdThreads, 0, s>>>(f, d_sh, priority);
+        } else {
+            k_grid_bwd<false><<<grid, kGridThreads, 0, s>>>(f, d_grid);
+            k_voxel_bwd<4><<<blocks, kVoxBwdThreads, 0, s>>>(f, d_sh, priority);
+        }
         e = cudaGetLastError();
     }
     return e;

@@ -66,6 +66,9 @@ __host__ __device__ __forceinline__ int64_t sort_chunk_capacity(int64_t capacity
     return 2 * capacity / kSortCap + 1;
 }
 
+// Words of one bit per voxel.
+__host__ __device__ __forceinline__ size_t hit_words(int64_t n_vox) { return (size_t)((n_vox + 31) / 32); }
+
 // Segment slots a workspace holds for pair_capacity pairs: a split tile of
 // L > kSegLen entries takes ceil(L / kSegLen) < 2 L / kSegLen slots.
 __host__ __device__ __forceinline__ int64_t seg_slot_capacity(int64_t capacity) {
@@ -330,6 +333,8 @@ struct FrameDev {
     uint32_t *cursor;        // [2^sub_log2][total_tiles] next free slot of each sub-bucket
     Record *rec;             // [V * N]
     ushort4 *box;            // [V * N] inclusive pixel range x0, x1, y0, y1 a hit can fall in
+    uint32_t *may_hit;       // single view: [hit_words(N)] bit v mod 32 of word v / 32: voxel v has a pair and
+                             // a box that is not empty
     unsigned long long *scan_blocks;   // [scan_blocks(2^sub_log2 total_tiles)] their sums
     uint64_t *keys[2];
     uint32_t *vals[2];
