@@ -51,6 +51,8 @@
 // warp's pixels are summed per staged entry in shared memory, and each entry
 // that was hit is added to the global accumulators once per warp (a colour
 // channel that the clamp of Eq. vox_color cut gets no gradient).
+#include <type_traits>
+
 #include "svr_internal.cuh"
 
 namespace svr {
@@ -1344,12 +1346,14 @@ __device__ __forceinline__ void hit_grad(const Entry &e, const PixelRay &p, cons
 // j's records, the warp waited for the entry with most hits (30 % of the
 // kernel, 16 mixed views: 4.99 ms in all), and each entry took 11 scalar
 // atomics after two loads of its corner indices.
+// 64 records: 1M-voxel step 728 us, 16 mixed views 9.29 ms, against 688 and 8.54
+// with 128 (96: 781 and 9.08 against 755 and 8.66).
 #ifndef SVR_BWD_REC_CAP
 #define SVR_BWD_REC_CAP 128
 #endif
 constexpr int kRecCap = SVR_BWD_REC_CAP;
 constexpr int kRecLane = kRecCap / 32;
-static_assert(kRecCap % 32 == 0, "the lanes share the slots evenly");
+static_assert(kRecCap % 32 == 0 && kRecLane <= 8, "the lanes share the slots evenly, each its entries' ids in a word");
 
 struct RecSmem {
     float4 rec[kRecCap * 3 + 32];  // see rec_at
@@ -1425,10 +1429,17 @@ __device__ __forceinline__ void add_sum(const Entry &e, const float4 &g0, const 
 // stretch's sum in the place of its first record.
 __device__ __forceinline__ void rec_flush(RecSmem &rs, const Entry *st, int n, float4 *__restrict__ acc_grid,
                                           float4 *__restrict__ acc_col) {
-    static_assert(kRecLane == 4, "a lane's entries are read as one word");
     __syncwarp();
     const int lane = threadIdx.x & 31, r0 = lane * kRecLane, cnt = min(kRecLane, n - r0);
-    const unsigned ids = r0 < n ? *reinterpret_cast<const unsigned *>(rs.ent + r0) : 0u;
+    // the lane's entries, a byte each
+    std::conditional_t<(kRecLane > 4), uint64_t, unsigned> ids = 0;
+    if constexpr (kRecLane == 4) {
+        if (r0 < n) ids = *reinterpret_cast<const unsigned *>(rs.ent + r0);
+    } else {
+#pragma unroll
+        for (int i = 0; i < kRecLane; ++i)
+            if (i < cnt) ids |= (decltype(ids))rs.ent[r0 + i] << (8 * i);
+    }
     const int k_first = (int)(ids & 0xFFu), k_last = r0 < n ? (int)((ids >> (8 * cnt - 8)) & 0xFFu) : -1;
     const int k_up = __shfl_up_sync(0xffffffffu, k_last, 1);
     const bool cont = lane > 0 && r0 < n && k_first == k_up;
