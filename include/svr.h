@@ -482,7 +482,7 @@ SVR_API int svr_debug_build(void);
 /* Waits for the current device, then writes its index-check report to
  * out[4] = {failed checks, site of the first (1 tile id, 2 tile range,
  * 3 voxel id, 4 gradient corner index, 5 record slot, 6 segment slot,
- * 7 block list length), its index, its bound} and clears it.
+ * 7 block list length, 8 sorted list length), its index, its bound} and clears it.
  * All zeros in builds without SVR_DEBUG.  out is a host array owned by the
  * caller; SVR_ERR_INVALID if it is NULL, SVR_ERR_CUDA on a CUDA error. */
 SVR_API int svr_debug_report(uint64_t *out);

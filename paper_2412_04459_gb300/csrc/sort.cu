@@ -15,8 +15,8 @@
 //                  pairwise merges, one thread-block cluster per list
 //
 // Where the parts of a pair fit 64 bits (Morton bits that can differ, sign
-// pattern, voxel id: every scene up to level 11 and 2^25 voxels, or level 14
-// and 2^19) pairs are emitted, sorted and merged as one word each and become
+// pattern, voxel id: every scene up to level 12 of fewer than 2^25 voxels, or
+// level 14 of fewer than 2^19) pairs are emitted, sorted and merged as one word each and become
 // (key, value) on the last write; otherwise the sort moves (Morton bits,
 // index in the list) words and the merge whole pairs.
 #include "svr_internal.cuh"
@@ -314,7 +314,8 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_sort_lists(FrameDev f) {
             if (!SVR_IN_BOUNDS(f.debug, kDbgRange, rg.y, f.capacity + 1)) continue;
             c0 = rg.x;
             n = (int)(rg.y - rg.x);
-            if (n > gt * kSortVT) continue;   // not reached: the class's longest list fits
+            // the class's longest list fits; one that did not would stay unsorted
+            if (!SVR_IN_BOUNDS(f.debug, kDbgSortList, n, gt * kSortVT + 1) || n > gt * kSortVT) continue;
         }
         const int g = threadIdx.x / gt, t = threadIdx.x & (gt - 1);
         uint64_t *s = smem + (size_t)g * (gt / 16 * 17 * kSortVT);

@@ -137,10 +137,10 @@ __device__ __forceinline__ int order_bucket(unsigned len, unsigned nseg) {
     return len ? 32 - __clz(len) + (nseg > 1 ? 1 : 0) : 0;
 }
 
-// Sort classes by list length: threads per list.  A list of 2^(c+8) to
-// 2^(c+9) - 1 pairs goes to class c = 1 .. 5 (32 2^(c-1) threads of 16 pairs
-// each, at least the longer end), a shorter one to class 0, whose lists take
-// a warp each as well (1024 pairs exactly, an unsplit list, fits class 2).
+// Sort classes by list length: threads per list.  A list of 2^(c+7) to
+// 2^(c+8) - 1 pairs goes to class c = 1 .. 5 (32 2^(c-1) threads of 16 pairs
+// each: 2^(c+8)), a shorter one to class 0, whose lists take a warp each as
+// well.  A list of exactly 1024 pairs, unsplit, goes to class 2, which it fills.
 constexpr int kSortClasses = 6;
 
 // Counters of the work order and the sort (cleared by k_scan_reduce, counted
@@ -173,6 +173,7 @@ enum DebugSite : unsigned {
     kDbgRecSlot = 5,     // gradient record slot >= kRecCap (render backward)
     kDbgSegSlot = 6,     // segment slot >= seg_slots (render)
     kDbgBlockList = 7,   // block list longer than its tile list or segment (render)
+    kDbgSortList = 8,    // tile list longer than its sort class takes (sort)
 };
 
 #ifdef SVR_DEBUG
