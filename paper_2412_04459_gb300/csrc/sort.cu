@@ -486,6 +486,10 @@ cudaError_t launch_order(const FrameDev &f, cudaStream_t s) {
 // tiles: 71 us, 133 with four); many tiles make many lists of two or three
 // chunks, whose rounds have work for fewer (8 x 2560x1440 views: 555 us with
 // eight CTAs, 292 with four, 189 with two; 16 mixed views: 113, 61 and 56).
+// Between, it is the number of long lists that decides, which the host does not
+// know.  svr_bin_sort with eight / two, us: 177 of them over 1,080 tiles 744 / 985, 458
+// over 4,240 651 / 581, 432 over 8,030 622 / 534, 181 over 14,400 540 / 530; none over
+// 8,030 106 / 122, 9,760 106 / 123, 14,400 114 / 125, one over 9,600 188 / 202.
 constexpr int kFewTiles = 8192;
 
 template <bool WORDS, int CLUSTER>

@@ -33,10 +33,13 @@ constexpr int kSegFields = 14;
 // A tile's pairs are counted and emitted through sub-buckets (by voxel id), so
 // that the atomics on a busy tile spread over separate cache lines; the
 // sub-buckets of a tile are adjacent in its range.  Fewer tiles are busier,
-// and the scan's cost grows with all of them: 32 up to 8192 tiles (emission of
-// a 2M-voxel preview over 280 tiles 99 -> 60 us against 8, 1M voxels over
-// 4,240 tiles 33.8 -> 32.5 us), 16 up to 131,072 (16 mixed views, 75,080 tiles:
-// 547 -> 497 us), else 8.
+// and the scan's cost grows with all of them: 32 up to 8192 tiles, 16 up to
+// 131,072, else 8.  Preprocess and binning, us with 8 / 16 / 32:
+//   1,080 tiles (8M voxels)   1504 / 1465 / 1401    57,600 (4 x 4M)  1836 / 1800 / 1820
+//   4,240                     1344 / 1335 / 1304    115,200 (2 x 1M)  471 /  480 /  526
+//   8,030                     1288 / 1284 / 1287    230,400 (4 x 1M)  800 /  828 /  914
+//   14,400 (1M voxels)         241 /  239 /  246    460,800 (8 x 2M) 2413 / 2479 / 2682
+// so 32 and 16 meet at the first line, and 16 and 8 between 57,600 and 115,200.
 __host__ __device__ __forceinline__ int tile_sub_log2(int64_t ntiles) {
     return ntiles <= 8192 ? 5 : ntiles <= 131072 ? 4 : 3;
 }
@@ -441,8 +444,10 @@ unsigned device_cached(DeviceCache &c, F compute) {
 // memory.  So the ten kernels from the tile masks to the forward do not wait
 // for one another's launch: 742 -> 718 us for the 1M-voxel step, 183 -> 174 us
 // for the smallest view.  The backward's kernels are launched plainly: with
-// them the step took 773 us.  Nor do the kernels of a large batch gain (16
-// mixed views, 75,080 tiles: 8.34 ms without, 8.37 with).
+// them the step took 773 us.  Large frames do not gain.  Preprocess to forward,
+// us without and with: 1M voxels over 8,030 tiles 417 and 396, 14,400 562 and 553,
+// 16,060 (two views) 696 and 683, 16,960 (four) 985 and 986, 28,800 (8M voxels, two)
+// 3147 and 3176; 8M voxels over 1,080 to 16,000 tiles lose up to 1 %.
 // Such a kernel is resident while the ones before it still write, so what it
 // reads is not constant for its lifetime: it loads with ordinary or L2 loads
 // only, which the wait orders, never through __ldg or const __restrict__
