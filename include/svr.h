@@ -206,12 +206,11 @@ SVR_API int svr_preprocess_views(svr_frame *frame, const svr_scene *scene, const
  * key = tile << 48 | (octpath XOR s replicated in all 16 triples) (the
  * direction-dependent Morton order of Sec. B.2), value = s << 29 | voxel id;
  * then a sort of each tile's range by the Morton bits that can differ (the
- * top 3 (max_level + 1) of the 48; with max_level = 16 all of them and the
- * value first), done tile by tile: merge sorts in shared memory, of chunks of
- * 8192 pairs in longer lists, whose chunks are then merged by clusters of
- * CTAs.  The result equals a sort
- * of all pairs by (key, value): within a tile distinct pairs have distinct
- * (key, value).  Also builds the render work order and the per-block lists.
+ * top 3 (max_level + 1) of the 48), equal ones by value, done tile by tile:
+ * merge sorts in shared memory, of chunks of 8192 pairs in longer lists, whose
+ * chunks are then merged by clusters of CTAs.  The result equals a sort of all
+ * pairs by (key, value), also where voxels overlap: within a tile distinct
+ * pairs have distinct (key, value).  Also builds the render work order and the per-block lists.
  * n_pairs_out: if not NULL, the call synchronises the stream, stores the
  * true pair count there, and returns SVR_ERR_CAPACITY if it exceeds the
  * capacity (no pair was written; re-run with a larger workspace) or

@@ -1948,9 +1948,10 @@ constexpr int kVoxBwdThreads = 128;
 constexpr int kShRow = 52;
 
 // A batch's views are taken VIEWS = 4 at a time, their loads in flight
-// together (0.82 -> 0.59 ms for 8 views of 8M voxels, 191 -> 133 us for 16 of
-// 1M); a single view by its own instantiation, which needs fewer registers (40
-// us for 1M voxels, 45 with four).
+// together (one at a time: 0.82 ms for 8 views of 8M voxels and 191 us for 16 of
+// 1M, against 0.60 and 134); a single view by its own instantiation, which needs
+// fewer registers (40 us for 1M voxels, 45 with four; 36 since it skips the voxels
+// that no pixel can hit, at seven CTAs per SM).
 template <int VIEWS>
 __global__ void __launch_bounds__(kVoxBwdThreads, VIEWS == 1 ? 7 : 5) k_voxel_bwd(FrameDev f, float *__restrict__ d_sh,
                                                               float *__restrict__ priority) {
@@ -2016,7 +2017,7 @@ __global__ void __launch_bounds__(kVoxBwdThreads, VIEWS == 1 ? 7 : 5) k_voxel_bw
 // two dependent loads and the scattered atomics: kGridIlp corners per thread are
 // in flight.  A kernel of its own, before k_voxel_bwd while the accumulators are
 // in L2: inside it, 79 us (1M voxels) and 1.28 ms (8M, 8 views) for both against
-// 31 + 40 us and 0.29 + 0.60 ms; as other CTAs of one launch, 116 us and 1.54 ms.
+// 31 + 40 us and 0.29 + 0.60 ms then; as other CTAs of one launch, 116 us and 1.54 ms.
 // A warp takes 32 voxels and, ONE (a single view), skips those that no pixel can
 // hit.
 constexpr int kGridThreads = 256, kGridIlp = 4;
