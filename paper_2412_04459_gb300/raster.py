@@ -126,7 +126,8 @@ class _StatusRead(threading.local):
     def get(self, device: torch.device):
         slot = self.slots.get(device.index)
         if slot is None:
-            slot = (torch.empty(16, dtype=torch.int32, pin_memory=True), torch.cuda.Event())
+            # host memory whatever the caller's default device
+            slot = (torch.empty(16, dtype=torch.int32, device="cpu", pin_memory=True), torch.cuda.Event())
             self.slots[device.index] = slot
         return slot
 
