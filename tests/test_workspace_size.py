@@ -1,6 +1,6 @@
-"""The workspace takes no more than the buffers of the layout that had separate
-gradient accumulators of 12 bytes per voxel and view: a scene and capacity that
-fitted a memory still do."""
+"""At the capacity that a frame takes by itself (four pairs per voxel and view) the
+workspace is no larger than the buffers of the layout that had separate gradient
+accumulators of 12 bytes per voxel and view: a scene that fitted still does."""
 import pytest
 
 import synth
